@@ -124,15 +124,12 @@ struct MfTraceBufs {
   double *defer_part;       // [defer_list_cap / 8] FP64 sum of each chunk
   uint32_t *defer_chunk;    // [defer_list_cap / 8] record of each chunk (~0: none)
   uint64_t defer_cap, defer_list_cap;
-  // vertex slots of the expand items of the whole search: k_expand_vertices
-  // records the slot of item j of warp w of a chunk at
-  // item_slot[warp_base[w] + j] (~0u: outside the domain) and the first item
-  // of each edge in edge_item_off (~0: not recorded); k_expand_edges and the
-  // cell enumeration's link tables read them instead of looking the
-  // vertices up (warp_base[w] = ~0: the warp's items did not fit, look them
-  // up); absent when null
+  // vertex slots of the expand items of the whole search: the vertices pass
+  // records the slot of item r of edge e at item_slot[edge_item_off[e] + r]
+  // (~0u: outside the domain; edge_item_off ~0: the edge's items did not fit,
+  // look them up); the edges pass and the cell enumeration's link tables read
+  // them instead of looking the vertices up; absent when null
   uint32_t *item_slot;
-  unsigned long long *warp_base;
   unsigned long long *edge_item_off;
   uint64_t item_cap;
 };
@@ -589,6 +586,10 @@ void mf_exclusive_scan(const int64_t *in, int64_t *out, int64_t n, int64_t *scra
 uint64_t mf_next_pow2(uint64_t x);
 void mf_launch_seeds(const MfFrame &F, const MfTraceBufs &B, const double *seeds, int64_t n,
                      bool vertices, cudaStream_t s);
+// One pass of the search over edges [e0, e0 + n): the new vertices of their
+// 2-simplex cofaces, or (after those are evaluated) the new crossing edges.
+void mf_launch_expand(const MfFrame &F, const MfTraceBufs &B, uint64_t e0, uint64_t n, bool edges,
+                      int sms, cudaStream_t st);
 // The crossing n-simplices of edges [0, n_edges) with their sign masks and
 // CSR row lengths (in B.cell_off), and, once cell_off is scanned, the CSR
 // fill of B.cell_idx (a missing edge sets err_missing).

@@ -45,8 +45,6 @@ __global__ void k_prepare_rbf(int d, int n, const double *sv, const double *alph
 __global__ void k_rbf_blocks(int d, int n, int nblk, const float *sv32, float *blo, float *bhi);
 __global__ void k_seed_vertices(MfFrame F, MfTraceBufs B, const double *seeds, int64_t n);
 __global__ void k_seed_edges(MfFrame F, MfTraceBufs B, const double *seeds, int64_t n);
-__global__ void k_expand_vertices(MfFrame F, MfTraceBufs B, uint64_t e0, uint64_t n);
-__global__ void k_expand_edges(MfFrame F, MfTraceBufs B, uint64_t e0, uint64_t n);
 namespace {
 
 const int64_t kScanTile = 512 * 8;
@@ -315,10 +313,9 @@ extern "C" int mf_trace_noalloc(const mf_rbf *rbf, const mf_domain *dom, const m
   while (fe > fs) {
     for (uint64_t a = fs; a < fe; a += cap) {
       const uint64_t m = fe - a < cap ? fe - a : cap;
-      const unsigned g = (unsigned)((m + 255) / 256);  // a warp per 32 edges, 8 per block
-      k_expand_vertices<<<g, 256, 0, st>>>(F, B, a, m);
+      mf_launch_expand(F, B, a, m, false, sms, st);
       eval();
-      k_expand_edges<<<g, 256, 0, st>>>(F, B, a, m);
+      mf_launch_expand(F, B, a, m, true, sms, st);
     }
     if (cudaGetLastError() != cudaSuccess) return MF_ERR_CUDA;
     if ((rc = sync_read(&h, cnt, st))) return rc;

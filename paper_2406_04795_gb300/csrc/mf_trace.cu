@@ -10,7 +10,7 @@
 //                while level L-1 was expanded, so the list is also the queue.
 //
 // One BFS level, per frontier chunk of <= batch_cap edges:
-//   k_expand_vertices  warp per 32 edges, lane per coface item (the new
+//   k_expand_vertices  warp per 1 to 32 edges, lane per coface item (the new
 //                      vertex w of one 2-simplex coface, query type 3): w is
 //                      inserted into the vertex table; first inserters append
 //                      it to the vertex list.
@@ -165,66 +165,137 @@ __device__ __forceinline__ uint32_t expand_item_decode(uint32_t S, int d, uint32
   return deposit_bits((r >> 1) + 1u, ~S & ((1u << d) - 1u));
 }
 
-// Visits the new vertex of one item; returns 1 if it lies outside the box.
-// *slot: its table slot (~0u outside the box or with a full table).
-__device__ __forceinline__ unsigned expand_vertices_item(const MfFrame &F, const MfTraceBufs &B,
-                                                         uint64_t e, uint32_t S, int kind,
-                                                         uint32_t M, uint32_t *slot = nullptr) {
-  const int d = F.d;
-  int32_t w[MF_MAXD];
-  load_y(B.edge_y + e * d, d, w);
-  if (kind == 0) mf_add_mask(d, w, M, 1);
-  else if (kind == 1) mf_add_mask(d, w, S | M, 1);
-  else mf_add_mask(d, w, M, -1);
-  if (vertex_in(F, w)) {
-    const uint64_t sl = mf_visit_vertex(F, B, w);
-    if (slot) *slot = sl == ~0ull ? ~0u : (uint32_t)sl;
-    return 0;
-  }
-  if (slot) *slot = ~0u;
-  return 1;
+// The vertex y + sgn e(Q) of an item (Q = M, S | M or M; sgn = -1 for kind 2).
+__device__ __forceinline__ void expand_item_vertex(int d, const int32_t *y, uint32_t S, int kind,
+                                                   uint32_t M, int32_t *w) {
+  const uint32_t Q = kind == 1 ? S | M : M;
+  const int sgn = kind == 2 ? -1 : 1;
+#pragma unroll
+  for (int k = 0; k < MF_MAXD; k++) w[k] = k < d ? y[k] + (((Q >> k) & 1u) ? sgn : 0) : 0;
 }
 
-// Under the sign rule s = [f >= 0] a crossing triangle has exactly two
-// crossing edges (Sec. IV-A): the parent and the one joining the new vertex w
-// to the parent end whose sign differs from s(w).
-// slot: the new vertex's table slot recorded by k_expand_vertices (~0u:
+// List indices for the lanes with take = true (all 32 lanes call).  ONE: all
+// lanes share the counter (one trace), one ballot and one atomic; otherwise
+// the lanes are grouped by counter first.
+template <bool ONE>
+__device__ __forceinline__ unsigned long long expand_alloc(unsigned long long *counter, bool take) {
+  if (!ONE) return mf_warp_alloc(counter, take);
+  const unsigned m = __ballot_sync(0xffffffffu, take);
+  if (!m) return 0;
+  const int lane = threadIdx.x & 31, leader = __ffs(m) - 1;
+  unsigned long long base = 0;
+  if (lane == leader) base = atomicAdd(counter, (unsigned long long)__popc(m));
+  base = __shfl_sync(0xffffffffu, base, leader);
+  return base + (unsigned long long)__popc(m & ((1u << lane) - 1u));
+}
+
+// One round of the vertices pass (all 32 lanes, converged; have: this lane
+// holds an item of parent y, S): inserts the item's new vertex into the
+// vertex table, first inserters append it to the vertex list.  Returns its
+// table slot (~0u: no item, outside the box or a full table); *out: 1 when it
+// lies outside the box.
+template <bool ONE>
+__device__ __forceinline__ uint32_t expand_vertices_round(const MfFrame &F, const MfTraceBufs &B,
+                                                          bool have, const int32_t *y, uint32_t S,
+                                                          int kind, uint32_t M, unsigned *out) {
+  const int d = F.d;
+  int32_t w[MF_MAXD];
+  expand_item_vertex(d, y, S, kind, M, w);
+  const bool in = have && vertex_in(F, w);
+  *out = have && !in ? 1u : 0u;
+  bool won = false;
+  uint64_t slot = ~0ull;
+  if (in) {
+    slot = mf_table_insert<2>(B.vtab_key, B.vtab_mask, mf_vertex_key(F, w), &won);
+    if (slot == ~0ull) atomicOr(&B.cnt->err_table_full, 1u);
+  }
+  const bool take = slot != ~0ull && won;
+  const unsigned long long idx = expand_alloc<ONE>(have ? &B.cnt->n_vertices : nullptr, take);
+  if (take) {
+    if (idx >= B.max_vertices) {
+      atomicOr(&B.cnt->err_overflow, 1u);
+    } else {
+#pragma unroll
+      for (int k = 0; k < MF_MAXD; k++)
+        if (k < d) B.vert_y[idx * d + k] = w[k];
+      B.vert_slot[idx] = (uint32_t)slot;
+      if (B.vtab_idx) B.vtab_idx[slot] = (uint32_t)idx;
+    }
+  }
+  return slot == ~0ull ? ~0u : (uint32_t)slot;
+}
+
+// One round of the edges pass.  Under the sign rule s = [f >= 0] a crossing
+// triangle has exactly two crossing edges (Sec. IV-A): the parent and the one
+// joining the new vertex w to the parent end whose sign differs from s(w).
+// That edge's base vertex is y + sgn e(Q) and its mask and end values follow
+// from the kind by selects, so that the round has one table probe whatever
+// the kinds of its lanes (six call sites of the probe, one per kind and end,
+// ran one after the other within a warp).
+// slot: the new vertex's table slot recorded by the vertices pass (~0u:
 // outside the box), or MF_SLOT_UNKNOWN to look it up.
 #define MF_SLOT_UNKNOWN 0xfffffffeu
-__device__ __forceinline__ void expand_edges_item(const MfFrame &F, const MfTraceBufs &B,
-                                                  uint64_t e, uint32_t S, int kind, uint32_t M,
-                                                  uint32_t slot = MF_SLOT_UNKNOWN) {
+template <bool ONE>
+__device__ __forceinline__ void expand_edges_round(const MfFrame &F, const MfTraceBufs &B,
+                                                   bool have, const int32_t *y, uint32_t S,
+                                                   double f0, double f1, int kind, uint32_t M,
+                                                   uint32_t slot) {
   const int d = F.d;
-  int32_t y[MF_MAXD], w[MF_MAXD];
-  load_y(B.edge_y + e * d, d, y);
-  load_y(y, d, w);
-  if (kind == 0) mf_add_mask(d, w, M, 1);
-  else if (kind == 1) mf_add_mask(d, w, S | M, 1);
-  else mf_add_mask(d, w, M, -1);
-  double fw;
-  if (slot == MF_SLOT_UNKNOWN) {
-    if (!vertex_in(F, w)) return;
-    fw = mf_lookup_f(F, B, w);
-  } else {
-    if (slot == ~0u) return;
-    fw = mf_vtab_f(B, slot);
-  }
-  const double f0 = B.edge_f[2 * e], f1 = B.edge_f[2 * e + 1];
-  const bool cross0 = (fw >= 0.0) != (f0 >= 0.0);
-  if (kind == 0) {
-    if (cross0) mf_emit_edge(F, B, y, M, f0, fw);
-    else mf_emit_edge(F, B, w, S & ~M, fw, f1);
-  } else if (kind == 1) {
-    if (cross0) {
-      mf_emit_edge(F, B, y, S | M, f0, fw);
+  double fw = 0.0;
+  if (have) {
+    if (slot == MF_SLOT_UNKNOWN) {
+      int32_t w[MF_MAXD];
+      expand_item_vertex(d, y, S, kind, M, w);
+      have = vertex_in(F, w);
+      if (have) fw = mf_lookup_f(F, B, w);
     } else {
-      mf_add_mask(d, y, S, 1);
-      mf_emit_edge(F, B, y, M, f1, fw);
+      have = slot != ~0u;
+      if (have) fw = mf_vtab_f(B, slot);
     }
-  } else {
-    if (cross0) mf_emit_edge(F, B, w, M, fw, f0);
-    else mf_emit_edge(F, B, w, M | S, fw, f1);
   }
+  const bool cross0 = (fw >= 0.0) != (f0 >= 0.0);
+  uint32_t Q, mask;
+  double fa, fb;
+  if (kind == 0) {
+    Q = cross0 ? 0u : M;
+    mask = cross0 ? M : S & ~M;
+    fa = cross0 ? f0 : fw;
+    fb = cross0 ? fw : f1;
+  } else if (kind == 1) {
+    Q = cross0 ? 0u : S;
+    mask = cross0 ? S | M : M;
+    fa = cross0 ? f0 : f1;
+    fb = fw;
+  } else {
+    Q = M;
+    mask = cross0 ? M : M | S;
+    fa = fw;
+    fb = cross0 ? f0 : f1;
+  }
+  const int sgn = kind == 2 ? -1 : 1;
+  int32_t b[MF_MAXD];
+#pragma unroll
+  for (int k = 0; k < MF_MAXD; k++) b[k] = k < d ? y[k] + (((Q >> k) & 1u) ? sgn : 0) : 0;
+  bool won = false;
+  uint64_t es = ~0ull;
+  if (have) {
+    es = mf_table_insert<2>(B.etab_key, B.etab_mask, mf_edge_key(F, b, mask), &won);
+    if (es == ~0ull) atomicOr(&B.cnt->err_table_full, 1u);
+  }
+  const bool take = es != ~0ull && won;
+  const unsigned long long idx = expand_alloc<ONE>(have ? &B.cnt->n_edges : nullptr, take);
+  if (!take) return;
+  if (idx >= B.max_edges) {
+    atomicOr(&B.cnt->err_overflow, 1u);
+    return;
+  }
+#pragma unroll
+  for (int k = 0; k < MF_MAXD; k++)
+    if (k < d) B.edge_y[idx * d + k] = b[k];
+  B.edge_mask[idx] = mask;
+  B.edge_f[2 * idx] = fa;
+  B.edge_f[2 * idx + 1] = fb;
+  mf_etab_val(B, es) = (uint32_t)idx;
 }
 
 // Inclusive warp scan of the per-lane item counts into s_end[0..31]; returns
@@ -254,57 +325,96 @@ __device__ __forceinline__ int expand_owner(const uint32_t *s_end, uint32_t j, u
 
 #define EXPAND_WARPS 8
 
-// Warp per 32 consecutive edges of [e0, e0 + n), lane per coface item, so
-// that no lane idles on masks that select no coface.
+// Edges per warp of a pass over n edges by nwarps warps: 32 when the level
+// fills the chip, fewer when it does not, down to the number whose items fit
+// one round of the warp's lanes (an edge has at most 2^d - 2).  The passes
+// are chains of dependent accesses (slot, f, probe, append), so a level that
+// leaves SMs empty takes as long as its longest warp: with 32 edges per warp a
+// d = 3 level of 500 edges ran 6 rounds on 2 blocks (36 us), with 4 edges 1
+// round on 16 blocks.
+__device__ __forceinline__ int expand_group(int d, unsigned long long n, unsigned long long nwarps) {
+  int g = d <= 2 ? 16 : d == 3 ? 4 : d == 4 ? 2 : 1;
+  while (g < 32 && n > (unsigned long long)g * nwarps) g <<= 1;
+  return g;
+}
+
+struct ExpandShared {
+  uint32_t end[EXPAND_WARPS][32], S[EXPAND_WARPS][32];
+  unsigned long long off[EXPAND_WARPS][32];  // each edge's first item in the slot record
+  int32_t y[EXPAND_WARPS][32][MF_MAXD];
+  double f[EXPAND_WARPS][32][2];  // edges pass: the end values
+};
+
+// Edges [e0, e0 + n): a warp takes expand_group edges, lane per coface item,
+// so that no lane idles on masks that select no coface.
 template <bool EDGES>
-__device__ __forceinline__ void expand_warp(const MfFrame &F, const MfTraceBufs &B, uint64_t e0,
-                                            uint64_t n) {
-  __shared__ uint32_t s_end[EXPAND_WARPS][32], s_S[EXPAND_WARPS][32];
+__device__ __forceinline__ void expand_range(const MfFrame &F, const MfTraceBufs &B, uint64_t e0,
+                                             uint64_t n) {
+  __shared__ ExpandShared sh;
   const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5;
-  const uint64_t first = (blockIdx.x * (uint64_t)EXPAND_WARPS + wi) * 32;
-  if (first >= n) return;  // whole warp
   const int d = F.d;
-  uint32_t S = 0, c = 0;
-  if (first + lane < n) {
-    S = B.edge_mask[e0 + first + lane];
-    c = S ? expand_item_count(S, d) : 0u;
-  }
-  s_S[wi][lane] = S;
-  const uint32_t total = expand_warp_scan(c, s_end[wi]);
-  // the warp's items in the chunk's slot record (see MfTraceBufs.item_slot)
-  const uint64_t wg = blockIdx.x * (uint64_t)EXPAND_WARPS + wi;
-  unsigned long long ib = ~0ull;
-  if (B.item_slot) {
-    if (EDGES) {
-      ib = B.warp_base[wg];
-    } else {
-      if (lane == 0) {
-        ib = atomicAdd(&B.cnt->n_items, (unsigned long long)total);
-        if (ib + total > B.item_cap) ib = ~0ull;
-        B.warp_base[wg] = ib;
-      }
-      ib = __shfl_sync(0xffffffffu, ib, 0);
-      // each lane's edge: the first of its items
-      if (B.edge_item_off && first + lane < n)
-        B.edge_item_off[e0 + first + lane] =
-            ib == ~0ull ? ~0ull : ib + (lane ? s_end[wi][lane - 1] : 0u);
-    }
-  }
+  const uint64_t nwarps = (uint64_t)gridDim.x * EXPAND_WARPS;
+  const uint64_t G = (uint64_t)expand_group(d, n, nwarps);
   unsigned nb = 0;
-  for (uint32_t j = lane; j < total; j += 32) {
-    uint32_t r;
-    const int o = expand_owner(s_end[wi], j, &r);
-    const uint32_t So = s_S[wi][o];
-    int kind;
-    const uint32_t M = expand_item_decode(So, d, r, &kind);
-    if (EDGES) {
-      expand_edges_item(F, B, e0 + first + o, So, kind, M,
-                        ib != ~0ull ? B.item_slot[ib + j] : MF_SLOT_UNKNOWN);
-    } else {
-      uint32_t sl;
-      nb += expand_vertices_item(F, B, e0 + first + o, So, kind, M, &sl);
-      if (ib != ~0ull) B.item_slot[ib + j] = sl;
+  for (uint64_t first = (blockIdx.x * (uint64_t)EXPAND_WARPS + wi) * G; first < n;
+       first += nwarps * G) {
+    const uint64_t e = e0 + first + lane;
+    const bool mine = lane < (int)G && first + lane < n;
+    uint32_t S = 0, c = 0;
+    if (mine) {
+      S = B.edge_mask[e];
+      c = S ? expand_item_count(S, d) : 0u;
+#pragma unroll
+      for (int k = 0; k < MF_MAXD; k++)
+        if (k < d) sh.y[wi][lane][k] = B.edge_y[e * d + k];
+      if (EDGES) {
+        const double2 f = reinterpret_cast<const double2 *>(B.edge_f)[e];
+        sh.f[wi][lane][0] = f.x;
+        sh.f[wi][lane][1] = f.y;
+      }
     }
+    sh.S[wi][lane] = S;
+    const uint32_t total = expand_warp_scan(c, sh.end[wi]);
+    // the edges' items in the slot record (see MfTraceBufs.item_slot)
+    unsigned long long off = ~0ull;
+    if (B.item_slot) {
+      if (EDGES) {
+        if (mine) off = B.edge_item_off[e];
+      } else {
+        unsigned long long ib = 0;
+        if (lane == 0) {
+          ib = atomicAdd(&B.cnt->n_items, (unsigned long long)total);
+          if (ib + total > B.item_cap) ib = ~0ull;
+        }
+        ib = __shfl_sync(0xffffffffu, ib, 0);
+        if (ib != ~0ull) off = ib + (lane ? sh.end[wi][lane - 1] : 0u);
+        if (mine) B.edge_item_off[e] = off;
+      }
+    }
+    sh.off[wi][lane] = off;
+    __syncwarp();
+    for (uint32_t j0 = 0; j0 < total; j0 += 32) {
+      const uint32_t j = j0 + lane;
+      const bool have = j < total;
+      uint32_t r;
+      const int o = expand_owner(sh.end[wi], have ? j : 0u, &r);
+      const uint32_t So = sh.S[wi][o];
+      const unsigned long long io = sh.off[wi][o];
+      int kind;
+      const uint32_t M = expand_item_decode(So, d, r, &kind);
+      if (EDGES) {
+        uint32_t sl = MF_SLOT_UNKNOWN;
+        if (have && io != ~0ull) sl = B.item_slot[io + r];
+        expand_edges_round<true>(F, B, have, sh.y[wi][o], So, sh.f[wi][o][0], sh.f[wi][o][1], kind,
+                                 M, sl);
+      } else {
+        unsigned out;
+        const uint32_t sl = expand_vertices_round<true>(F, B, have, sh.y[wi][o], So, kind, M, &out);
+        nb += out;
+        if (have && io != ~0ull) B.item_slot[io + r] = sl;
+      }
+    }
+    __syncwarp();  // the next group overwrites this warp's shared entries
   }
   if (!EDGES) {
     nb = __reduce_add_sync(0xffffffffu, nb);
@@ -312,14 +422,20 @@ __device__ __forceinline__ void expand_warp(const MfFrame &F, const MfTraceBufs 
   }
 }
 
+// D < MF_MAXD: the exact dimension, so that the coordinate loops and the key
+// have no predicated axes; MF_MAXD serves the rest at run time.
+template <int D>
 __global__ void __launch_bounds__(EXPAND_WARPS * 32) k_expand_vertices(MfFrame F, MfTraceBufs B,
                                                                        uint64_t e0, uint64_t n) {
-  expand_warp<false>(F, B, e0, n);
+  if (D < MF_MAXD) __builtin_assume(F.d == D);
+  expand_range<false>(F, B, e0, n);
 }
 
+template <int D>
 __global__ void __launch_bounds__(EXPAND_WARPS * 32) k_expand_edges(MfFrame F, MfTraceBufs B,
                                                                     uint64_t e0, uint64_t n) {
-  expand_warp<true>(F, B, e0, n);
+  if (D < MF_MAXD) __builtin_assume(F.d == D);
+  expand_range<true>(F, B, e0, n);
 }
 
 // ---------------------------------------------------------------------------
@@ -785,59 +901,73 @@ template <bool EDGES>
 __global__ void __launch_bounds__(EXPAND_WARPS * 32) k_b_expand(const MfSlot *slots,
                                                                 const MfSlotState *st,
                                                                 const MfBatchPlan *P, int n) {
-  __shared__ uint32_t s_end[EXPAND_WARPS][32], s_S[EXPAND_WARPS][32];
+  __shared__ ExpandShared sh;
   __shared__ int s_t[EXPAND_WARPS][32];
-  __shared__ unsigned long long s_e[EXPAND_WARPS][32], s_io[EXPAND_WARPS][32];
   const unsigned long long total = P->px[n];
   const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5;
   const unsigned long long nwarps = (unsigned long long)gridDim.x * EXPAND_WARPS;
-  for (unsigned long long g = blockIdx.x * (unsigned long long)EXPAND_WARPS + wi; g * 32 < total;
-       g += nwarps) {
-    const unsigned long long item = g * 32 + lane;
+  // edges per warp as for one trace (the slots' dimensions differ: d = 4)
+  const unsigned long long G = (unsigned long long)expand_group(4, total, nwarps);
+  for (unsigned long long first = (blockIdx.x * (unsigned long long)EXPAND_WARPS + wi) * G;
+       first < total; first += nwarps * G) {
+    const unsigned long long item = first + lane;
+    const bool mine = lane < (int)G && item < total;
     uint32_t S = 0, c = 0;
     int t = 0;
-    unsigned long long e = 0;
-    if (item < total) {
-      t = mf_slot_of(P->px, n, item);
-      e = st[t].cursor + (item - P->px[t]);
-      S = slots[t].B.edge_mask[e];
-      c = S ? expand_item_count(S, slots[t].F.d) : 0u;
-    }
-    s_S[wi][lane] = S;
-    s_t[wi][lane] = t;
-    s_e[wi][lane] = e;
     // the edge's first item in its trace's slot record (see
     // MfTraceBufs.item_slot; per edge, as the warp's edges may belong to
     // several traces): taken by the vertices pass, read by the edges pass
     unsigned long long io = ~0ull;
-    if (item < total && slots[t].B.item_slot) {
+    if (mine) {
+      t = mf_slot_of(P->px, n, item);
       const MfTraceBufs &TB = slots[t].B;
+      const unsigned long long e = st[t].cursor + (item - P->px[t]);
+      const int d = slots[t].F.d;
+      S = TB.edge_mask[e];
+      c = S ? expand_item_count(S, d) : 0u;
+#pragma unroll
+      for (int k = 0; k < MF_MAXD; k++)
+        if (k < d) sh.y[wi][lane][k] = TB.edge_y[e * d + k];
       if (EDGES) {
-        io = TB.edge_item_off[e];
-      } else {
-        io = atomicAdd(&TB.cnt->n_items, (unsigned long long)c);
-        if (io + c > TB.item_cap) io = ~0ull;
-        TB.edge_item_off[e] = io;
+        const double2 f = reinterpret_cast<const double2 *>(TB.edge_f)[e];
+        sh.f[wi][lane][0] = f.x;
+        sh.f[wi][lane][1] = f.y;
+      }
+      if (TB.item_slot) {
+        if (EDGES) {
+          io = TB.edge_item_off[e];
+        } else {
+          io = atomicAdd(&TB.cnt->n_items, (unsigned long long)c);
+          if (io + c > TB.item_cap) io = ~0ull;
+          TB.edge_item_off[e] = io;
+        }
       }
     }
-    s_io[wi][lane] = io;
-    const uint32_t nit = expand_warp_scan(c, s_end[wi]);
-    for (uint32_t j = lane; j < nit; j += 32) {
+    sh.S[wi][lane] = S;
+    s_t[wi][lane] = t;
+    sh.off[wi][lane] = io;
+    const uint32_t nit = expand_warp_scan(c, sh.end[wi]);
+    for (uint32_t j0 = 0; j0 < nit; j0 += 32) {
+      const uint32_t j = j0 + lane;
+      const bool have = j < nit;
       uint32_t r;
-      const int o = expand_owner(s_end[wi], j, &r);
+      const int o = expand_owner(sh.end[wi], have ? j : 0u, &r);
       const MfSlot &SL = slots[s_t[wi][o]];
-      const uint32_t So = s_S[wi][o];
-      const unsigned long long oo = s_io[wi][o];
+      const uint32_t So = sh.S[wi][o];
+      const unsigned long long oo = sh.off[wi][o];
       int kind;
       const uint32_t M = expand_item_decode(So, SL.F.d, r, &kind);
       if (EDGES) {
-        expand_edges_item(SL.F, SL.B, s_e[wi][o], So, kind, M,
-                          oo != ~0ull ? SL.B.item_slot[oo + r] : MF_SLOT_UNKNOWN);
+        uint32_t sl = MF_SLOT_UNKNOWN;
+        if (have && oo != ~0ull) sl = SL.B.item_slot[oo + r];
+        expand_edges_round<false>(SL.F, SL.B, have, sh.y[wi][o], So, sh.f[wi][o][0],
+                                  sh.f[wi][o][1], kind, M, sl);
       } else {
-        uint32_t sl;
-        if (expand_vertices_item(SL.F, SL.B, s_e[wi][o], So, kind, M, &sl))
-          atomicAdd(&SL.B.cnt->n_boundary, 1ull);
-        if (oo != ~0ull) SL.B.item_slot[oo + r] = sl;
+        unsigned out;
+        const uint32_t sl =
+            expand_vertices_round<false>(SL.F, SL.B, have, sh.y[wi][o], So, kind, M, &out);
+        if (out) atomicAdd(&SL.B.cnt->n_boundary, 1ull);
+        if (have && oo != ~0ull) SL.B.item_slot[oo + r] = sl;
       }
     }
     __syncwarp();  // the next group overwrites this warp's shared entries
@@ -1264,6 +1394,26 @@ void mf_launch_cells_enum(const MfFrame &F, const MfTraceBufs &B, uint64_t n_edg
   if (n_edges == 0) return;
   k_cells_enum<<<(unsigned)((n_edges * 32 + 255) / 256), 256, 0, st>>>(F, B, n_edges);
 }
+// Warps for one lane round of each edge's items, at most what the device
+// holds a few times over (the kernels pick the edges per warp).
+void mf_launch_expand(const MfFrame &F, const MfTraceBufs &B, uint64_t e0, uint64_t n, bool edges,
+                      int sms, cudaStream_t st) {
+  if (n == 0) return;
+  const unsigned g = (unsigned)std::min<uint64_t>((n + EXPAND_WARPS - 1) / EXPAND_WARPS,
+                                                  (uint64_t)sms * 8);
+  switch (F.d) {
+#define MF_CASE(DD)                                                                   \
+  case DD:                                                                            \
+    if (edges) k_expand_edges<DD><<<g, EXPAND_WARPS * 32, 0, st>>>(F, B, e0, n);       \
+    else k_expand_vertices<DD><<<g, EXPAND_WARPS * 32, 0, st>>>(F, B, e0, n);          \
+    break;
+    MF_CASE(2) MF_CASE(3) MF_CASE(4) MF_CASE(5) MF_CASE(6) MF_CASE(7)
+#undef MF_CASE
+    default:
+      if (edges) k_expand_edges<MF_MAXD><<<g, EXPAND_WARPS * 32, 0, st>>>(F, B, e0, n);
+      else k_expand_vertices<MF_MAXD><<<g, EXPAND_WARPS * 32, 0, st>>>(F, B, e0, n);
+  }
+}
 void mf_launch_seeds(const MfFrame &F, const MfTraceBufs &B, const double *seeds, int64_t n,
                      bool vertices, cudaStream_t s) {
   const unsigned g = (unsigned)((n + 127) / 128);
@@ -1494,20 +1644,17 @@ extern "C" int mf_trace(mf_ctx *ctx, const mf_rbf *rbf, const mf_domain *dom,
   uint64_t cap = opts->batch_cap_edges > 0 ? (uint64_t)opts->batch_cap_edges : (1ull << 24);
   if (ctx->tune.frontier_chunk > 0 && ctx->tune.frontier_chunk < cap) cap = ctx->tune.frontier_chunk;
   // the expand items' vertex slots of the whole search: up to (2^d - 2)
-  // items per edge (at most 2^31, halved while the budget refuses), the
-  // first item of each edge and the bases of one chunk's warps
+  // items per edge (at most 2^31, halved while the budget refuses) and the
+  // first item of each edge
   {
-    const uint64_t ce = std::min<uint64_t>(cap, ME);
-    const uint64_t nw = (ce + 255) / 256 * EXPAND_WARPS + EXPAND_WARPS;
     auto al = [](size_t x) { return (x + 255) & ~(size_t)255; };
     std::string keep = ctx->err;
     for (uint64_t ic = std::min<uint64_t>(ME * ((1ull << d) - 2), 1ull << 31); ic >= (1ull << 20);
          ic >>= 1) {
-      char *q = (char *)mf_ctx_buffer(ctx, MF_SLOT_ITEMS, al(ic * 4) + al(nw * 8) + al(ME * 8));
+      char *q = (char *)mf_ctx_buffer(ctx, MF_SLOT_ITEMS, al(ic * 4) + al(ME * 8));
       if (q) {
         B.item_slot = (uint32_t *)q;
-        B.warp_base = (unsigned long long *)(q + al(ic * 4));
-        B.edge_item_off = (unsigned long long *)(q + al(ic * 4) + al(nw * 8));
+        B.edge_item_off = (unsigned long long *)(q + al(ic * 4));
         B.item_cap = ic;
         break;
       }
@@ -1546,10 +1693,9 @@ extern "C" int mf_trace(mf_ctx *ctx, const mf_rbf *rbf, const mf_domain *dom,
   while (fe > fs) {
     for (uint64_t a = fs; a < fe; a += cap) {
       const uint64_t n = std::min(cap, fe - a);
-      const unsigned g = (unsigned)((n + EXPAND_WARPS * 32 - 1) / (EXPAND_WARPS * 32));
       {
         MfProfScope ps(ctx, MF_PH_EXPAND_V, st, 1, (int64_t)n);
-        k_expand_vertices<<<g, EXPAND_WARPS * 32, 0, st>>>(F, B, a, n);
+        mf_launch_expand(F, B, a, n, false, sms, st);
       }
       {
         MfProfScope ps(ctx, MF_PH_EVAL, st, mixed ? (B.vlist ? 4 : 3) : 2);
@@ -1557,7 +1703,7 @@ extern "C" int mf_trace(mf_ctx *ctx, const mf_rbf *rbf, const mf_domain *dom,
       }
       {
         MfProfScope ps(ctx, MF_PH_EXPAND_E, st, 1, (int64_t)n);
-        k_expand_edges<<<g, EXPAND_WARPS * 32, 0, st>>>(F, B, a, n);
+        mf_launch_expand(F, B, a, n, true, sms, st);
       }
     }
     rc = mf_cuda_check(ctx, cudaGetLastError(), "BFS kernels");
