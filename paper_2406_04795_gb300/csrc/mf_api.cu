@@ -23,7 +23,13 @@ extern "C" int mf_ctx_create(int device, size_t budget, mf_ctx **out) {
   size_t freeb = 0, totalb = 0;
   if (cudaMemGetInfo(&freeb, &totalb) != cudaSuccess) { delete c; return MF_ERR_CUDA; }
   c->budget = budget ? budget : (size_t)(0.9 * (double)freeb);
-  if (cudaMallocHost((void **)&c->h_counters, sizeof(MfCounters)) != cudaSuccess) {
+  bool ok = cudaMallocHost((void **)&c->h_counters, 2 * sizeof(MfCounters)) == cudaSuccess;
+  for (int i = 0; i < 2; i++)
+    ok = ok && cudaEventCreateWithFlags(&c->step_event[i], cudaEventDisableTiming) == cudaSuccess;
+  if (!ok) {
+    for (auto e : c->step_event)
+      if (e) cudaEventDestroy(e);
+    if (c->h_counters) cudaFreeHost(c->h_counters);
     delete c;
     return MF_ERR_CUDA;
   }
@@ -95,6 +101,8 @@ extern "C" void mf_ctx_destroy(mf_ctx *c) {
   for (auto e : c->prof.pool) cudaEventDestroy(e);
   for (int s = 0; s < MF_NUM_SLOTS; s++)
     if (c->slot_ptr[s]) cudaFree(c->slot_ptr[s]);
+  for (auto e : c->step_event)
+    if (e) cudaEventDestroy(e);
   if (c->h_counters) cudaFreeHost(c->h_counters);
   delete c;
 }

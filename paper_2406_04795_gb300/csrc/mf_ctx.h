@@ -63,7 +63,8 @@ struct mf_ctx {
   std::string err;
   void *slot_ptr[MF_NUM_SLOTS] = {};
   size_t slot_bytes[MF_NUM_SLOTS] = {};
-  MfCounters *h_counters = nullptr;  // pinned host mirror of the device counters
+  MfCounters *h_counters = nullptr;  // pinned host mirrors of the device counters [2]
+  cudaEvent_t step_event[2] = {};    // the search's reads of them
   MfTraceState last;
   MfSubdivState sub;
   MfProfiler prof;

@@ -2100,7 +2100,7 @@ void mf_b_launch_roots(const MfSlot *slots, MfBatchPlan *P, int n, const int32_t
 // Launchers
 // ---------------------------------------------------------------------------
 void mf_launch_eval_vertices_f64(const MfFrame &F, const MfRbfDev &R, const MfTraceBufs &B,
-                                 const MfTune &T, int sms, cudaStream_t st) {
+                                 const MfTune &T, int sms, cudaStream_t st, bool advance) {
   const int g = sms * T.eval_bps;
   switch (F.d) {
 #define MF_CASE(DD) \
@@ -2109,12 +2109,12 @@ void mf_launch_eval_vertices_f64(const MfFrame &F, const MfRbfDev &R, const MfTr
 #undef MF_CASE
     default: k_eval_vertices_f64<MF_MAXD><<<g, EVAL_WARPS * 32, 0, st>>>(F, R, B);
   }
-  k_advance_eval<<<1, 1, 0, st>>>(B.cnt);
+  if (advance) k_advance_eval<<<1, 1, 0, st>>>(B.cnt);
 }
 
 void mf_launch_eval_vertices_mixed(const MfFrame &F, const MfRbfDev &R, const MfTraceBufs &B,
                                    int precision, double band, const MfTune &T, int sms,
-                                   cudaStream_t st) {
+                                   cudaStream_t st, bool advance) {
   if (precision == MF_MIXED_BF16)
     mf_launch_eval_vertices_tc(F, R, B, band, T.tc_chunk, sms, st);
   else
@@ -2135,7 +2135,7 @@ void mf_launch_eval_vertices_mixed(const MfFrame &F, const MfRbfDev &R, const Mf
 #undef MF_CASE
     default: k_recheck_vertices_f64<MF_MAXD><<<sms * 8, EVAL_WARPS * 32, 0, st>>>(F, R, B);
   }
-  k_advance_eval<<<1, 1, 0, st>>>(B.cnt);
+  if (advance) k_advance_eval<<<1, 1, 0, st>>>(B.cnt);
 }
 
 template <int DD, int MINB>

@@ -59,7 +59,12 @@ struct MfCounters {
   unsigned long long n_defer;      // root steps handed to the lane-per-edge FP64 kernel
   unsigned long long n_defer_list; // their strong-term list entries
   unsigned long long n_redo;       // deferred steps not accepted (solved again in full)
-  unsigned long long n_items;      // expand items of the current chunk given a vertex slot
+  unsigned long long n_items;      // expand items given a vertex slot
+  // the search's current step: edges [lv_begin, lv_begin + lv_n) of the level
+  // that ends at lv_end (lv_n = 0: the search has ended), steps of at most
+  // lv_cap edges, and the levels opened so far
+  unsigned long long lv_begin, lv_end, lv_n, lv_cap, levels;
+  unsigned int lv_ticket;          // blocks of the edges pass that have finished
   unsigned int err_table_full;     // a hash probe ran past the table
   unsigned int err_overflow;       // a list ran past its capacity
   unsigned int err_missing;        // a vertex expected in the table was absent
@@ -588,6 +593,9 @@ void mf_launch_seeds(const MfFrame &F, const MfTraceBufs &B, const double *seeds
                      bool vertices, cudaStream_t s);
 // One pass of the search over edges [e0, e0 + n): the new vertices of their
 // 2-simplex cofaces, or (after those are evaluated) the new crossing edges.
+// n = MF_STEP: the counters' current step, which the edges pass then advances
+// (v_evaluated and n_recheck_done included).
+#define MF_STEP (~0ull)
 void mf_launch_expand(const MfFrame &F, const MfTraceBufs &B, uint64_t e0, uint64_t n, bool edges,
                       int sms, cudaStream_t st);
 // The crossing n-simplices of edges [0, n_edges) with their sign masks and
@@ -608,11 +616,13 @@ struct MfTune {
 
 // Evaluate f at vertex-list entries [begin, end) read from the device counter
 // (FP64 path); writes f into each vertex's table slot.
+// advance: mark them evaluated afterwards (a step of the search leaves that to
+// its edges pass).
 void mf_launch_eval_vertices_f64(const MfFrame &F, const MfRbfDev &R, const MfTraceBufs &B,
-                                 const MfTune &T, int sms, cudaStream_t st);
+                                 const MfTune &T, int sms, cudaStream_t st, bool advance = true);
 void mf_launch_eval_vertices_mixed(const MfFrame &F, const MfRbfDev &R, const MfTraceBufs &B,
                                    int precision, double band, const MfTune &T, int sms,
-                                   cudaStream_t st);
+                                   cudaStream_t st, bool advance = true);
 // fast: the mixed paths' root accuracy (|dt| <= 1e-6 instead of 1e-9), with
 // fewer terms in the FP64 step.
 void mf_launch_roots_f64(const MfFrame &F, const MfRbfDev &R, const MfTraceBufs &B,

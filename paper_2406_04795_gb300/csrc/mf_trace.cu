@@ -422,12 +422,50 @@ __device__ __forceinline__ void expand_range(const MfFrame &F, const MfTraceBufs
   }
 }
 
+// The search's steps live in the counters, so that the host can enqueue several
+// without reading any of them back (see mf_trace).  First step: the seed edges.
+__global__ void k_search_start(MfTraceBufs B, unsigned long long cap) {
+  MfCounters &c = *B.cnt;
+  const bool err = c.err_table_full || c.err_missing || c.err_overflow || c.err_timeout;
+  const unsigned long long ne = err || c.n_edges > B.max_edges ? 0ull : c.n_edges;
+  c.lv_begin = 0;
+  c.lv_end = ne;
+  c.lv_cap = cap;
+  c.lv_n = ne < cap ? ne : cap;
+  c.levels = ne > 0 ? 1 : 0;
+  c.lv_ticket = 0;
+}
+
+// End of a step (one thread, after every block of the edges pass): the rest of
+// the level, or the next one, or no further step when the level appended no
+// edge or an error was set.
+__device__ __forceinline__ void search_next(const MfTraceBufs &B) {
+  volatile MfCounters &c = *B.cnt;
+  const bool err = c.err_table_full || c.err_missing || c.err_overflow || c.err_timeout;
+  const unsigned long long ne = c.n_edges, at = c.lv_begin + c.lv_n;
+  unsigned long long end = c.lv_end;
+  c.v_evaluated = c.n_vertices;
+  c.n_recheck_done = c.n_recheck;
+  if (at >= end && ne > end && ne <= B.max_edges && !err) {
+    end = ne;
+    c.levels = c.levels + 1;
+  }
+  const unsigned long long left = err ? 0ull : end - at;
+  c.lv_begin = at;
+  c.lv_end = end;
+  c.lv_n = left < c.lv_cap ? left : c.lv_cap;
+}
+
 // D < MF_MAXD: the exact dimension, so that the coordinate loops and the key
 // have no predicated axes; MF_MAXD serves the rest at run time.
 template <int D>
 __global__ void __launch_bounds__(EXPAND_WARPS * 32) k_expand_vertices(MfFrame F, MfTraceBufs B,
                                                                        uint64_t e0, uint64_t n) {
   if (D < MF_MAXD) __builtin_assume(F.d == D);
+  if (n == MF_STEP) {
+    e0 = B.cnt->lv_begin;
+    n = B.cnt->lv_n;
+  }
   expand_range<false>(F, B, e0, n);
 }
 
@@ -435,7 +473,24 @@ template <int D>
 __global__ void __launch_bounds__(EXPAND_WARPS * 32) k_expand_edges(MfFrame F, MfTraceBufs B,
                                                                     uint64_t e0, uint64_t n) {
   if (D < MF_MAXD) __builtin_assume(F.d == D);
+  const bool step = n == MF_STEP;
+  if (step) {
+    e0 = B.cnt->lv_begin;
+    n = B.cnt->lv_n;
+    if (n == 0) return;  // every block of the launch sees the same step
+  }
   expand_range<true>(F, B, e0, n);
+  if (step) {  // the last block to finish opens the next step
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      __threadfence();
+      if (atomicAdd(&B.cnt->lv_ticket, 1u) == gridDim.x - 1) {
+        __threadfence();
+        B.cnt->lv_ticket = 0;
+        search_next(B);
+      }
+    }
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -1399,8 +1454,8 @@ void mf_launch_cells_enum(const MfFrame &F, const MfTraceBufs &B, uint64_t n_edg
 void mf_launch_expand(const MfFrame &F, const MfTraceBufs &B, uint64_t e0, uint64_t n, bool edges,
                       int sms, cudaStream_t st) {
   if (n == 0) return;
-  const unsigned g = (unsigned)std::min<uint64_t>((n + EXPAND_WARPS - 1) / EXPAND_WARPS,
-                                                  (uint64_t)sms * 8);
+  const uint64_t full = (uint64_t)sms * 8;
+  const unsigned g = (unsigned)(n == MF_STEP ? full : std::min(full, (n + EXPAND_WARPS - 1) / EXPAND_WARPS));
   switch (F.d) {
 #define MF_CASE(DD)                                                                   \
   case DD:                                                                            \
@@ -1420,6 +1475,8 @@ void mf_launch_seeds(const MfFrame &F, const MfTraceBufs &B, const double *seeds
   if (vertices) k_seed_vertices<<<g, 128, 0, s>>>(F, B, seeds, n);
   else k_seed_edges<<<g, 128, 0, s>>>(F, B, seeds, n);
 }
+
+#define SEARCH_AHEAD 2  // steps enqueued between two reads of the counters (see mf_trace)
 
 static int read_counters(mf_ctx *ctx, const MfTraceBufs &B, cudaStream_t st) {
   int rc = mf_cuda_check(ctx, cudaMemcpyAsync(ctx->h_counters, B.cnt, sizeof(MfCounters),
@@ -1669,9 +1726,11 @@ extern "C" int mf_trace(mf_ctx *ctx, const mf_rbf *rbf, const mf_domain *dom,
   cudaMemsetAsync(B.etab_key, 0xFF, (B.etab_mask + 1) * 16, st);
   cudaMemsetAsync(B.vtab_key, 0xFF, (B.vtab_mask + 1) * 16, st);
 
-  auto eval = [&]() {
-    if (mixed) mf_launch_eval_vertices_mixed(F, R, B, opts->precision, band, ctx->tune, sms, st);
-    else mf_launch_eval_vertices_f64(F, R, B, ctx->tune, sms, st);
+  auto eval = [&](bool advance) {
+    if (mixed)
+      mf_launch_eval_vertices_mixed(F, R, B, opts->precision, band, ctx->tune, sms, st, advance);
+    else
+      mf_launch_eval_vertices_f64(F, R, B, ctx->tune, sms, st, advance);
   };
 
   // Locate edges (Fig. 3)
@@ -1679,42 +1738,50 @@ extern "C" int mf_trace(mf_ctx *ctx, const mf_rbf *rbf, const mf_domain *dom,
     const unsigned g = (unsigned)((n_seeds + 127) / 128);
     MfProfScope ps(ctx, MF_PH_SEEDS, st, mixed ? (B.vlist ? 6 : 5) : 4, n_seeds);
     k_seed_vertices<<<g, 128, 0, st>>>(F, B, seeds, n_seeds);
-    eval();
+    eval(true);
     k_seed_edges<<<g, 128, 0, st>>>(F, B, seeds, n_seeds);
   }
+  k_search_start<<<1, 1, 0, st>>>(B, (unsigned long long)cap);
   rc = mf_cuda_check(ctx, cudaGetLastError(), "seed kernels");
   if (rc) return rc;
-  rc = read_counters(ctx, B, st);
-  if (rc) return rc;
 
-  // Search edges (Fig. 4): one level per pass, each in chunks of <= cap edges.
-  uint64_t fs = 0, fe = ctx->h_counters->n_edges;
-  int64_t levels = fe > 0 ? 1 : 0;
-  while (fe > fs) {
-    for (uint64_t a = fs; a < fe; a += cap) {
-      const uint64_t n = std::min(cap, fe - a);
+  // Search edges (Fig. 4): the kernels of a step take its edges from the
+  // counters, and its edges pass opens the next step, so nothing is read back
+  // in between.  The host keeps two groups of SEARCH_AHEAD steps enqueued and
+  // reads the counters of the older one while the newer one runs; steps after
+  // the last find no edges and return at once (about 6 us each).
+  MfCounters *const hc = ctx->h_counters;  // [2], pinned
+  for (int it = 0;; it++) {
+    for (int k = 0; k < SEARCH_AHEAD; k++) {
       {
-        MfProfScope ps(ctx, MF_PH_EXPAND_V, st, 1, (int64_t)n);
-        mf_launch_expand(F, B, a, n, false, sms, st);
+        MfProfScope ps(ctx, MF_PH_EXPAND_V, st, 1);
+        mf_launch_expand(F, B, 0, MF_STEP, false, sms, st);
       }
       {
-        MfProfScope ps(ctx, MF_PH_EVAL, st, mixed ? (B.vlist ? 4 : 3) : 2);
-        eval();
+        MfProfScope ps(ctx, MF_PH_EVAL, st, mixed ? (B.vlist ? 3 : 2) : 1);
+        eval(false);
       }
       {
-        MfProfScope ps(ctx, MF_PH_EXPAND_E, st, 1, (int64_t)n);
-        mf_launch_expand(F, B, a, n, true, sms, st);
+        MfProfScope ps(ctx, MF_PH_EXPAND_E, st, 1);
+        mf_launch_expand(F, B, 0, MF_STEP, true, sms, st);
       }
     }
-    rc = mf_cuda_check(ctx, cudaGetLastError(), "BFS kernels");
+    cudaMemcpyAsync(&hc[it & 1], B.cnt, sizeof(MfCounters), cudaMemcpyDeviceToHost, st);
+    rc = mf_cuda_check(ctx, cudaEventRecord(ctx->step_event[it & 1], st), "BFS kernels");
     if (rc) return rc;
-    rc = read_counters(ctx, B, st);
+    if (it == 0) continue;
+    rc = mf_cuda_check(ctx, cudaEventSynchronize(ctx->step_event[(it - 1) & 1]), "trace kernels");
     if (rc) return rc;
-    fs = fe;
-    fe = ctx->h_counters->n_edges;
-    if (fe > fs) levels++;
+    if (hc[(it - 1) & 1].lv_n == 0) break;
   }
-  const uint64_t E = fe;
+  rc = read_counters(ctx, B, st);
+  if (rc) return rc;
+  const uint64_t E = hc->n_edges;
+  const int64_t levels = (int64_t)hc->levels;
+  if (ctx->prof.on) {
+    ctx->prof.stats.units[MF_PH_EXPAND_V] += (int64_t)E;
+    ctx->prof.stats.units[MF_PH_EXPAND_E] += (int64_t)E;
+  }
 
   // Roots (the iterative intersection solve of Sec. VI), FP64 Newton.
   if (opts->flags & MF_WANT_ROOTS) {
