@@ -742,54 +742,45 @@ __global__ void k_advance_eval(MfCounters *c) {
 }
 
 // ---------------------------------------------------------------------------
-// Mixed FP32 SIMT evaluator: thread per MIX_VPT points, support vectors in
-// shared memory tiles.  Per point it accumulates
+// Mixed FP32 SIMT evaluator.  Per point it accumulates
 //   acc = sum alpha_j e_j,  A = sum |alpha_j| e_j,  Q = sum |alpha_j| e_j r_j^2
 // and bounds |f~ - f| by the coordinate rounding (eta = 2.01 u (|x|max +
 // |s|max) per coordinate, |r~^2 - r^2| <= 2 eta sqrt(d) r + d eta^2, and
 // sum |alpha| e r <= sqrt(A Q)), the ex2 error (2^-20), the exponent rounding
 // ((d+2) u gamma r^2) and the blocked FP32 summation.
+//
+// Bound by the FP32 pipe: 2 d + 5 operations and one ex2 per term.  A block
+// takes 32 points, lane per point; its warps take the tiles of MIX_TILE
+// support vectors in turn, each staged in the warp's own shared memory and
+// read back four vectors per load by all lanes at once.  The tile sums are
+// added in tile order, so f does not depend on the number of warps.  Splitting
+// the vectors over warps keeps the chip busy at the search's few thousand new
+// vertices per step, where a thread per point ran one long serial loop.
+// Measured against that (GB300): mf_eval of 100,000 points, 8192 vectors, d = 6
+// 2.66 -> 1.43 ms; a d = 4 trace with 333 vectors (2800 new vertices a step)
+// 11.5 -> 9.65 ms.
 // ---------------------------------------------------------------------------
-#define MIX_THREADS 128
-#define MIX_VPT 2
+#define MIX_WARPS 8
 #define MIX_TILE 256
 
-__device__ __forceinline__ void mix_tile_loop(const MfRbfDev &R, const float (*xs)[MF_MAXD],
-                                              float *acc, float *A, float *Q, const float *s_sv,
-                                              const float *s_al, int cnt, float g2) {
-  for (int j = 0; j < cnt; j++) {
-    float s[MF_MAXD];
-#pragma unroll
-    for (int k = 0; k < MF_MAXD; k++) s[k] = k < R.d ? s_sv[k * MIX_TILE + j] : 0.f;
-    const float al = s_al[j];
-    const float aa = fabsf(al);
-#pragma unroll
-    for (int v = 0; v < MIX_VPT; v++) {
-      float r2 = 0.f;
-#pragma unroll
-      for (int k = 0; k < MF_MAXD; k++)
-        if (k < R.d) {
-          float t = xs[v][k] - s[k];
-          r2 = fmaf(t, t, r2);
-        }
-      const float e = ex2_approx(-g2 * r2);
-      acc[v] = fmaf(al, e, acc[v]);
-      const float ae = aa * e;
-      A[v] += ae;
-      Q[v] = fmaf(ae, r2, Q[v]);
-    }
-  }
-}
+template <int D>
+struct MixShared {
+  double x[D][32];
+  float part[MIX_WARPS][32], A[MIX_WARPS][32], Q[MIX_WARPS][32];
+  // [warp][axis, then alpha][MIX_TILE], 16-byte rows; the launch reserves it
+  // for its own number of warps
+  __align__(16) float sv[1][D + 1][MIX_TILE];
+};
 
 // Source of points: vertex list (lattice) or a plain [n][d] array.
-template <bool VERTS>
-__global__ void __launch_bounds__(MIX_THREADS) k_eval_mixed_f32(MfFrame F, MfRbfDev R, MfTraceBufs B,
-                                                                const double *pts, int64_t npts,
-                                                                double *fout, uint8_t *flag,
-                                                                double band) {
-  __shared__ float s_sv[MF_MAXD * MIX_TILE];
-  __shared__ float s_al[MIX_TILE];
-  const int d = R.d;
+template <bool VERTS, int D>
+__global__ void __launch_bounds__(MIX_WARPS * 32) k_eval_mixed_f32(MfFrame F, MfRbfDev R, MfTraceBufs B,
+                                                                   const double *pts, int64_t npts,
+                                                                   double *fout, uint8_t *flag,
+                                                                   double band) {
+  extern __shared__ __align__(16) unsigned char mix_raw[];
+  MixShared<D> &sh = *reinterpret_cast<MixShared<D> *>(mix_raw);
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, W = blockDim.x >> 5;
   uint64_t begin = 0, end = (uint64_t)npts;
   if (VERTS) {
     begin = B.cnt->v_evaluated;
@@ -798,85 +789,154 @@ __global__ void __launch_bounds__(MIX_THREADS) k_eval_mixed_f32(MfFrame F, MfRbf
   }
   const float g2 = (float)(R.gamma * 1.4426950408889634);
   const double u = 5.9604644775390625e-08;  // 2^-24
-  const uint64_t per_block = (uint64_t)MIX_THREADS * MIX_VPT;
-  for (uint64_t base = begin + (uint64_t)blockIdx.x * per_block; base < end;
-       base += (uint64_t)gridDim.x * per_block) {
-    float xs[MIX_VPT][MF_MAXD];
-    double xmax[MIX_VPT];
-    uint64_t idx[MIX_VPT];
-#pragma unroll
-    for (int v = 0; v < MIX_VPT; v++) {
-      idx[v] = base + (uint64_t)v * MIX_THREADS + threadIdx.x;
-      double x[MF_MAXD];
-#pragma unroll
-      for (int k = 0; k < MF_MAXD; k++) x[k] = 0.0;
-      if (idx[v] < end) {
+  for (uint64_t base = begin + (uint64_t)blockIdx.x * 32; base < end; base += (uint64_t)gridDim.x * 32) {
+    // the points' coordinates, one (axis, point) per thread (mf_vertex_x's
+    // operation order)
+    for (int q = threadIdx.x; q < 32 * D; q += blockDim.x) {
+      const int k = q >> 5;
+      const uint64_t i = base + lane;
+      double x = 0.0;
+      if (i < end) {
         if (VERTS) {
-          int32_t y[MF_MAXD];
+          long long s = 0;
+          int32_t yk = 0;
 #pragma unroll
-          for (int k = 0; k < MF_MAXD; k++) y[k] = k < d ? B.vert_y[idx[v] * d + k] : 0;
-          mf_vertex_x(F, y, x);
+          for (int m = 0; m < D; m++) {
+            const int32_t y = B.vert_y[i * D + m];
+            s += y;
+            if (m == k) yk = y;
+          }
+          x = __dadd_rn(__dmul_rn(F.lam, __dsub_rn((double)yk, __dmul_rn(F.c, (double)s))), F.o[k]);
         } else {
-#pragma unroll
-          for (int k = 0; k < MF_MAXD; k++) x[k] = k < d ? pts[idx[v] * d + k] : 0.0;
+          x = pts[i * D + k];
         }
       }
-      xmax[v] = 0.0;
+      sh.x[k][lane] = x;
+    }
+    __syncthreads();
+    float xs[D];
 #pragma unroll
-      for (int k = 0; k < MF_MAXD; k++) {
-        xs[v][k] = (float)x[k];
-        xmax[v] = fmax(xmax[v], fabs(x[k]));
+    for (int k = 0; k < D; k++) xs[k] = (float)sh.x[k][lane];
+    float acc = 0.f, A = 0.f, Q = 0.f;
+    for (int t0 = 0; t0 < R.n; t0 += W * MIX_TILE) {
+      const int j0 = t0 + w * MIX_TILE;
+      float part = 0.f;
+      if (j0 < R.n) {
+        const int cnt = min(MIX_TILE, R.n - j0), cnt4 = (cnt + 3) & ~3;
+        __syncwarp();  // the warp's previous tile has been read
+        for (int i = lane; i < cnt4; i += 32) {
+          const bool in = i < cnt;  // the padding adds zeros
+#pragma unroll
+          for (int k = 0; k < D; k++) sh.sv[w][k][i] = in ? R.sv32[(int64_t)k * R.n + j0 + i] : 0.f;
+          sh.sv[w][D][i] = in ? R.alpha32[j0 + i] : 0.f;
+        }
+        __syncwarp();
+#pragma unroll 2
+        for (int j = 0; j < cnt4; j += 4) {
+          float r2[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+          for (int k = 0; k < D; k++) {
+            const float4 s = *reinterpret_cast<const float4 *>(&sh.sv[w][k][j]);
+            const float t[4] = {xs[k] - s.x, xs[k] - s.y, xs[k] - s.z, xs[k] - s.w};
+#pragma unroll
+            for (int i = 0; i < 4; i++) r2[i] = fmaf(t[i], t[i], r2[i]);
+          }
+          const float4 a4 = *reinterpret_cast<const float4 *>(&sh.sv[w][D][j]);
+          const float al[4] = {a4.x, a4.y, a4.z, a4.w};
+#pragma unroll
+          for (int i = 0; i < 4; i++) {
+            const float e = ex2_approx(-g2 * r2[i]);
+            part = fmaf(al[i], e, part);
+            const float ae = fabsf(al[i]) * e;
+            A += ae;
+            Q = fmaf(ae, r2[i], Q);
+          }
+        }
+      }
+      if (W == 1) {
+        acc += part;
+      } else {
+        sh.part[w][lane] = part;
+        __syncthreads();
+        if (w == 0)
+          for (int q = 0; q < W && t0 + q * MIX_TILE < R.n; q++) acc += sh.part[q][lane];
+        __syncthreads();
       }
     }
-    float acc[MIX_VPT], A[MIX_VPT], Q[MIX_VPT];
-#pragma unroll
-    for (int v = 0; v < MIX_VPT; v++) acc[v] = A[v] = Q[v] = 0.f;
-    for (int t0 = 0; t0 < R.n; t0 += MIX_TILE) {
-      const int cnt = min(MIX_TILE, R.n - t0);
+    if (W > 1) {
+      sh.A[w][lane] = A;
+      sh.Q[w][lane] = Q;
       __syncthreads();
-      for (int i = threadIdx.x; i < cnt; i += MIX_THREADS) {
-        for (int k = 0; k < d; k++) s_sv[k * MIX_TILE + i] = R.sv32[(int64_t)k * R.n + t0 + i];
-        s_al[i] = R.alpha32[t0 + i];
-      }
-      __syncthreads();
-      float part[MIX_VPT];
-#pragma unroll
-      for (int v = 0; v < MIX_VPT; v++) part[v] = 0.f;
-      mix_tile_loop(R, xs, part, A, Q, s_sv, s_al, cnt, g2);
-#pragma unroll
-      for (int v = 0; v < MIX_VPT; v++) acc[v] += part[v];
     }
+    const uint64_t i = base + lane;
+    if (w == 0 && i < end) {
+      for (int q = 1; q < W; q++) {
+        A += sh.A[q][lane];
+        Q += sh.Q[q][lane];
+      }
+      double xmax = 0.0;
 #pragma unroll
-    for (int v = 0; v < MIX_VPT; v++) {
-      if (idx[v] >= end) continue;
-      const double D = xmax[v] + (double)R.smax;
-      const double eta = 2.01 * u * D;
-      const double Av = (double)A[v], Qv = (double)Q[v];
-      const double coord = R.gamma * (2.0 * eta * sqrt((double)d) * sqrt(Av * Qv) + d * eta * eta * Av);
+      for (int k = 0; k < D; k++) xmax = fmax(xmax, fabs(sh.x[k][lane]));
+      const double Dm = xmax + (double)R.smax;
+      const double eta = 2.01 * u * Dm;
+      const double Av = (double)A, Qv = (double)Q;
+      const double coord =
+          R.gamma * (2.0 * eta * sqrt((double)D) * sqrt(Av * Qv) + D * eta * eta * Av);
       const double eps_exp = 9.5367431640625e-07;  // 2^-20, above ex2.approx's error
       const double nsum = (double)MIX_TILE + (double)R.n / MIX_TILE + 2.0;  // blocked FP32 sums
       const double bound = (coord + Av * (eps_exp + (nsum + 2.0) * u) +
-                            Qv * R.gamma * (d + 2) * u) * 1.02 + 1e-30;
-      const double fx = (double)acc[v] + R.b;
+                            Qv * R.gamma * (D + 2) * u) * 1.02 + 1e-30;
+      const double fx = (double)acc + R.b;
       const bool recheck = fabs(fx) <= fmax(bound, band);
       if (VERTS) {
-        const uint32_t slot = B.vert_slot[idx[v]];
+        const uint32_t slot = B.vert_slot[i];
         mf_vtab_f(B, slot) = fx;
         if (recheck) {
           unsigned long long q = atomicAdd(&B.cnt->n_recheck, 1ull);
-          if (q < B.max_vertices) B.recheck[q] = (uint32_t)idx[v];
+          if (q < B.max_vertices) B.recheck[q] = (uint32_t)i;
           else atomicOr(&B.cnt->err_overflow, 1u);
         }
       } else {
-        fout[idx[v]] = fx;
-        flag[idx[v]] = recheck ? 1 : 0;
+        fout[i] = fx;
+        flag[i] = recheck ? 1 : 0;
       }
     }
+    __syncthreads();  // the next points' coordinates and sums
+  }
+}
+
+// Launch: a warp per tile up to MIX_WARPS, and as many blocks as the points
+// need (n_max: their number, or an upper bound) up to what fits the chip.
+template <bool VERTS, int D>
+static void launch_mixed_f32_d(const MfFrame &F, const MfRbfDev &R, const MfTraceBufs &B,
+                               const double *pts, int64_t npts, double *fout, uint8_t *flag,
+                               double band, int sms, cudaStream_t st) {
+  const int W = std::min(MIX_WARPS, (R.n + MIX_TILE - 1) / MIX_TILE);
+  const int bytes = (int)(sizeof(MixShared<D>) + (W - 1) * sizeof(MixShared<D>::sv));
+  cudaFuncSetAttribute(k_eval_mixed_f32<VERTS, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  const int64_t full = (int64_t)sms * 8;
+  const int64_t g = VERTS ? full : std::min(full, (npts + 31) / 32);
+  k_eval_mixed_f32<VERTS, D><<<(unsigned)g, W * 32, bytes, st>>>(F, R, B, pts, npts, fout, flag, band);
+}
+
+template <bool VERTS>
+static void launch_mixed_f32(const MfFrame &F, const MfRbfDev &R, const MfTraceBufs &B,
+                             const double *pts, int64_t npts, double *fout, uint8_t *flag,
+                             double band, int sms, cudaStream_t st) {
+  switch (R.d) {
+#define MF_CASE(DD)                                                                           \
+  case DD: launch_mixed_f32_d<VERTS, DD>(F, R, B, pts, npts, fout, flag, band, sms, st); break;
+    MF_CASE(2) MF_CASE(3) MF_CASE(4) MF_CASE(5) MF_CASE(6) MF_CASE(7) MF_CASE(8)
+#undef MF_CASE
+    default: break;
   }
 }
 
 // FP64 evaluation of flagged plain points (mf_eval mixed recheck), or of all
 // points when flag == NULL.
+// Exact dimensions: 200,000 points, 2048 vectors, d = 5: 1.87 -> 1.22 ms
+// against the run-time d.
+template <int D>
 __global__ void __launch_bounds__(EVAL_WARPS * 32) k_eval_points_f64(MfRbfDev R, const double *pts, int64_t n,
                                                         double *fout, const uint8_t *flag) {
   __shared__ int sq[EVAL_WARPS][2][64];
@@ -885,11 +945,23 @@ __global__ void __launch_bounds__(EVAL_WARPS * 32) k_eval_points_f64(MfRbfDev R,
   unsigned long long terms[2] = {0, 0};
   for (int64_t i = (int64_t)blockIdx.x * EVAL_WARPS + w; i < n; i += nwarps) {
     if (flag && !flag[i]) continue;
-    double x[MF_MAXD];
+    double x[D];
 #pragma unroll
-    for (int k = 0; k < MF_MAXD; k++) x[k] = k < R.d ? pts[i * R.d + k] : 0.0;
-    F64Acc a = warp_f64<false, MF_MAXD>(R, x, nullptr, sq[w][0], sq[w][1], terms);
+    for (int k = 0; k < D; k++) x[k] = k < R.d ? pts[i * R.d + k] : 0.0;
+    F64Acc a = warp_f64<false, D>(R, x, nullptr, sq[w][0], sq[w][1], terms);
     if (lane == 0) fout[i] = a.f;
+  }
+}
+
+static void launch_eval_points_f64(const MfRbfDev &R, const double *pts, int64_t n, double *fout,
+                                   const uint8_t *flag, int sms, cudaStream_t st) {
+  const unsigned g = (unsigned)std::min<int64_t>((int64_t)sms * 8, (n + EVAL_WARPS - 1) / EVAL_WARPS);
+  switch (R.d) {
+#define MF_CASE(DD) \
+  case DD: k_eval_points_f64<DD><<<g, EVAL_WARPS * 32, 0, st>>>(R, pts, n, fout, flag); break;
+    MF_CASE(2) MF_CASE(3) MF_CASE(4) MF_CASE(5) MF_CASE(6) MF_CASE(7)
+#undef MF_CASE
+    default: k_eval_points_f64<MF_MAXD><<<g, EVAL_WARPS * 32, 0, st>>>(R, pts, n, fout, flag);
   }
 }
 
@@ -2118,7 +2190,7 @@ void mf_launch_eval_vertices_mixed(const MfFrame &F, const MfRbfDev &R, const Mf
   if (precision == MF_MIXED_BF16)
     mf_launch_eval_vertices_tc(F, R, B, band, T.tc_chunk, sms, st);
   else
-    k_eval_mixed_f32<true><<<sms * 4, MIX_THREADS, 0, st>>>(F, R, B, nullptr, 0, nullptr, nullptr, band);
+    launch_mixed_f32<true>(F, R, B, nullptr, 0, nullptr, nullptr, band, sms, st);
   if (B.vlist) {  // the root screen's per-vertex lists
     switch (F.d) {
 #define MF_CASE(DD) \
@@ -2356,16 +2428,15 @@ extern "C" int mf_eval(mf_ctx *ctx, const mf_rbf *rbf, const double *q, int64_t 
   if (n == 0) return MF_OK;
   const int sms = ctx->sms;
   if (precision == MF_FP64) {
-    k_eval_points_f64<<<sms * 8, EVAL_WARPS * 32, 0, st>>>(R, q, n, f_out, nullptr);
+    launch_eval_points_f64(R, q, n, f_out, nullptr, sms, st);
   } else {
     uint8_t *flag = (uint8_t *)mf_ctx_buffer(ctx, MF_SLOT_SCAN, (size_t)n + 256);
     if (!flag) return MF_ERR_OOM;
     MfFrame F;
     mf_frame_lattice(&F, R.d, 1.0, nullptr);
     MfTraceBufs B = {};
-    k_eval_mixed_f32<false><<<sms * 4, MIX_THREADS, 0, st>>>(F, R, B, q, n, f_out, flag,
-                                                             band > 0 ? band : 1e-3);
-    k_eval_points_f64<<<sms * 8, EVAL_WARPS * 32, 0, st>>>(R, q, n, f_out, flag);
+    launch_mixed_f32<false>(F, R, B, q, n, f_out, flag, band > 0 ? band : 1e-3, sms, st);
+    launch_eval_points_f64(R, q, n, f_out, flag, sms, st);
   }
   rc = mf_cuda_check(ctx, cudaGetLastError(), "mf_eval launch");
   if (rc) return rc;
