@@ -306,10 +306,10 @@ extern "C" int mf_trace_batch(mf_ctx *ctx, int32_t n, const mf_rbf *rbfs, const 
     if (hs[t].err)
       return mf_set_error(ctx, MF_ERR_MAXEDGES, "trace %d exceeded its capacities or a table", t);
   // --- roots and cells of all traces
+  uint32_t dims = 0;
+  for (int t = 0; t < n; t++) dims |= 1u << slots[t].F.d;
   {
     MfProfScope ps(ctx, MF_PH_ROOTS, st, 2);
-    uint32_t dims = 0;
-    for (int t = 0; t < n; t++) dims |= 1u << slots[t].F.d;
     mf_b_launch_roots(d_slots, d_plan, n, nullptr, dims, ctx->tune.roots_group, sms, st);
   }
   bool any_cells = false;
@@ -319,7 +319,7 @@ extern "C" int mf_trace_batch(mf_ctx *ctx, int32_t n, const mf_rbf *rbfs, const 
   if (any_cells) {
     {
       MfProfScope ps(ctx, MF_PH_CELLS, st, 2);
-      mf_b_launch_cells(d_slots, d_plan, n, nullptr, sms, st);
+      mf_b_launch_cells(d_slots, d_plan, n, nullptr, dims, sms, st);
     }
     for (int t = 0; t < n; t++)
       cudaMemcpyAsync(&hc[t], slots[t].B.cnt, sizeof(MfCounters), cudaMemcpyDeviceToHost, st);
@@ -767,7 +767,7 @@ extern "C" int mf_server_step(mf_server *s, void *stream, int32_t *n_running, in
     bool cells = false;
     for (int t : fin) cells = cells || (s->slots[t].flags & MF_WANT_CELLS);
     if (cells) {
-      mf_b_launch_cells(s->d_slots, s->d_plan, n, s->d_only, sms, st);
+      mf_b_launch_cells(s->d_slots, s->d_plan, n, s->d_only, dims, sms, st);
       for (int t : fin)
         if (s->slot_req[t] >= 0)
           cudaMemcpyAsync(&s->reqs[s->slot_req[t]].cnt, s->slots[t].B.cnt, sizeof(MfCounters),

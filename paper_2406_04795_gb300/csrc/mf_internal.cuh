@@ -212,8 +212,9 @@ void mf_b_launch_update(const MfSlot *slots, MfSlotState *st, MfBatchPlan *P, in
 // dim > 0 restricts mode 0 (roots) to the slots of that dimension.
 void mf_b_launch_plan_edges(const MfSlot *slots, MfBatchPlan *P, int n, int cells,
                             const int32_t *only, cudaStream_t s, int dim = 0);
-void mf_b_launch_cells(const MfSlot *slots, MfBatchPlan *P, int n, const int32_t *only, int sms,
-                       cudaStream_t s);
+// dims: bit d set when some slot has dimension d (one exact-d launch each).
+void mf_b_launch_cells(const MfSlot *slots, MfBatchPlan *P, int n, const int32_t *only,
+                       uint32_t dims, int sms, cudaStream_t s);
 void mf_b_launch_cell_edges(const MfSlot *slots, MfBatchPlan *P, int n, bool fill,
                             const int32_t *only, int sms, cudaStream_t s);
 // Vertex evaluation of every slot: FP64 or FP32 SIMT warps, the tensor-core

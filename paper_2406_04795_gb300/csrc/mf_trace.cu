@@ -528,33 +528,39 @@ __constant__ uint32_t c_fact[13] = {1u, 1u, 2u, 6u, 24u, 120u, 720u, 5040u, 4032
 // y + e(M) for M within S (a), y + e(S) + e(M) (b) or y - e(M) (c) for M
 // within T = {0..d-1} \ S, indexed by M's bits compressed to S or T.
 // Entry bit 0: in the vertex table (in the domain); bit 1: f >= 0.
-#define LINK_MAX (1 << MF_MAXD)
+template <int D>
 struct CellLink {
-  uint8_t a[LINK_MAX], b[LINK_MAX], c[LINK_MAX];
-  uint16_t cnt[LINK_MAX];      // chains of p1 prefixes (subsets of S)
-  uint16_t cc[LINK_MAX / 2];   // chains of suffix sets after d (subsets of T)
-  uint32_t cum[LINK_MAX / 2 + 1];  // prefix sums of the p2 orderings per suffix set
+  static constexpr int NA = 1 << D, NT = 1 << (D - 1);
+  uint32_t cum[NT + 1];  // prefix sums of the p2 orderings per suffix set
+  uint16_t cnt[NA];      // chains of p1 prefixes (subsets of S)
+  uint16_t cc[NT];       // chains of suffix sets after d (subsets of T)
+  uint8_t a[NA], b[NT], c[NT];
 };
 #define CELL_WARPS 8
 
-__device__ __forceinline__ void cells_enum_edge(const MfFrame &F, const MfTraceBufs &B, uint64_t e,
-                                                int lane, CellLink &L);
+// Lanes per edge.  The work of an edge is its link table (2^|S| + 2^(d-|S|+1)
+// entries), the chain counts of as many subsets, and its cells (about 1.5 at
+// d = 3, 3 at d = 4, 8 at d = 5, 29 at d = 6): a whole warp leaves most lanes
+// idle below d = 6, and the kernel is bound by instruction issue (63 % of the
+// cycles at d = 5).  A warp per edge -> W lanes: 11.6 -> 7.9 ms for the edges
+// of a d = 5 proof at lambda = 0.08, 2.12 -> 1.46 ms at 0.15, 0.86 -> 0.34 ms
+// for a d = 4 proof; at d = 6 the two measure alike (2.5 and 2.6 ms).
+template <int D>
+struct CellLanes {
+  static constexpr int W = D <= 3 ? 4 : D <= 5 ? 8 : D == 6 ? 16 : 32;
+};
 
-__global__ void __launch_bounds__(CELL_WARPS * 32) k_cells_enum(MfFrame F, MfTraceBufs B,
-                                                                uint64_t n_edges) {
-  __shared__ CellLink sl[CELL_WARPS];
-  const int lane = threadIdx.x & 31;
-  const uint64_t e = (blockIdx.x * (uint64_t)blockDim.x + threadIdx.x) >> 5;
-  if (e >= n_edges) return;
-  cells_enum_edge(F, B, e, lane, sl[threadIdx.x >> 5]);
-}
-
-// The n-cofaces j = lane, lane + 32, ... of edge e (all lanes of the warp).
-// Orderings and permutations are kept as 4-bit nibbles in 64-bit words, so
-// the decode needs no indexed arrays (they would live in local memory).
+// The cells of edge e (W lanes of the warp; all 32 lanes call together; have
+// false: some edge of the range all the same, whose cells are not written).
+// Orderings and permutations are kept as 4-bit nibbles in 64-bit words, so the
+// decode needs no indexed arrays (they would live in local memory).  ONE: the
+// warp's edges belong to one trace.
+template <int D, bool ONE>
 __device__ __forceinline__ void cells_enum_edge(const MfFrame &F, const MfTraceBufs &B, uint64_t e,
-                                                int lane, CellLink &L) {
-  const int d = F.d;
+                                                bool have, CellLink<D> &L) {
+  constexpr int W = CellLanes<D>::W;
+  const int lane = threadIdx.x & 31, sl = lane & (W - 1);
+  const int d = D < MF_MAXD ? D : F.d;
   int32_t y[MF_MAXD];
   load_y(B.edge_y + e * d, d, y);
   const uint32_t S = B.edge_mask[e], T = ~S & ((1u << d) - 1u);
@@ -567,8 +573,8 @@ __device__ __forceinline__ void cells_enum_edge(const MfFrame &F, const MfTraceB
   // and the one after), whose vertex slots the expansion recorded
   const unsigned long long ioff = B.edge_item_off ? B.edge_item_off[e] : ~0ull;
   const uint8_t c_y = B.edge_f[2 * e] >= 0.0 ? 3 : 1, c_ys = B.edge_f[2 * e + 1] >= 0.0 ? 3 : 1;
-  __syncwarp();  // the previous edge's cofaces have read the table
-  for (int q = lane; q < na + 2 * nb; q += 32) {
+  __syncwarp();  // the previous edges' cells have read the tables
+  for (int q = sl; q < na + 2 * nb; q += W) {
     uint8_t *dst;
     uint32_t M;
     int sgn = 1;
@@ -624,36 +630,10 @@ __device__ __forceinline__ void cells_enum_edge(const MfFrame &F, const MfTraceB
   // prefix sets all pass B (U = S itself always passes); cc[W] = orderings
   // of W, built from its last element, whose suffix sets all pass A
   const uint32_t ys = (L.a[0] >> 1) & 1u;
-  if (na <= 32 && nc <= 32) {
-    // lane u holds cnt[u] and cc[u]; each level sums the lanes one bit below
-    const uint32_t u = (uint32_t)lane;
-    const uint32_t ca = u < (uint32_t)na ? L.a[u] : 0u;
-    const bool oka = u < (uint32_t)na && (u == (uint32_t)(na - 1) || !(ca & 1u) || ((ca >> 1) & 1u) == ys);
-    const bool okc = u < (uint32_t)nc && !(L.c[u] & 1u);
-    uint32_t cv = u == 0 ? 1u : 0u, qv = u == 0 ? 1u : 0u;
-    const int levels = n1 > nt ? n1 : nt;
-    for (int lev = 1; lev <= levels; lev++) {
-      uint32_t sa = 0, sc = 0;
-#pragma unroll
-      for (int b = 0; b < 5; b++) {
-        const uint32_t va = __shfl_xor_sync(0xffffffffu, cv, 1 << b);
-        const uint32_t vc = __shfl_xor_sync(0xffffffffu, qv, 1 << b);
-        if ((u >> b) & 1u) {
-          sa += va;
-          sc += vc;
-        }
-      }
-      if (__popc(u) == lev) {
-        cv = oka ? sa : 0u;
-        qv = okc ? sc : 0u;
-      }
-    }
-    if (u < (uint32_t)na) L.cnt[u] = (uint16_t)cv;
-    if (u < (uint32_t)nc) L.cc[u] = (uint16_t)qv;
-    __syncwarp();
-  } else
-  for (int lev = 0; lev <= n1 || lev <= nt; lev++) {
-    for (int u = lane; u < na; u += 32) {
+  const int levels = (int)__reduce_max_sync(0xffffffffu, (unsigned)(n1 > nt ? n1 : nt));
+  const int most_nc = 1 << __reduce_max_sync(0xffffffffu, (unsigned)nt);
+  for (int lev = 0; lev <= levels; lev++) {
+    for (int u = sl; u < na; u += W) {
       if (__popc(u) != lev) continue;
       uint32_t v = 1;
       if (u) {
@@ -664,7 +644,7 @@ __device__ __forceinline__ void cells_enum_edge(const MfFrame &F, const MfTraceB
       }
       L.cnt[u] = (uint16_t)v;
     }
-    for (int w = lane; w < nc; w += 32) {
+    for (int w = sl; w < nc; w += W) {
       if (__popc(w) != lev) continue;
       uint32_t v = 1;
       if (w) {
@@ -679,25 +659,38 @@ __device__ __forceinline__ void cells_enum_edge(const MfFrame &F, const MfTraceB
   // cum[w]: p2 orderings whose suffix set (compressed) is below w: each set
   // W contributes cc[W] (|T| - |W|)! (the rest of T in any order before d)
   uint32_t run = 0;
-  for (int base = 0; base < nc; base += 32) {
-    const int w = base + lane;
+  for (int w0 = 0; w0 < most_nc; w0 += W) {
+    const int w = w0 + sl;
     uint32_t inc = w < nc ? (uint32_t)L.cc[w] * c_fact[nt - __popc(w)] : 0u;
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const uint32_t v = __shfl_up_sync(0xffffffffu, inc, o);
-      if (lane >= o) inc += v;
+    for (int o = 1; o < W; o <<= 1) {
+      const uint32_t v = __shfl_up_sync(0xffffffffu, inc, o, W);
+      if (sl >= o) inc += v;
     }
     if (w < nc) L.cum[w + 1] = run + inc;
-    run += __shfl_sync(0xffffffffu, inc, 31);
+    run += __shfl_sync(0xffffffffu, inc, W - 1, W);
   }
-  if (lane == 0) L.cum[0] = 0;
+  if (sl == 0) L.cum[0] = 0;
   __syncwarp();
-  const uint32_t c1 = L.cnt[na - 1], total = c1 * run;
-  if (total == 0) return;
+  const uint32_t c1 = L.cnt[na - 1], total = have ? c1 * run : 0u;
+  // room for the warp's cells: one atomic where its edges share the counter
   unsigned long long base = 0;
-  if (lane == 0) base = atomicAdd(&B.cnt->n_cells, (unsigned long long)total);
-  base = __shfl_sync(0xffffffffu, base, 0);
-  for (uint32_t k = lane; k < total; k += 32) {
+  if (ONE) {
+    uint32_t my = 0, all = 0;
+#pragma unroll
+    for (int q = 0; q < 32 / W; q++) {
+      const uint32_t v = __shfl_sync(0xffffffffu, total, q * W);
+      if (q < lane / W) my += v;
+      all += v;
+    }
+    if (all == 0) return;
+    if (lane == 0) base = atomicAdd(&B.cnt->n_cells, (unsigned long long)all);
+    base = __shfl_sync(0xffffffffu, base, 0) + my;
+  } else {
+    if (sl == 0 && total) base = atomicAdd(&B.cnt->n_cells, (unsigned long long)total);
+    base = __shfl_sync(0xffffffffu, base, 0, W);
+  }
+  for (uint32_t k = sl; k < total; k += W) {
     const unsigned long long idx = base + k;
     if (idx >= B.max_cells) { atomicOr(&B.cnt->err_overflow, 1u); continue; }
     // unrank: k = k1 + c1 k2; the ordering of S from its last element back
@@ -808,6 +801,19 @@ __device__ __forceinline__ void cells_enum_edge(const MfFrame &F, const MfTraceB
     if (B.cell_sgn) B.cell_sgn[idx] = inm | (posm << 16);
     if (B.cell_off) B.cell_off[idx] = (int64_t)__popc(P) * (int64_t)__popc(N);
   }
+}
+
+template <int D>
+__global__ void __launch_bounds__(CELL_WARPS * 32) k_cells_enum(MfFrame F, MfTraceBufs B,
+                                                                uint64_t n_edges) {
+  constexpr int W = CellLanes<D>::W, PER = 32 / W;
+  __shared__ CellLink<D> sl[CELL_WARPS * PER];
+  if (D < MF_MAXD) __builtin_assume(F.d == D);
+  const uint64_t first = (blockIdx.x * (uint64_t)CELL_WARPS + (threadIdx.x >> 5)) * PER;
+  if (first >= n_edges) return;  // whole warp
+  const uint64_t e = first + (threadIdx.x & 31) / W;
+  const bool have = e < n_edges;
+  cells_enum_edge<D, true>(F, B, have ? e : first, have, sl[threadIdx.x / W]);
 }
 
 // Cell -> traced edges: the (d+1)d/2 edges of the cell (query type 2) found
@@ -1149,16 +1155,22 @@ __global__ void k_b_plan_edges(const MfSlot *slots, MfBatchPlan *P, int n, int m
   if (t == 0) p[n] = total;
 }
 
+// Cells of the slots of dimension D (the plan's pe prefix holds only those).
+template <int D>
 __global__ void __launch_bounds__(CELL_WARPS * 32) k_b_cells_enum(const MfSlot *slots,
                                                                   const MfBatchPlan *P, int n) {
-  __shared__ CellLink sl[CELL_WARPS];
+  constexpr int W = CellLanes<D>::W, PER = 32 / W;
+  __shared__ CellLink<D> sl[CELL_WARPS * PER];
   const unsigned long long total = P->pe[n];
-  const int lane = threadIdx.x & 31;
-  const unsigned long long nwarps = ((unsigned long long)gridDim.x * blockDim.x) >> 5;
-  for (unsigned long long item = (blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x) >> 5;
-       item < total; item += nwarps) {
+  const unsigned long long step = (unsigned long long)gridDim.x * CELL_WARPS * PER;
+  for (unsigned long long first =
+           (blockIdx.x * (unsigned long long)CELL_WARPS + (threadIdx.x >> 5)) * PER;
+       first < total; first += step) {
+    unsigned long long item = first + (threadIdx.x & 31) / W;
+    const bool have = item < total;
+    if (!have) item = first;
     const int t = mf_slot_of(P->pe, n, item);
-    cells_enum_edge(slots[t].F, slots[t].B, item - P->pe[t], lane, sl[threadIdx.x >> 5]);
+    cells_enum_edge<D, false>(slots[t].F, slots[t].B, item - P->pe[t], have, sl[threadIdx.x / W]);
   }
 }
 
@@ -1201,10 +1213,19 @@ void mf_b_launch_plan_edges(const MfSlot *slots, MfBatchPlan *P, int n, int cell
                             const int32_t *only, cudaStream_t s, int dim) {
   k_b_plan_edges<<<1, MF_MAX_SLOTS, 0, s>>>(slots, P, n, cells, only, dim);
 }
-void mf_b_launch_cells(const MfSlot *slots, MfBatchPlan *P, int n, const int32_t *only, int sms,
-                       cudaStream_t s) {
-  k_b_plan_edges<<<1, MF_MAX_SLOTS, 0, s>>>(slots, P, n, 2, only, 0);
-  k_b_cells_enum<<<sms * 8, 256, 0, s>>>(slots, P, n);
+void mf_b_launch_cells(const MfSlot *slots, MfBatchPlan *P, int n, const int32_t *only,
+                       uint32_t dims, int sms, cudaStream_t s) {
+  for (int dd = 2; dd <= MF_MAXD; dd++) {
+    if (!((dims >> dd) & 1u)) continue;
+    k_b_plan_edges<<<1, MF_MAX_SLOTS, 0, s>>>(slots, P, n, 2, only, dd);
+    switch (dd) {
+#define MF_CASE(DD) \
+  case DD: k_b_cells_enum<DD><<<sms * 8, CELL_WARPS * 32, 0, s>>>(slots, P, n); break;
+      MF_CASE(2) MF_CASE(3) MF_CASE(4) MF_CASE(5) MF_CASE(6) MF_CASE(7) MF_CASE(8)
+#undef MF_CASE
+      default: break;
+    }
+  }
 }
 void mf_b_launch_cell_edges(const MfSlot *slots, MfBatchPlan *P, int n, bool fill,
                             const int32_t *only, int sms, cudaStream_t s) {
@@ -1447,7 +1468,16 @@ void mf_launch_cells_fill(const MfFrame &F, const MfTraceBufs &B, uint64_t n_cel
 }
 void mf_launch_cells_enum(const MfFrame &F, const MfTraceBufs &B, uint64_t n_edges, cudaStream_t st) {
   if (n_edges == 0) return;
-  k_cells_enum<<<(unsigned)((n_edges * 32 + 255) / 256), 256, 0, st>>>(F, B, n_edges);
+  switch (F.d) {
+#define MF_CASE(DD)                                                                         \
+  case DD: {                                                                                \
+    constexpr uint64_t per = CELL_WARPS * (32 / CellLanes<DD>::W);                          \
+    k_cells_enum<DD><<<(unsigned)((n_edges + per - 1) / per), CELL_WARPS * 32, 0, st>>>(F, B, n_edges); \
+  } break;
+    MF_CASE(2) MF_CASE(3) MF_CASE(4) MF_CASE(5) MF_CASE(6) MF_CASE(7) MF_CASE(8)
+#undef MF_CASE
+    default: break;
+  }
 }
 // Warps for one lane round of each edge's items, at most what the device
 // holds a few times over (the kernels pick the edges per warp).
@@ -1795,7 +1825,7 @@ extern "C" int mf_trace(mf_ctx *ctx, const mf_rbf *rbf, const mf_domain *dom,
   if ((opts->flags & MF_WANT_CELLS) && E > 0) {
     {
       MfProfScope ps(ctx, MF_PH_CELLS, st, 1, (int64_t)E);
-      k_cells_enum<<<(unsigned)((E * 32 + 255) / 256), 256, 0, st>>>(F, B, E);
+      mf_launch_cells_enum(F, B, E, st);
     }
     rc = mf_cuda_check(ctx, cudaGetLastError(), "cell kernels");
     if (rc) return rc;
