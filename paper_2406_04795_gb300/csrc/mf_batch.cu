@@ -16,8 +16,6 @@
 #include "mf_internal.cuh"
 #include "mf_ctx.h"
 
-bool mf_domain_table_host(MfFrame *F, std::vector<int2> &tab);
-
 namespace {
 
 struct Bump {
@@ -38,7 +36,8 @@ struct TraceLayout {
   uint64_t IC;
   size_t vtab_idx, vlist_off, vlist_n, vlist;  // root-screen lists (0 bytes: none)
   uint64_t ME, MV, MC, TE, TV, VL;
-  std::vector<int2> tab;
+  int64_t dom_rows;  // rows of the domain table (0: none)
+  const MfRbfStats *stats;  // of the prepared support vectors (device)
 };
 
 // One step of every active trace (captured into the graph's loop body).
@@ -116,7 +115,7 @@ int mf_layout_trace(mf_ctx *ctx, const mf_rbf *rbf, const mf_domain *dom, const 
   memset(S, 0, sizeof(*S));
   int rc = mf_build_frame(ctx, r.d, o->lambda, dom, &S->F);
   if (rc) return rc;
-  if (!mf_domain_table_host(&S->F, l->tab)) l->tab.clear();
+  l->dom_rows = mf_domain_rows(&S->F);
   const int d = r.d;
   l->ME = o->max_edges > 0 ? (uint64_t)o->max_edges : (1ull << 20);
   l->MV = o->max_vertices > 0 ? (uint64_t)o->max_vertices : l->ME;
@@ -126,7 +125,7 @@ int mf_layout_trace(mf_ctx *ctx, const mf_rbf *rbf, const mf_domain *dom, const 
   l->TE = mf_next_pow2(l->ME + l->ME / 3 + 1);
   l->TV = mf_next_pow2(l->MV + l->MV / 3 + 1);
   l->rbf = bump->take(mf_rbf_prep_bytes(d, r.n_sv));
-  l->dom = bump->take(l->tab.size() * sizeof(int2) + 8);
+  l->dom = bump->take((size_t)l->dom_rows * d * sizeof(int2) + 8);
   l->cnt = bump->take(sizeof(MfCounters));
   l->etab_key = bump->take(l->TE * 16);
   l->vtab_key = bump->take(l->TV * 16);
@@ -159,17 +158,16 @@ int mf_layout_trace(mf_ctx *ctx, const mf_rbf *rbf, const mf_domain *dom, const 
   return MF_OK;
 }
 
-// Prepares the support vectors, uploads the domain table, points the slot's
-// buffers into base + the layout's offsets, and clears counters and tables.
+// Enqueues the preparation of the support vectors and the domain table, points
+// the slot's buffers into base + the layout's offsets, and clears counters and
+// tables.  mf_finish_trace completes the slot from the support vectors'
+// statistics.
 int mf_setup_trace(mf_ctx *ctx, const mf_rbf *rbf, const mf_trace_opts *o, char *base,
                    TraceLayout *l, MfSlot *S, cudaStream_t st) {
-  int rc = mf_prepare_rbf_at(ctx, rbf, base + l->rbf, &S->R, st);
+  const int rc = mf_prepare_rbf_launch(ctx, rbf, base + l->rbf, &S->R, &l->stats, st);
   if (rc) return rc;
-  if (!l->tab.empty()) {
-    rc = mf_cuda_check(ctx, cudaMemcpyAsync(base + l->dom, l->tab.data(), l->tab.size() * sizeof(int2),
-                                            cudaMemcpyHostToDevice, st),
-                       "domain table");
-    if (rc) return rc;
+  if (l->dom_rows) {
+    mf_launch_domain_table(S->F, (int2 *)(base + l->dom), st);
     S->F.dom_tab = (const int2 *)(base + l->dom);
   }
   MfTraceBufs &B = S->B;
@@ -202,7 +200,6 @@ int mf_setup_trace(mf_ctx *ctx, const mf_rbf *rbf, const mf_trace_opts *o, char 
     B.vlist_n = (uint32_t *)(base + l->vlist_n);
     B.vlist = (int32_t *)(base + l->vlist);
     B.vlist_cap = l->VL;
-    B.list_r2 = mf_list_r2(S->F, S->R, o->precision != MF_FP64 && !(o->flags & MF_ROOTS_FP64_EXACT));
   } else {  // no per-vertex lists: the root screen scans the blocks
     B.vtab_idx = nullptr;
     B.vlist = nullptr;
@@ -219,6 +216,15 @@ int mf_setup_trace(mf_ctx *ctx, const mf_rbf *rbf, const mf_trace_opts *o, char 
   cudaMemsetAsync(B.cnt, 0, sizeof(MfCounters), st);
   cudaMemsetAsync(B.etab_key, 0xFF, l->TE * 16, st);
   cudaMemsetAsync(B.vtab_key, 0xFF, l->TV * 16, st);
+  return MF_OK;
+}
+
+int mf_finish_trace(mf_ctx *ctx, const mf_rbf *rbf, const mf_trace_opts *o, const MfRbfStats &h,
+                    MfSlot *S) {
+  const int rc = mf_prepare_rbf_finish(ctx, rbf, h, &S->R);
+  if (rc) return rc;
+  if (S->B.vlist)
+    S->B.list_r2 = mf_list_r2(S->F, S->R, o->precision != MF_FP64 && !(o->flags & MF_ROOTS_FP64_EXACT));
   return MF_OK;
 }
 
@@ -254,8 +260,21 @@ extern "C" int mf_trace_batch(mf_ctx *ctx, int32_t n, const mf_rbf *rbfs, const 
   cudaMemsetAsync(d_plan, 0, sizeof(MfBatchPlan), st);
   int rc;
   // --- per-trace preparation (support vectors, domain tables, tables)
+  // all enqueued, then one wait for their statistics
+  std::vector<MfRbfStats> hs0(n);
   for (int t = 0; t < n; t++) {
     rc = mf_setup_trace(ctx, &rbfs[t], &opts[t], arena, &L[t], &slots[t], st);
+    if (rc) {
+      cudaStreamSynchronize(st);  // nothing enqueued may outlive the call's inputs
+      return rc;
+    }
+  }
+  for (int t = 0; t < n; t++)
+    cudaMemcpyAsync(&hs0[t], L[t].stats, sizeof(MfRbfStats), cudaMemcpyDeviceToHost, st);
+  rc = mf_cuda_check(ctx, cudaStreamSynchronize(st), "batch preparation");
+  if (rc) return rc;
+  for (int t = 0; t < n; t++) {
+    rc = mf_finish_trace(ctx, &rbfs[t], &opts[t], hs0[t], &slots[t]);
     if (rc) return rc;
   }
   rc = mf_cuda_check(ctx, cudaMemcpyAsync(d_slots, slots.data(), sizeof(MfSlot) * n,
@@ -695,6 +714,12 @@ extern "C" int mf_server_step(mf_server *s, void *stream, int32_t *n_running, in
       break;  // wait for memory
     }
     rc = mf_setup_trace(ctx, &r.rbf, &r.opts, s->arena + s->data_off + off, &l, &S, st);
+    if (!rc) {
+      MfRbfStats h;
+      cudaMemcpyAsync(&h, l.stats, sizeof(h), cudaMemcpyDeviceToHost, st);
+      rc = mf_cuda_check(ctx, cudaStreamSynchronize(st), "server admission");
+      if (!rc) rc = mf_finish_trace(ctx, &r.rbf, &r.opts, h, &S);
+    }
     if (rc) {
       s->alloc.give(off, b.off);
       r.state = rc;

@@ -567,10 +567,21 @@ int mf_cuda_check(mf_ctx *ctx, cudaError_t e, const char *what);
 void *mf_ctx_buffer(mf_ctx *ctx, int slot, size_t bytes);
 int mf_ctx_sm_count(mf_ctx *ctx);
 
-// RBF preparation (mf_eval.cu): SoA FP32/FP64 copies in context buffers.
-int mf_prepare_rbf(mf_ctx *ctx, const mf_rbf *rbf, MfRbfDev *out, cudaStream_t st);
+// RBF preparation (mf_eval.cu): SoA FP32/FP64 copies in context buffers.  The
+// launch half enqueues it into `base` (mf_rbf_prep_bytes bytes of device
+// memory) and sets out's pointers; the finish half sets its scalars from the
+// statistics that the launch half left at *out_stats (device), once the caller
+// has read them back.
+struct MfRbfStats {
+  double sum_abs_alpha;
+  float max_abs_s;
+  int bad;  // NaN / Inf in the inputs
+};
+int mf_prepare_rbf(mf_ctx *ctx, const mf_rbf *rbf, MfRbfDev *out, cudaStream_t st);  // both, in MF_SLOT_RBF
 size_t mf_rbf_prep_bytes(int d, int64_t n);
-int mf_prepare_rbf_at(mf_ctx *ctx, const mf_rbf *rbf, char *base, MfRbfDev *out, cudaStream_t st);
+int mf_prepare_rbf_launch(mf_ctx *ctx, const mf_rbf *rbf, char *base, MfRbfDev *out,
+                          const MfRbfStats **out_stats, cudaStream_t st);
+int mf_prepare_rbf_finish(mf_ctx *ctx, const mf_rbf *rbf, const MfRbfStats &h, MfRbfDev *out);
 // Squared radius of a vertex's root-screen list: the screen radius around
 // any point of an edge leaving the vertex.  The longest edge is lam |L e(M)|
 // with |L e(M)|^2 = k (1 - 2ck + c^2 k d) for |M| = k; the margins cover the
@@ -588,6 +599,11 @@ static inline float mf_list_r2(const MfFrame &F, const MfRbfDev &R, bool fast = 
 }
 // Trace host helpers (mf_trace.cu).
 int mf_build_frame(mf_ctx *ctx, int d, double lam, const mf_domain *dom, MfFrame *F);
+// The exact domain table (MfFrame::dom_tab): its rows (0: none, the kernels
+// then test the domain in FP64), setting F->smin / F->sspan; and its contents,
+// written to dev ([rows][d]).
+int64_t mf_domain_rows(MfFrame *F);
+void mf_launch_domain_table(const MfFrame &F, int2 *dev, cudaStream_t st);
 void mf_exclusive_scan(const int64_t *in, int64_t *out, int64_t n, int64_t *scratch, cudaStream_t st);
 uint64_t mf_next_pow2(uint64_t x);
 void mf_launch_seeds(const MfFrame &F, const MfTraceBufs &B, const double *seeds, int64_t n,

@@ -32,12 +32,7 @@
 static __device__ __align__(256) unsigned char g_mf_noalloc_scratch[MF_NOALLOC_SCRATCH_BYTES];
 
 // Kernels of the traced path (defined in mf_trace.cu / mf_eval.cu).
-struct MfRbfStats {
-  double sum_abs_alpha;
-  float max_abs_s;
-  int bad;
-};
-__global__ void k_prepare_rbf(int d, int n, const double *sv, const double *alpha, const int32_t *perm,
+__global__ void k_prepare_rbf(int d, int n, const double *sv, const double *alpha, const int32_t *place,
                               float *sv32, float *svlo32, double *sv64, double *alpha64,
                               float *alpha32, float *strong32, double *exp_tab, double *sv64r,
                               float *svhl, float *sv3, float *alpha_lo32, float2 *exp_df,

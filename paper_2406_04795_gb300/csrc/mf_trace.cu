@@ -1369,16 +1369,25 @@ static int build_frame(mf_ctx *ctx, int d, double lam, const mf_domain *dom, MfF
 // order (this translation unit's host code is compiled without contraction).
 // Fills `tab` and sets F->smin / F->sspan; false if the table would be too
 // large (the kernels then test the domain in FP64).
-bool mf_domain_table_host(MfFrame *F, std::vector<int2> &tab) {
-  const int d = F->d;
+int64_t mf_domain_rows(MfFrame *F) {
   long long smin = 0, smax = 0;
-  for (int i = 0; i < d; i++) {
+  for (int i = 0; i < F->d; i++) {
     smin += F->ymin[i];
     smax += (long long)F->ymin[i] + F->range[i] - 1;
   }
   const long long span = smax - smin + 1;
   F->dom_tab = nullptr;
-  if (span <= 0 || span > (1ll << 22)) return false;
+  if (span <= 0 || span > (1ll << 22)) return 0;
+  F->smin = (int32_t)smin;
+  F->sspan = (int32_t)span;
+  return span;
+}
+
+bool mf_domain_table_host(MfFrame *F, std::vector<int2> &tab) {
+  const int d = F->d;
+  const int64_t span = mf_domain_rows(F);
+  if (!span) return false;
+  const long long smin = F->smin, smax = smin + span - 1;
   tab.assign((size_t)span * d, int2());
   for (long long s = smin; s <= smax; s++) {
     const double cs = F->c * (double)s;
@@ -1410,24 +1419,60 @@ bool mf_domain_table_host(MfFrame *F, std::vector<int2> &tab) {
       tab[(size_t)(s - smin) * d + i] = v;
     }
   }
-  F->smin = (int32_t)smin;
-  F->sspan = (int32_t)span;
   return true;
 }
 
+// The same table on the device, one (s, axis) per thread, with the kernels' own
+// operations.
+__global__ void __launch_bounds__(128) k_domain_table(MfFrame F, int2 *tab) {
+  const int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  const int d = F.d;
+  if (q >= (int64_t)F.sspan * d) return;
+  const int i = (int)(q % d);
+  const long long s = F.smin + q / d;
+  double o = 0.0, blo = 0.0, bhi = 0.0;
+  long long y0 = 0, y1 = 0;
+#pragma unroll
+  for (int k = 0; k < MF_MAXD; k++)
+    if (k == i) {
+      o = F.o[k];
+      blo = F.lo[k];
+      bhi = F.hi[k];
+      y0 = F.ymin[k];
+      y1 = y0 + F.range[k] - 1;
+    }
+  const double cs = __dmul_rn(F.c, (double)s);
+  auto x_of = [&](long long y) {
+    return __dadd_rn(__dmul_rn(F.lam, __dsub_rn((double)y, cs)), o);
+  };
+  long long a = y0, b = y1 + 1;  // first y with x >= lo
+  while (a < b) {
+    const long long m = a + (b - a) / 2;
+    if (x_of(m) >= blo) b = m; else a = m + 1;
+  }
+  const long long first = a;
+  a = y0 - 1;
+  b = y1;  // last y with x <= hi
+  while (a < b) {
+    const long long m = a + (b - a + 1) / 2;
+    if (x_of(m) <= bhi) a = m; else b = m - 1;
+  }
+  tab[q] = first <= a ? make_int2((int)first, (int)a) : make_int2(1 << 30, -(1 << 30));
+}
+
+void mf_launch_domain_table(const MfFrame &F, int2 *dev, cudaStream_t st) {
+  const int64_t n = (int64_t)F.sspan * F.d;
+  k_domain_table<<<(unsigned)((n + 127) / 128), 128, 0, st>>>(F, dev);
+}
+
 static int build_domain_table(mf_ctx *ctx, MfFrame *F, cudaStream_t st) {
-  std::vector<int2> tab;
-  if (!mf_domain_table_host(F, tab)) return MF_OK;  // FP64 test instead
-  int2 *dev = (int2 *)mf_ctx_buffer(ctx, MF_SLOT_DOMTAB, tab.size() * sizeof(int2));
+  const int64_t rows = mf_domain_rows(F);
+  if (!rows) return MF_OK;  // FP64 test instead
+  int2 *dev = (int2 *)mf_ctx_buffer(ctx, MF_SLOT_DOMTAB, (size_t)rows * F->d * sizeof(int2));
   if (!dev) return MF_ERR_OOM;
-  int rc = mf_cuda_check(ctx, cudaMemcpyAsync(dev, tab.data(), tab.size() * sizeof(int2),
-                                              cudaMemcpyHostToDevice, st),
-                         "domain table");
-  if (rc) return rc;
-  rc = mf_cuda_check(ctx, cudaStreamSynchronize(st), "domain table");
-  if (rc) return rc;
+  mf_launch_domain_table(*F, dev, st);
   F->dom_tab = dev;
-  return MF_OK;
+  return mf_cuda_check(ctx, cudaGetLastError(), "domain table");
 }
 
 extern "C" int mf_domain_table(int32_t d, double lambda, const mf_domain *dom, int32_t *smin,
