@@ -352,8 +352,14 @@ __device__ __forceinline__ void cert_sincos(double x, const double2 *tab, double
 }
 
 // FP32 record of a point for the whole-cell certificate: coordinates,
-// margin, deciding element (int bits), padded to whole 16-byte units.
+// margin, and one word with the deciding element (low 16 bits, signed) and
+// the verdict (bit 16), padded to whole 16-byte units.  The verdict rides
+// along because the cell pass is bound by its gathers: a separate byte per
+// point costs each row entry a second 32-byte sector.
 __host__ __device__ __forceinline__ int cert_rec_stride(int d) { return (d + 2 + 3) & ~3; }
+__device__ __forceinline__ float cert_rec_word(int element, bool verdict) {
+  return __int_as_float((element & 0xffff) | (verdict ? 0x10000 : 0));
+}
 
 // The link loops stay rolled: unrolling them per link count inlines the
 // distance routines once per link and pass, which overflows the instruction
@@ -755,7 +761,7 @@ __device__ __noinline__ bool cert_point(const CertShared &sh, int NL, const doub
     const int rs = cert_rec_stride(d);
     for (int k = 0; k < d; k++) rec32[p * rs + k] = (float)pts[p * d + k];
     rec32[p * rs + d] = (float)best;
-    rec32[p * rs + d + 1] = __int_as_float(be);
+    rec32[p * rs + d + 1] = cert_rec_word(be, best >= 0.0);
   }
   return false;
 }
@@ -845,7 +851,7 @@ __device__ __forceinline__ void cert_simple_eval(const CertShared &sh, int NL, c
     const int rs = cert_rec_stride(d);
     for (int q = 0; q < d; q++) rec32[p * rs + q] = (float)pts[p * d + q];
     rec32[p * rs + d] = (float)best;
-    rec32[p * rs + d + 1] = __int_as_float(be);
+    rec32[p * rs + d + 1] = cert_rec_word(be, best >= 0.0);
   }
 }
 
@@ -1055,6 +1061,20 @@ __device__ __forceinline__ void cert_rec_extend(const float4 (&v)[NV4], int d, f
   }
 }
 
+// The verdict of a point's record.
+template <int NV4>
+__device__ __forceinline__ uint32_t cert_rec_verdict(const float4 (&v)[NV4], int d) {
+  uint32_t w = 0;
+#pragma unroll
+  for (int q = 0; q < NV4; q++) {
+    const float vv[4] = {v[q].x, v[q].y, v[q].z, v[q].w};
+#pragma unroll
+    for (int h = 0; h < 4; h++)
+      if (4 * q + h == d + 1) w = (uint32_t)__float_as_int(vv[h]);
+  }
+  return (w >> 16) & 1u;
+}
+
 // One point's FP32 slack test (see above): sets yes when it certifies the
 // cell, undecided when its error bound straddles the decision.
 template <int NV4>
@@ -1069,7 +1089,7 @@ __device__ __forceinline__ void cert_rec_test(const float4 (&v)[NV4], int d, int
 #pragma unroll
     for (int h = 0; h < 4; h++) {
       if (4 * q + h == d) m = vv[h];
-      if (4 * q + h == d + 1) e = __float_as_int(vv[h]);
+      if (4 * q + h == d + 1) e = (int16_t)(__float_as_int(vv[h]) & 0xffff);
     }
   }
   if (e < 0 || e >= NE) return;
@@ -1100,8 +1120,7 @@ template <int NV4>
 __global__ void __launch_bounds__(256, 3) k_certify_cells_whole32(
     const int64_t *off, const int64_t *idx, int64_t n_cells, const float *rec32, const double *pts,
     int d, const double *margin, const int16_t *element, const float *L32, const double *L, int NE,
-    int64_t n_points, uint8_t *whole, unsigned *bad, const uint8_t *verdict,
-    uint8_t *cell_verdict) {
+    int64_t n_points, uint8_t *whole, unsigned *bad, uint8_t *cell_verdict) {
   const int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (c >= n_cells) return;
   const int64_t j0 = off[c], j1 = off[c + 1];
@@ -1126,11 +1145,11 @@ __global__ void __launch_bounds__(256, 3) k_certify_cells_whole32(
       atomicOr(bad, 1u);
       all = 0;
     }
-    if (cell_verdict && in) all &= verdict[i];
 #pragma unroll
     for (int q = 0; q < NV4; q++)
       cache[r][q] = in ? __ldg(R4 + i * NV4 + q) : make_float4(0.f, 0.f, 0.f, 0.f);
     if (in) {
+      all &= cert_rec_verdict<NV4>(cache[r], d);
       cert_rec_extend<NV4>(cache[r], d, lo, hi, P);
       valid |= 1u << r;
     }
@@ -1142,10 +1161,10 @@ __global__ void __launch_bounds__(256, 3) k_certify_cells_whole32(
       all = 0;
       continue;
     }
-    if (cell_verdict) all &= verdict[i];
     float4 v[NV4];
 #pragma unroll
     for (int q = 0; q < NV4; q++) v[q] = __ldg(R4 + i * NV4 + q);
+    all &= cert_rec_verdict<NV4>(v, d);
     cert_rec_extend<NV4>(v, d, lo, hi, P);
   }
   if (cell_verdict) cell_verdict[c] = (uint8_t)all;
@@ -1326,18 +1345,15 @@ extern "C" int mf_certify_ex(mf_ctx *ctx, const mf_robot *robot, const mf_scene 
     if (fast && nv4 == 1)
       k_certify_cells_whole32<1><<<gc, 256, 0, st>>>(cell_off, cell_idx, n_cells, rec32, points, d,
                                                       out->margin, elem, dL32, dL, NE, n_points,
-                                                      out->cell_whole, bad, out->point_verdict,
-                                                      out->cell_verdict);
+                                                      out->cell_whole, bad, out->cell_verdict);
     else if (fast && nv4 == 2)
       k_certify_cells_whole32<2><<<gc, 256, 0, st>>>(cell_off, cell_idx, n_cells, rec32, points, d,
                                                       out->margin, elem, dL32, dL, NE, n_points,
-                                                      out->cell_whole, bad, out->point_verdict,
-                                                      out->cell_verdict);
+                                                      out->cell_whole, bad, out->cell_verdict);
     else if (fast)
       k_certify_cells_whole32<3><<<gc, 256, 0, st>>>(cell_off, cell_idx, n_cells, rec32, points, d,
                                                       out->margin, elem, dL32, dL, NE, n_points,
-                                                      out->cell_whole, bad, out->point_verdict,
-                                                      out->cell_verdict);
+                                                      out->cell_whole, bad, out->cell_verdict);
     else
       k_certify_cells_whole<<<(unsigned)((n_cells + 255) / 256), 256, 0, st>>>(
           cell_off, cell_idx, n_cells, points, d, out->margin, elem, dL, NE, n_points,
