@@ -242,14 +242,11 @@ __device__ __forceinline__ bool point_deep_inside32(const CertObsT<float> &o, co
 // distance is then exactly 0); tested only when the bound is 0.  Its
 // candidates: the middle of the segment's slab-clipped interval in the
 // shrunk box (boxes), the final t and the projection of the centre
-// (cylinders), the closest point (spheres).  *ubd: an upper bound on the
-// same distance, from the squared distance at the final t plus eta (the
-// distance from one point of the segment).  Not inlined: the kernel calls
-// it from three places, and one copy keeps the code in the instruction
-// cache.
+// (cylinders), the closest point (spheres).  Not inlined: the kernel calls
+// it from two places, and one copy keeps the code in the instruction cache.
 __device__ __noinline__ float seg_obstacle_lb32(const CertObsT<float> &o, const float *pa,
                                                 const float *pb, float eta, float dlt, float *tmin,
-                                                bool *deep, float *ubd) {
+                                                bool *deep) {
   const float wa[3] = {pa[0] - o.t[0], pa[1] - o.t[1], pa[2] - o.t[2]};
   const float wb[3] = {pb[0] - o.t[0], pb[1] - o.t[1], pb[2] - o.t[2]};
   float a[3], dl[3];
@@ -272,7 +269,6 @@ __device__ __noinline__ float seg_obstacle_lb32(const CertObsT<float> &o, const 
       if (it < 3 && H > 0.f) t = fminf(fmaxf(t - G / H, 0.f), 1.f);
     }
     *tmin = t;
-    *ubd = sqrtf(F + eta) * 1.000001f;
     const float lbF = F - 2.f * fabsf(G) * (G > 0.f ? t : 1.f - t) - eta;
     *deep = !(lbF > 0.f) &&
             (point_deep_inside32(o, a, dl, tc, dlt) || point_deep_inside32(o, a, dl, t, dlt));
@@ -283,7 +279,6 @@ __device__ __noinline__ float seg_obstacle_lb32(const CertObsT<float> &o, const 
     const float c0 = fmaf(t, dl[0], a[0]), c1 = fmaf(t, dl[1], a[1]), c2 = fmaf(t, dl[2], a[2]);
     const float c2s = c0 * c0 + c1 * c1 + c2 * c2;
     const float lb = fmaxf(sqrtf(c2s) - o.h[0], 0.f);
-    *ubd = fmaxf(sqrtf(c2s + eta) * 1.000001f - o.h[0], 0.f) * 1.000001f;
     *deep = !(lb > 0.f) && point_deep_inside32(o, a, dl, t, dlt);
     return lb;
   }
@@ -306,7 +301,6 @@ __device__ __noinline__ float seg_obstacle_lb32(const CertObsT<float> &o, const 
     if (it < 3 && H > 0.f) t = fminf(fmaxf(t - G / H, 0.f), 1.f);
   }
   *tmin = t;
-  *ubd = sqrtf(F + eta) * 1.000001f;
   const float lbF = F - 2.f * fabsf(G) * (G > 0.f ? t : 1.f - t) - eta;
   *deep = false;
   if (!(lbF > 0.f)) {
@@ -391,6 +385,7 @@ __device__ __forceinline__ void cert_dh_step(double *T, double ct, double st, do
 struct CertShared {
   CertObs so[CERT_MAX_OBS];
   CertObsT<float> sof[CERT_MAX_OBS];
+  float4 srt[CERT_MAX_OBS];  // R^T t and max_c (|t_c| + h_c) (the first pass)
   double sdh[MF_MAXD * 4], srad[MF_MAXD], ssa[MF_MAXD], sca[MF_MAXD];
   float sdh32[MF_MAXD * 4], srad32[MF_MAXD], ssa32[MF_MAXD], sca32[MF_MAXD];
   double2 ssc[128];
@@ -419,6 +414,12 @@ __device__ __forceinline__ void cert_load_shared(CertShared &sh, int NL, const d
     }
     sh.so[i] = o;
     sh.sof[i] = of;
+    float4 rt;
+    rt.x = of.R[0] * of.t[0] + of.R[3] * of.t[1] + of.R[6] * of.t[2];
+    rt.y = of.R[1] * of.t[0] + of.R[4] * of.t[1] + of.R[7] * of.t[2];
+    rt.z = of.R[2] * of.t[0] + of.R[5] * of.t[1] + of.R[8] * of.t[2];
+    rt.w = fmaxf(fmaxf(fabsf(of.t[0]) + of.h[0], fabsf(of.t[1]) + of.h[1]), fabsf(of.t[2]) + of.h[2]);
+    sh.srt[i] = rt;
   }
   for (int i = threadIdx.x; i < NL * 4; i += blockDim.x) {
     sh.sdh[i] = dh[i];
@@ -449,17 +450,275 @@ struct CertRec {
   int32_t loc;  // the point's thread in the block
 };
 
-// Point p: margin = max over (element, obstacle) of radius - distance, its
-// verdict, deciding element and FP32 record.  FAST: after the FP32 bounds,
-// a point that at most two exact pair evaluations settle returns true with
-// its record in *simple for cert_simple_eval; every other point is appended
-// to queue and left to a FAST = false pass.
-template <bool FAST>
-__device__ __noinline__ bool cert_point(const CertShared &sh, int NL, const double *radius, int NS,
+__device__ __forceinline__ float cert_sqrt(float x) {  // relative error below 2^-22
+  float y;
+  asm("sqrt.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+
+// The first pass's running state: the two pairs with the largest bounds ub on
+// their margin, the third-largest bound, and the elements inside an obstacle.
+struct CertTop {
+  float ub1, ub2, ub3, lb1, lb2, t1, t2;
+  int e1, k1, e2, k2;
+  uint64_t deep_lo, deep_hi;
+};
+
+__device__ __forceinline__ void cert_top_add(CertTop &c, int e, int k, float ub, float lb, float t,
+                                             bool deep) {
+  if (deep) {
+    if (e < 64) c.deep_lo |= 1ull << e;
+    else c.deep_hi |= 1ull << (e - 64);
+    return;
+  }
+  if (ub > c.ub1) {
+    c.ub3 = c.ub2;
+    c.e2 = c.e1;
+    c.k2 = c.k1;
+    c.t2 = c.t1;
+    c.lb2 = c.lb1;
+    c.ub2 = c.ub1;
+    c.ub1 = ub;
+    c.e1 = e;
+    c.k1 = k;
+    c.t1 = t;
+    c.lb1 = lb;
+  } else if (ub > c.ub2) {
+    c.ub3 = c.ub2;
+    c.ub2 = ub;
+    c.e2 = e;
+    c.k2 = k;
+    c.t2 = t;
+    c.lb2 = lb;
+  } else if (ub > c.ub3) {
+    c.ub3 = ub;
+  }
+}
+
+// The bounds of element e (the segment p .. p + dw, or the point p when POINT;
+// es: its largest coordinate) against every obstacle.  Per pair, in FP32 from
+// the FP32 chain, a lower and an upper bound on the distance (a point's and a
+// sphere's are the distance itself, the others' by seg_obstacle_lb32's
+// method); widened by a slack of 1e-4 (1 + the largest coordinate), far above
+// the FP32 rounding of the chain and of these operations (about 1e-5 of that
+// scale), they bound the true distance, so that
+// radius - them bounds the pair's margin from above (ub) and below (lb).  The
+// Newton steps on F' only choose t; both bounds hold at any t.  A pair whose
+// segment provably has a point inside the obstacle shrunk by the slack is at
+// distance exactly 0 (deep).  The element is in registers and the obstacles'
+// types are uniform over the warp; a point (a robot sphere) needs no search
+// for t, about a fifth of a segment's operations.
+template <bool POINT>
+__device__ __forceinline__ void cert_bounds(const CertShared &sh, int nobs, int e, float rad,
+                                            const float *p, const float *dw, float es, CertTop &c) {
+  for (int k = 0; k < nobs; k++) {
+    const CertObsT<float> &o = sh.sof[k];
+    const float4 rt = sh.srt[k];
+    const float scale = fmaxf(fmaxf(es, rt.w), 1.f);
+    const float eta = 4e-5f * (1.f + scale) * (1.f + scale), sl = 1e-4f * (1.f + scale);
+    // the element in the obstacle's frame
+    float a[3], dl[3];
+#pragma unroll
+    for (int i = 0; i < 3; i++) {
+      const float r = i == 0 ? rt.x : (i == 1 ? rt.y : rt.z);
+      a[i] = fmaf(o.R[i], p[0], fmaf(o.R[3 + i], p[1], fmaf(o.R[6 + i], p[2], -r)));
+      if (!POINT) dl[i] = fmaf(o.R[i], dw[0], fmaf(o.R[3 + i], dw[1], o.R[6 + i] * dw[2]));
+    }
+    const int type = o.type;
+    float t = 0.f, lbd, ubd;
+    bool deep = false;
+    if (POINT) {
+      float F;
+      if (type == MF_BOX) {
+        const float q0 = fabsf(a[0]) - o.h[0], q1 = fabsf(a[1]) - o.h[1], q2 = fabsf(a[2]) - o.h[2];
+        const float x = fmaxf(q0, 0.f), y = fmaxf(q1, 0.f), z = fmaxf(q2, 0.f);
+        F = fmaf(x, x, fmaf(y, y, z * z));
+        deep = fmaxf(fmaxf(q0, q1), q2) <= -sl;
+      } else if (type == MF_CYLINDER) {
+        const float rr = fmaf(a[0], a[0], a[1] * a[1]);
+        const float qr = cert_sqrt(rr) - o.h[0], qz = fabsf(a[2]) - o.h[1];
+        const float x = fmaxf(qr, 0.f), z = fmaxf(qz, 0.f);
+        F = fmaf(x, x, z * z);
+        deep = fmaxf(qr, qz) <= -sl;
+      } else {
+        const float q = cert_sqrt(fmaf(a[0], a[0], fmaf(a[1], a[1], a[2] * a[2]))) - o.h[0];
+        const float x = fmaxf(q, 0.f);
+        F = x * x;
+        deep = q <= -sl;
+      }
+      lbd = cert_sqrt(F);
+      ubd = lbd * 1.000001f;
+    } else {
+      const float dd = fmaf(dl[0], dl[0], fmaf(dl[1], dl[1], dl[2] * dl[2]));
+      const float ad = fmaf(a[0], dl[0], fmaf(a[1], dl[1], a[2] * dl[2]));
+      if (dd > 0.f) t = fminf(fmaxf(__fdividef(-ad, dd), 0.f), 1.f);
+      const float tc = t;
+      float F = 0.f, G = 0.f;  // F(t) and F'(t) / 2
+      if (type == MF_BOX) {
+#pragma unroll
+        for (int it = 0; it <= 3; it++) {
+          float H = 0.f;  // F''(t) / 2
+          F = 0.f;
+          G = 0.f;
+#pragma unroll
+          for (int i = 0; i < 3; i++) {
+            const float x = fmaf(t, dl[i], a[i]);
+            const float q = fmaxf(fabsf(x) - o.h[i], 0.f);
+            F = fmaf(q, q, F);
+            G = fmaf(copysignf(q, x), dl[i], G);
+            H = fmaf(q > 0.f ? dl[i] : 0.f, dl[i], H);
+          }
+          if (it < 3 && H > 0.f) t = fminf(fmaxf(t - __fdividef(G, H), 0.f), 1.f);
+        }
+      } else if (type == MF_CYLINDER) {
+#pragma unroll 1
+        for (int it = 0; it <= 3; it++) {
+          float H;
+          cyl_fgh<float>(a, dl, o.h[0], o.h[1], t, F, G, H);
+          if (it < 3 && H > 0.f) t = fminf(fmaxf(t - __fdividef(G, H), 0.f), 1.f);
+        }
+      } else {
+        const float x = fmaf(t, dl[0], a[0]), y = fmaf(t, dl[1], a[1]), z = fmaf(t, dl[2], a[2]);
+        const float q = fmaxf(cert_sqrt(fmaf(x, x, fmaf(y, y, z * z))) - o.h[0], 0.f);
+        F = q * q;
+      }
+      // the distance at t bounds the minimum from above; from below, convexity
+      // does, with eta for the cancellation in it (a sphere's t is exact)
+      ubd = cert_sqrt(F) * 1.000001f;
+      const float lbF =
+          type == MF_SPHERE ? F : F - 2.f * fabsf(G) * (G > 0.f ? t : 1.f - t) - eta;
+      lbd = lbF > 0.f ? cert_sqrt(lbF) : 0.f;
+      if (!(lbF > 0.f)) {
+        float td = t;
+        if (type == MF_BOX) {  // the middle of the segment's part in the shrunk box
+          float t0 = 0.f, t1 = 1.f;
+#pragma unroll
+          for (int i = 0; i < 3; i++) {
+            const float hs = o.h[i] - sl;
+            if (dl[i] != 0.f) {
+              const float inv = __fdividef(1.f, dl[i]);
+              const float ta = (-hs - a[i]) * inv, tb = (hs - a[i]) * inv;
+              t0 = fmaxf(t0, fminf(ta, tb));
+              t1 = fminf(t1, fmaxf(ta, tb));
+            }
+          }
+          td = t0 <= t1 ? 0.5f * (t0 + t1) : t;
+        }
+        deep = point_deep_inside32(o, a, dl, td, sl) ||
+               (type == MF_CYLINDER && point_deep_inside32(o, a, dl, tc, sl));
+      }
+    }
+    cert_top_add(c, e, k, rad - (lbd - sl), rad - (ubd + sl), t, deep);
+  }
+}
+
+// First pass for point p: the FP32 chain, each link's elements bounded against
+// every obstacle as the chain reaches it.  Bound by instruction issue over
+// elements x obstacles.  It used to share the full search's code, which keeps
+// the chain in indexed (local) arrays and treats a sphere as a zero-length
+// segment; with the element in registers, points without a search for t and
+// bounds tight enough to queue fewer points, certifying 500,000 points (6
+// capsules and 18 robot spheres, 18 obstacles) takes 2.5 ms instead of 4.7,
+// and this pass over a d = 5 proof at lambda = 0.08 6.4 ms instead of 8.2.
+// A point that at most two exact pair
+// evaluations settle returns true with its record in *simple for
+// cert_simple_eval; every other point is appended to queue.
+__device__ __forceinline__ bool cert_first(const CertShared &sh, int NL, const double *radius,
+                                           int NS, int nobs, const double *pts, int64_t p, int d,
+                                           CertRec *simple, uint32_t *queue,
+                                           unsigned long long *nq) {
+  const int NC = radius ? NL : 0;
+  CertTop c;
+  c.ub1 = c.ub2 = c.ub3 = c.lb1 = c.lb2 = -INFINITY;
+  c.t1 = c.t2 = 0.f;
+  c.e1 = c.k1 = c.e2 = c.k2 = -1;
+  c.deep_lo = c.deep_hi = 0;
+  float T[12] = {1, 0, 0, 0, 0, 1, 0, 0, 0, 0, 1, 0};
+#pragma unroll 1
+  for (int i = 0; i < NL; i++) {
+    const float p0[3] = {T[3], T[7], T[11]};
+    const float th = (float)pts[p * d + i] + sh.sdh32[4 * i];
+    const float dd = sh.sdh32[4 * i + 1], aa = sh.sdh32[4 * i + 2];
+    float st, ct;
+    sincosf(th, &st, &ct);
+    const float sa = sh.ssa32[i], ca = sh.sca32[i];
+#pragma unroll
+    for (int r = 0; r < 3; r++) {  // T <- T A (cert_dh_step's order)
+      const float t0 = T[4 * r], t1 = T[4 * r + 1], t2 = T[4 * r + 2], t3 = T[4 * r + 3];
+      const float c0 = fmaf(t0, ct, t1 * st);
+      const float v = fmaf(t1, ct, -(t0 * st));
+      T[4 * r] = c0;
+      T[4 * r + 1] = fmaf(v, ca, t2 * sa);
+      T[4 * r + 2] = fmaf(t2, ca, -(v * sa));
+      T[4 * r + 3] = fmaf(aa, c0, fmaf(dd, t2, t3));
+    }
+    if (NC) {
+      const float dw[3] = {T[3] - p0[0], T[7] - p0[1], T[11] - p0[2]};
+      float es = 0.f;
+#pragma unroll
+      for (int q = 0; q < 3; q++) es = fmaxf(es, fmaxf(fabsf(p0[q]), fabsf(T[4 * q + 3])));
+      cert_bounds<false>(sh, nobs, i, sh.srad32[i], p0, dw, es, c);
+    }
+#pragma unroll 1
+    for (int s = 0; s < NS; s++) {
+      if (sh.ssl[s] != i) continue;
+      float x[3], es = 0.f;
+#pragma unroll
+      for (int r = 0; r < 3; r++) {
+        x[r] = fmaf(T[4 * r], sh.ssc32[3 * s],
+                    fmaf(T[4 * r + 1], sh.ssc32[3 * s + 1],
+                         fmaf(T[4 * r + 2], sh.ssc32[3 * s + 2], T[4 * r + 3])));
+        es = fmaxf(es, fabsf(x[r]));
+      }
+      cert_bounds<true>(sh, nobs, NC + s, sh.ssr32[s], x, x, es, c);
+    }
+  }
+  // L = max(margins of the elements inside an obstacle, lb1, lb2) is a lower
+  // bound on the point's margin.  When the third-largest bound lies below L by
+  // more than the gap, only the two pairs with the largest bounds (those of
+  // them whose bound reaches L - gap) can hold the maximum or tie with it,
+  // besides the elements inside an obstacle (margin = radius): their exact
+  // evaluations settle the point (cert_simple_eval).  The gap covers the FP32
+  // rounding of the bounds, the FP64 distance's 2e-12 and the 1e-9 tie.
+  double best_in = -INFINITY;
+  for (uint64_t w = c.deep_lo; w; w &= w - 1) {
+    const int e = __ffsll((long long)w) - 1;
+    best_in = fmax(best_in, e < NC ? sh.srad[e] : sh.ssr64[e - NC]);
+  }
+  for (uint64_t w = c.deep_hi; w; w &= w - 1)
+    best_in = fmax(best_in, sh.ssr64[64 + __ffsll((long long)w) - 1 - NC]);
+  const double L = fmax(best_in, (double)fmaxf(c.lb1, c.lb2));
+  const double thr = L - 4e-6 * (1.0 + fabs(L));
+  if (c.e1 < 0 || (double)c.ub3 < thr) {
+    CertRec r;
+    r.deep_lo = c.deep_lo;
+    r.deep_hi = c.deep_hi;
+    r.e1 = r.k1 = r.e2 = r.k2 = 0xff;
+    r.t1 = c.t1;
+    r.t2 = c.t2;
+    r.loc = 0;
+    if (c.e1 >= 0 && (double)c.ub1 >= thr) {
+      r.e1 = (uint8_t)c.e1;
+      r.k1 = (uint8_t)c.k1;
+    }
+    if (c.e2 >= 0 && (double)c.ub2 >= thr) {
+      r.e2 = (uint8_t)c.e2;
+      r.k2 = (uint8_t)c.k2;
+    }
+    *simple = r;
+    return true;
+  }
+  const unsigned long long q = atomicAdd(nq, 1ull);
+  queue[q] = (uint32_t)p;
+  return false;
+}
+
+// Point p in full: margin = max over (element, obstacle) of radius - distance,
+// its verdict, deciding element and FP32 record.
+__device__ __noinline__ void cert_point(const CertShared &sh, int NL, const double *radius, int NS,
                                         int nobs, const double *pts, int64_t p, int d,
                                         uint8_t *verdict, double *margin, int16_t *element,
-                                        float *rec32, CertRec *simple, uint32_t *queue,
-                                        unsigned long long *nq) {
+                                        float *rec32) {
   const CertObs *so = sh.so;
   const CertObsT<float> *sof = sh.sof;
   const double *sdh = sh.sdh, *srad = sh.srad, *ssa = sh.ssa, *sca = sh.sca;
@@ -587,7 +846,7 @@ __device__ __noinline__ bool cert_point(const CertShared &sh, int NL, const doub
   // inside it shrunk by the same 1e-4 (1 + scale), which covers the FP32
   // chain's error in every coordinate) is at distance exactly 0: its margin
   // is the element's radius, with no FP64 work (*deep).
-  auto upper = [&](int e, int k, float *tmin, bool *deep, float *lower = nullptr) -> float {
+  auto upper = [&](int e, int k, float *tmin, bool *deep) -> float {
     float a[3], b[3];
     const float rad = elem32(e, a, b);
     float scale = 1.f;
@@ -598,9 +857,7 @@ __device__ __noinline__ bool cert_point(const CertShared &sh, int NL, const doub
     // squared distance stays far below 4e-5 (1 + scale)^2
     const float eta = 4e-5f * (1.f + scale) * (1.f + scale);
     const float sl = 1e-4f * (1.f + scale);
-    float ubd;
-    const float lbd = seg_obstacle_lb32(sof[k], a, b, eta, sl, tmin, deep, &ubd);
-    if (lower) *lower = rad - (ubd + sl);
+    const float lbd = seg_obstacle_lb32(sof[k], a, b, eta, sl, tmin, deep);
     return rad - (lbd - sl);
   };
   auto rad64 = [&](int e) -> double { return e < NC ? srad[e] : ssr64[e - NC]; };
@@ -608,10 +865,7 @@ __device__ __noinline__ bool cert_point(const CertShared &sh, int NL, const doub
   // first by element ein); the other pairs give bounds ub (largest ub1 at
   // (bi, bk), second ub2; per element the largest, ube, and whether it has
   // a deep pair)
-  float ub1 = -INFINITY, ub2 = -INFINITY, tb = 0.f, lb1 = -INFINITY;
-  // FAST: the pair with the second-largest bound (ub2) and the third bound
-  float ub3 = -INFINITY, tb2 = 0.f, lb2 = -INFINITY;
-  int bi2 = -1, bk2 = -1;
+  float ub1 = -INFINITY, ub2 = -INFINITY, tb = 0.f;
   int bi = -1, bk = -1, ein = -1;
   double best_in = -INFINITY;
   float ube[CERT_MAX_ELEM];
@@ -622,9 +876,9 @@ __device__ __noinline__ bool cert_point(const CertShared &sh, int NL, const doub
   for (int e = 0; e < NE; e++) {
     float um = -INFINITY;
     for (int k = 0; k < nobs; k++) {
-      float tk, lbk;
+      float tk;
       bool deep;
-      const float ub = upper(e, k, &tk, &deep, &lbk);
+      const float ub = upper(e, k, &tk, &deep);
       if (deep) {
         if (e < 64) deep_lo |= 1ull << e;
         else deep_hi |= 1ull << (e - 64);
@@ -636,68 +890,16 @@ __device__ __noinline__ bool cert_point(const CertShared &sh, int NL, const doub
       }
       um = fmaxf(um, ub);
       if (ub > ub1) {
-        if (FAST) {
-          ub3 = ub2;
-          bi2 = bi;
-          bk2 = bk;
-          tb2 = tb;
-          lb2 = lb1;
-        }
         ub2 = ub1;
         ub1 = ub;
         bi = e;
         bk = k;
         tb = tk;
-        lb1 = lbk;
       } else if (ub > ub2) {
-        if (FAST) {
-          ub3 = ub2;
-          bi2 = e;
-          bk2 = k;
-          tb2 = tk;
-          lb2 = lbk;
-        }
         ub2 = ub;
-      } else if (FAST && ub > ub3) {
-        ub3 = ub;
       }
     }
     ube[e] = um;
-  }
-  if (FAST) {
-    // L = max(best_in, lb1, lb2) is a lower bound on the point's margin
-    // (lb: the pair's margin bound from the upper distance bound of the FP32
-    // chain plus the same slack).  When the third-largest bound lies below
-    // L by more than the gap, only the two pairs with the largest bounds
-    // (those of them whose bound reaches L - gap) can hold the maximum or tie
-    // with it, besides the elements inside an obstacle (margin = radius):
-    // their exact evaluations settle the point (cert_simple_eval).  The gap
-    // covers the FP32 rounding of the bounds, the FP64 distance's 2e-12 and
-    // the 1e-9 tie.
-    const double L = fmax(best_in, (double)fmaxf(lb1, lb2));
-    const double thr = L - 4e-6 * (1.0 + fabs(L));
-    if (bi < 0 || (double)ub3 < thr) {
-      CertRec r;
-      r.deep_lo = deep_lo;
-      r.deep_hi = deep_hi;
-      r.e1 = r.k1 = r.e2 = r.k2 = 0xff;
-      r.t1 = tb;
-      r.t2 = tb2;
-      r.loc = 0;
-      if (bi >= 0 && (double)ub1 >= thr) {
-        r.e1 = (uint8_t)bi;
-        r.k1 = (uint8_t)bk;
-      }
-      if (bi2 >= 0 && (double)ub2 >= thr) {
-        r.e2 = (uint8_t)bi2;
-        r.k2 = (uint8_t)bk2;
-      }
-      *simple = r;
-      return true;
-    }
-    const unsigned long long q = atomicAdd(nq, 1ull);
-    queue[q] = (uint32_t)p;
-    return false;
   }
   // exact margins of the other pairs: first the one with the largest bound
   // (if it can exceed best_in), then (if the second-largest bound exceeds
@@ -763,7 +965,6 @@ __device__ __noinline__ bool cert_point(const CertShared &sh, int NL, const doub
     rec32[p * rs + d] = (float)best;
     rec32[p * rs + d + 1] = cert_rec_word(be, best >= 0.0);
   }
-  return false;
 }
 
 // A settled point (CertRec): the FP64 chain to the deeper of the pairs'
@@ -878,8 +1079,7 @@ __global__ void __launch_bounds__(CERT_THREADS) k_certify_points(
   CertRec rec;
   bool simple = false;
   if (p < n)
-    simple = cert_point<true>(sh, NL, radius, NS, nobs, pts, p, d, verdict, margin, element, rec32,
-                              &rec, queue, nq);
+    simple = cert_first(sh, NL, radius, NS, nobs, pts, p, d, &rec, queue, nq);
   // counting sort of the settled points by (chain depth, obstacle type) of
   // their deeper pair within the block (key 0: no exact evaluation)
   int key = 0, pos = 0;
@@ -935,8 +1135,7 @@ __global__ void __launch_bounds__(CERT_THREADS) k_certify_points_rest(
   const unsigned long long m = *nq;
   for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < m;
        i += (uint64_t)gridDim.x * blockDim.x)
-    cert_point<false>(sh, NL, radius, NS, nobs, pts, (int64_t)queue[i], d, verdict, margin,
-                      element, rec32, nullptr, nullptr, nullptr);
+    cert_point(sh, NL, radius, NS, nobs, pts, (int64_t)queue[i], d, verdict, margin, element, rec32);
 }
 
 // Whole-cell certificate (one thread per cell): with lo_k / hi_k the range of
