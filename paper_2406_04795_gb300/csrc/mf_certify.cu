@@ -620,9 +620,9 @@ __device__ __forceinline__ void cert_bounds(const CertShared &sh, int nobs, int 
 // bounds tight enough to queue fewer points, certifying 500,000 points (6
 // capsules and 18 robot spheres, 18 obstacles) takes 2.5 ms instead of 4.7,
 // and this pass over a d = 5 proof at lambda = 0.08 6.4 ms instead of 8.2.
-// A point that at most two exact pair
-// evaluations settle returns true with its record in *simple for
-// cert_simple_eval; every other point is appended to queue.
+// A point that at most two exact pair evaluations settle returns true with its
+// record in *simple for cert_simple_eval; every other point is appended to
+// queue.
 __device__ __forceinline__ bool cert_first(const CertShared &sh, int NL, const double *radius,
                                            int NS, int nobs, const double *pts, int64_t p, int d,
                                            CertRec *simple, uint32_t *queue,

@@ -765,6 +765,7 @@ __device__ int warp_vertex_list(const MfRbfDev &R, const float *xh, float list_r
 template <int D>
 __global__ void __launch_bounds__(EVAL_WARPS * 32) k_vertex_lists(MfFrame F, MfRbfDev R, MfTraceBufs B) {
   __shared__ int slist[EVAL_WARPS][LIST_CAP];
+  mf_dep_wait();
   const int w = threadIdx.x >> 5;
   const uint64_t begin = B.cnt->v_evaluated;
   uint64_t end = B.cnt->n_vertices;
@@ -787,6 +788,7 @@ template <int D>
 __global__ void __launch_bounds__(EVAL_WARPS * 32) k_eval_vertices_f64(MfFrame F, MfRbfDev R, MfTraceBufs B) {
   __shared__ int sq[EVAL_WARPS][2][64];
   __shared__ int slist[EVAL_WARPS][LIST_CAP];
+  mf_dep_wait();
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint64_t begin = B.cnt->v_evaluated;
   uint64_t end = B.cnt->n_vertices;
@@ -818,6 +820,7 @@ __global__ void __launch_bounds__(EVAL_WARPS * 32) k_eval_vertices_f64(MfFrame F
 template <int D>
 __global__ void __launch_bounds__(EVAL_WARPS * 32) k_recheck_vertices_f64(MfFrame F, MfRbfDev R, MfTraceBufs B) {
   __shared__ int sq[EVAL_WARPS][2][64];
+  mf_dep_wait();
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint64_t begin = B.cnt->n_recheck_done;
   uint64_t end = B.cnt->n_recheck;
@@ -888,6 +891,7 @@ __global__ void __launch_bounds__(MIX_WARPS * 32) k_eval_mixed_f32(MfFrame F, Mf
   extern __shared__ __align__(16) unsigned char mix_raw[];
   MixShared<D> &sh = *reinterpret_cast<MixShared<D> *>(mix_raw);
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, W = blockDim.x >> 5;
+  mf_dep_wait();
   uint64_t begin = 0, end = (uint64_t)npts;
   if (VERTS) {
     begin = B.cnt->v_evaluated;
@@ -1023,7 +1027,8 @@ static void launch_mixed_f32_d(const MfFrame &F, const MfRbfDev &R, const MfTrac
   cudaFuncSetAttribute(k_eval_mixed_f32<VERTS, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
   const int64_t full = (int64_t)sms * 8;
   const int64_t g = VERTS ? full : std::min(full, (npts + 31) / 32);
-  k_eval_mixed_f32<VERTS, D><<<(unsigned)g, W * 32, bytes, st>>>(F, R, B, pts, npts, fout, flag, band);
+  mf_launch_dep(k_eval_mixed_f32<VERTS, D>, (unsigned)g, W * 32, bytes, st, F, R, B, pts, npts, fout,
+                flag, band);
 }
 
 template <bool VERTS>
@@ -2283,10 +2288,10 @@ void mf_launch_eval_vertices_f64(const MfFrame &F, const MfRbfDev &R, const MfTr
   const int g = sms * T.eval_bps;
   switch (F.d) {
 #define MF_CASE(DD) \
-  case DD: k_eval_vertices_f64<DD><<<g, EVAL_WARPS * 32, 0, st>>>(F, R, B); break;
+  case DD: mf_launch_dep(k_eval_vertices_f64<DD>, g, EVAL_WARPS * 32, 0, st, F, R, B); break;
     MF_CASE(2) MF_CASE(3) MF_CASE(4) MF_CASE(5) MF_CASE(6) MF_CASE(7)
 #undef MF_CASE
-    default: k_eval_vertices_f64<MF_MAXD><<<g, EVAL_WARPS * 32, 0, st>>>(F, R, B);
+    default: mf_launch_dep(k_eval_vertices_f64<MF_MAXD>, g, EVAL_WARPS * 32, 0, st, F, R, B);
   }
   if (advance) k_advance_eval<<<1, 1, 0, st>>>(B.cnt);
 }
@@ -2301,18 +2306,18 @@ void mf_launch_eval_vertices_mixed(const MfFrame &F, const MfRbfDev &R, const Mf
   if (B.vlist) {  // the root screen's per-vertex lists
     switch (F.d) {
 #define MF_CASE(DD) \
-  case DD: k_vertex_lists<DD><<<sms * 8, EVAL_WARPS * 32, 0, st>>>(F, R, B); break;
+  case DD: mf_launch_dep(k_vertex_lists<DD>, sms * 8, EVAL_WARPS * 32, 0, st, F, R, B); break;
       MF_CASE(2) MF_CASE(3) MF_CASE(4) MF_CASE(5) MF_CASE(6) MF_CASE(7)
 #undef MF_CASE
-      default: k_vertex_lists<MF_MAXD><<<sms * 8, EVAL_WARPS * 32, 0, st>>>(F, R, B);
+      default: mf_launch_dep(k_vertex_lists<MF_MAXD>, sms * 8, EVAL_WARPS * 32, 0, st, F, R, B);
     }
   }
   switch (F.d) {
 #define MF_CASE(DD) \
-  case DD: k_recheck_vertices_f64<DD><<<sms * 8, EVAL_WARPS * 32, 0, st>>>(F, R, B); break;
+  case DD: mf_launch_dep(k_recheck_vertices_f64<DD>, sms * 8, EVAL_WARPS * 32, 0, st, F, R, B); break;
     MF_CASE(2) MF_CASE(3) MF_CASE(4) MF_CASE(5) MF_CASE(6) MF_CASE(7)
 #undef MF_CASE
-    default: k_recheck_vertices_f64<MF_MAXD><<<sms * 8, EVAL_WARPS * 32, 0, st>>>(F, R, B);
+    default: mf_launch_dep(k_recheck_vertices_f64<MF_MAXD>, sms * 8, EVAL_WARPS * 32, 0, st, F, R, B);
   }
   if (advance) k_advance_eval<<<1, 1, 0, st>>>(B.cnt);
 }

@@ -311,6 +311,7 @@ template <int D, int N>
 __global__ void __launch_bounds__(TC_M, TcCfg<N>::kCtasPerSm) k_eval_tc(MfFrame F, MfRbfDev R,
                                                                         MfTraceBufs B, double band) {
   __shared__ TcShared<N> sh;
+  mf_dep_wait();
   const uint64_t begin = B.cnt->v_evaluated;
   uint64_t end = B.cnt->n_vertices;
   if (end > B.max_vertices) end = B.max_vertices;
@@ -372,7 +373,7 @@ static void launch_tc(const MfFrame &F, const MfRbfDev &R, const MfTraceBufs &B,
   case DD:                                                                                \
     cudaFuncSetAttribute(k_eval_tc<DD, N>, cudaFuncAttributeMaxDynamicSharedMemorySize,   \
                          (int)dyn);                                                       \
-    k_eval_tc<DD, N><<<grid, TC_M, dyn, st>>>(F, R, B, band);                             \
+    mf_launch_dep(k_eval_tc<DD, N>, grid, TC_M, dyn, st, F, R, B, band);                  \
     break;
     MF_CASE(2) MF_CASE(3) MF_CASE(4) MF_CASE(5) MF_CASE(6) MF_CASE(7) MF_CASE(8)
 #undef MF_CASE

@@ -331,7 +331,7 @@ __device__ __forceinline__ int expand_owner(const uint32_t *s_end, uint32_t j, u
 // are chains of dependent accesses (slot, f, probe, append), so a level that
 // leaves SMs empty takes as long as its longest warp: with 32 edges per warp a
 // d = 3 level of 500 edges ran 6 rounds on 2 blocks (36 us), with 4 edges 1
-// round on 16 blocks.
+// round on 16 blocks (9 us; the vertex pass 15 -> 6).
 __device__ __forceinline__ int expand_group(int d, unsigned long long n, unsigned long long nwarps) {
   int g = d <= 2 ? 16 : d == 3 ? 4 : d == 4 ? 2 : 1;
   while (g < 32 && n > (unsigned long long)g * nwarps) g <<= 1;
@@ -346,10 +346,11 @@ struct ExpandShared {
 };
 
 // Edges [e0, e0 + n): a warp takes expand_group edges, lane per coface item,
-// so that no lane idles on masks that select no coface.
+// so that no lane idles on masks that select no coface.  Returns the number of
+// blocks of the grid that have work (the first ones).
 template <bool EDGES>
-__device__ __forceinline__ void expand_range(const MfFrame &F, const MfTraceBufs &B, uint64_t e0,
-                                             uint64_t n) {
+__device__ __forceinline__ unsigned expand_range(const MfFrame &F, const MfTraceBufs &B, uint64_t e0,
+                                                 uint64_t n) {
   __shared__ ExpandShared sh;
   const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5;
   const int d = F.d;
@@ -420,6 +421,8 @@ __device__ __forceinline__ void expand_range(const MfFrame &F, const MfTraceBufs
     nb = __reduce_add_sync(0xffffffffu, nb);
     if (lane == 0 && nb) atomicAdd(&B.cnt->n_boundary, (unsigned long long)nb);
   }
+  const uint64_t used = (n + G * EXPAND_WARPS - 1) / (G * EXPAND_WARPS);
+  return (unsigned)(used < gridDim.x ? used : gridDim.x);
 }
 
 // The search's steps live in the counters, so that the host can enqueue several
@@ -461,7 +464,8 @@ __device__ __forceinline__ void search_next(const MfTraceBufs &B) {
 template <int D>
 __global__ void __launch_bounds__(EXPAND_WARPS * 32) k_expand_vertices(MfFrame F, MfTraceBufs B,
                                                                        uint64_t e0, uint64_t n) {
-  if (D < MF_MAXD) __builtin_assume(F.d == D);
+  if (D < MF_MAXD) F.d = D;  // the coordinate loops then unroll to exactly D
+  mf_dep_wait();
   if (n == MF_STEP) {
     e0 = B.cnt->lv_begin;
     n = B.cnt->lv_n;
@@ -472,19 +476,20 @@ __global__ void __launch_bounds__(EXPAND_WARPS * 32) k_expand_vertices(MfFrame F
 template <int D>
 __global__ void __launch_bounds__(EXPAND_WARPS * 32) k_expand_edges(MfFrame F, MfTraceBufs B,
                                                                     uint64_t e0, uint64_t n) {
-  if (D < MF_MAXD) __builtin_assume(F.d == D);
+  if (D < MF_MAXD) F.d = D;  // the coordinate loops then unroll to exactly D
+  mf_dep_wait();
   const bool step = n == MF_STEP;
   if (step) {
     e0 = B.cnt->lv_begin;
     n = B.cnt->lv_n;
     if (n == 0) return;  // every block of the launch sees the same step
   }
-  expand_range<true>(F, B, e0, n);
-  if (step) {  // the last block to finish opens the next step
+  const unsigned used = expand_range<true>(F, B, e0, n);
+  if (step && blockIdx.x < used) {  // the last of those blocks to finish opens the next step
     __syncthreads();
     if (threadIdx.x == 0) {
       __threadfence();
-      if (atomicAdd(&B.cnt->lv_ticket, 1u) == gridDim.x - 1) {
+      if (atomicAdd(&B.cnt->lv_ticket, 1u) == used - 1) {
         __threadfence();
         B.cnt->lv_ticket = 0;
         search_next(B);
@@ -808,7 +813,7 @@ __global__ void __launch_bounds__(CELL_WARPS * 32) k_cells_enum(MfFrame F, MfTra
                                                                 uint64_t n_edges) {
   constexpr int W = CellLanes<D>::W, PER = 32 / W;
   __shared__ CellLink<D> sl[CELL_WARPS * PER];
-  if (D < MF_MAXD) __builtin_assume(F.d == D);
+  if (D < MF_MAXD) F.d = D;  // the coordinate loops then unroll to exactly D
   const uint64_t first = (blockIdx.x * (uint64_t)CELL_WARPS + (threadIdx.x >> 5)) * PER;
   if (first >= n_edges) return;  // whole warp
   const uint64_t e = first + (threadIdx.x & 31) / W;
@@ -1534,14 +1539,14 @@ void mf_launch_expand(const MfFrame &F, const MfTraceBufs &B, uint64_t e0, uint6
   switch (F.d) {
 #define MF_CASE(DD)                                                                   \
   case DD:                                                                            \
-    if (edges) k_expand_edges<DD><<<g, EXPAND_WARPS * 32, 0, st>>>(F, B, e0, n);       \
-    else k_expand_vertices<DD><<<g, EXPAND_WARPS * 32, 0, st>>>(F, B, e0, n);          \
+    mf_launch_dep(edges ? k_expand_edges<DD> : k_expand_vertices<DD>, g, EXPAND_WARPS * 32, 0, st, F, B, \
+                  e0, n);                                                             \
     break;
     MF_CASE(2) MF_CASE(3) MF_CASE(4) MF_CASE(5) MF_CASE(6) MF_CASE(7)
 #undef MF_CASE
     default:
-      if (edges) k_expand_edges<MF_MAXD><<<g, EXPAND_WARPS * 32, 0, st>>>(F, B, e0, n);
-      else k_expand_vertices<MF_MAXD><<<g, EXPAND_WARPS * 32, 0, st>>>(F, B, e0, n);
+      mf_launch_dep(edges ? k_expand_edges<MF_MAXD> : k_expand_vertices<MF_MAXD>, g,
+                    EXPAND_WARPS * 32, 0, st, F, B, e0, n);
   }
 }
 void mf_launch_seeds(const MfFrame &F, const MfTraceBufs &B, const double *seeds, int64_t n,
