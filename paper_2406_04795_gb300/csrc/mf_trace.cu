@@ -821,77 +821,63 @@ __global__ void __launch_bounds__(CELL_WARPS * 32) k_cells_enum(MfFrame F, MfTra
   cells_enum_edge<D, true>(F, B, have ? e : first, have, sl[threadIdx.x / W]);
 }
 
-// Cell -> traced edges: the (d+1)d/2 edges of the cell (query type 2) found
-// in the edge table.  FILL = false counts, FILL = true writes indices.
-template <bool FILL>
-__device__ __forceinline__ void cell_edges_item(const MfFrame &F, const MfTraceBufs &B, uint64_t c,
-                                                int64_t *cnt_or_off);
-
-template <bool FILL>
-__global__ void k_cells_edges(MfFrame F, MfTraceBufs B, uint64_t n_cells, int64_t *cnt_or_off) {
-  const uint64_t c = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
-  if (c >= n_cells) return;
-  cell_edges_item<FILL>(F, B, c, cnt_or_off);
-}
-
-template <bool FILL>
-__device__ __forceinline__ void cell_edges_item(const MfFrame &F, const MfTraceBufs &B, uint64_t c,
-                                                int64_t *cnt_or_off) {
-  // The cell's vertices v_0 = z, v_i = v_{i-1} + e(pi_{i-1}) (query type 5).
-  // Each of them lies in the domain iff it is in the vertex table: the BFS
-  // visits the third vertex of every 2-coface of a traced edge, and every
-  // vertex of this cell shares a 2-coface with the traced edge that made it.
-  // Inside one simplex all crossing edges between in-domain vertices are
-  // linked through 2-cofaces, so the traced edges of the cell are exactly its
-  // in-domain vertex pairs with different signs: the count pass needs only
-  // the d+1 vertex signs, and the fill pass looks up only those pairs.
-  const int d = F.d;
+// Cell -> traced edges: the (d+1)d/2 edges of the cell (query type 2) found in
+// the edge table.  The cell's vertices are v_0 = z, v_i = v_{i-1} + e(pi_{i-1})
+// (query type 5); each of them lies in the domain iff it is in the vertex
+// table: the BFS visits the third vertex of every 2-coface of a traced edge,
+// and every vertex of this cell shares a 2-coface with the traced edge that
+// made it.  Inside one simplex all crossing edges between in-domain vertices
+// are linked through 2-cofaces, so the traced edges of the cell are exactly its
+// in-domain vertex pairs with different signs, and only those are looked up,
+// by the sign mask that the enumeration left.  Bound by the probes' latency;
+// a vertex's key is computed once for all its pairs.
+template <int D>
+__device__ __forceinline__ void cell_fill_item(const MfFrame &F, const MfTraceBufs &B, uint64_t c,
+                                               const int64_t *off) {
+  const int d = D < MF_MAXD ? D : F.d;
   int32_t vi[MF_MAXD];
   load_y(B.cell_y + c * d, d, vi);
   // the permutation as 4-bit nibbles (no indexed local array)
   uint64_t pw = 0;
-  for (int k = 0; k < d; k++) pw |= (uint64_t)B.cell_perm[c * d + k] << (4 * k);
-  uint32_t sg;
-  if (!FILL) {
-    uint32_t in = 0, pos = 0;
-    int32_t w[MF_MAXD];
-    load_y(vi, d, w);
-    for (int i = 0; i <= d; i++) {
-      if (i > 0) {
-        const int p = (int)((pw >> (4 * (i - 1))) & 15ull);
 #pragma unroll
-        for (int k = 0; k < MF_MAXD; k++) w[k] += k == p ? 1 : 0;
-      }
-      const uint64_t slot = mf_table_find<2>(B.vtab_key, B.vtab_mask, mf_vertex_key(F, w));
-      if (slot == ~0ull) continue;
-      in |= 1u << i;
-      if (mf_vtab_f(B, slot) >= 0.0) pos |= 1u << i;
-    }
-    sg = in | (pos << 16);
-    B.cell_sgn[c] = sg;
-    cnt_or_off[c] = (int64_t)__popc(in & pos) * (int64_t)__popc(in & ~pos);
-    return;
-  }
-  sg = B.cell_sgn[c];
-  const uint32_t in = sg & 0xFFFFu, pos = sg >> 16;
-  int64_t at = cnt_or_off[c];
+  for (int k = 0; k < MF_MAXD; k++)
+    if (k < d) pw |= (uint64_t)B.cell_perm[c * d + k] << (4 * k);
+  const uint32_t sg = B.cell_sgn[c], in = sg & 0xFFFFu, pos = sg >> 16;
+  const uint32_t P = in & pos, N = in & ~pos;
+  int64_t at = off[c];
+#pragma unroll 1
   for (int i = 0; i < d; i++) {
-    uint32_t mask = 0;
-    for (int j = i + 1; j <= d; j++) {
-      mask |= 1u << (uint32_t)((pw >> (4 * (j - 1))) & 15ull);
-      if (!((in >> i) & (in >> j) & 1u) || ((pos >> i) & 1u) == ((pos >> j) & 1u)) continue;
-      const uint64_t slot = mf_table_find<2>(B.etab_key, B.etab_mask, mf_edge_key(F, vi, mask));
-      if (slot == ~0ull) {
-        atomicOr(&B.cnt->err_missing, 2u);
-        B.cell_idx[at++] = -1;
-        continue;
+    // the vertices after i with the other sign
+    const uint32_t other = ((P >> i) & 1u ? N : ((N >> i) & 1u ? P : 0u)) >> (i + 1);
+    if (other) {
+      const unsigned long long key = mf_vertex_key(F, vi) << d;
+      uint32_t mask = 0;
+#pragma unroll 1
+      for (int j = i + 1; j <= d; j++) {
+        mask |= 1u << (uint32_t)((pw >> (4 * (j - 1))) & 15ull);
+        if (!((other >> (j - i - 1)) & 1u)) continue;
+        const uint64_t slot = mf_table_find<2>(B.etab_key, B.etab_mask, key | mask);
+        if (slot == ~0ull) {
+          atomicOr(&B.cnt->err_missing, 2u);
+          B.cell_idx[at++] = -1;
+          continue;
+        }
+        B.cell_idx[at++] = (int64_t)mf_etab_val(B, slot);
       }
-      B.cell_idx[at++] = (int64_t)mf_etab_val(B, slot);
     }
     const int p = (int)((pw >> (4 * i)) & 15ull);
 #pragma unroll
     for (int k = 0; k < MF_MAXD; k++) vi[k] += k == p ? 1 : 0;
   }
+}
+
+template <int D>
+__global__ void __launch_bounds__(256) k_cells_fill(MfFrame F, MfTraceBufs B, uint64_t n_cells,
+                                                    const int64_t *off) {
+  const uint64_t c = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
+  if (c >= n_cells) return;
+  if (D < MF_MAXD) F.d = D;
+  cell_fill_item<D>(F, B, c, off);
 }
 
 // ---------------------------------------------------------------------------
@@ -1179,14 +1165,13 @@ __global__ void __launch_bounds__(CELL_WARPS * 32) k_b_cells_enum(const MfSlot *
   }
 }
 
-template <bool FILL>
-__global__ void k_b_cell_edges(const MfSlot *slots, const MfBatchPlan *P, int n) {
+__global__ void __launch_bounds__(256) k_b_cells_fill(const MfSlot *slots, const MfBatchPlan *P, int n) {
   const unsigned long long total = P->pc[n];
   const unsigned long long stride = (unsigned long long)gridDim.x * blockDim.x;
   for (unsigned long long item = blockIdx.x * (unsigned long long)blockDim.x + threadIdx.x;
        item < total; item += stride) {
     const int t = mf_slot_of(P->pc, n, item);
-    cell_edges_item<FILL>(slots[t].F, slots[t].B, item - P->pc[t], slots[t].B.cell_off);
+    cell_fill_item<MF_MAXD>(slots[t].F, slots[t].B, item - P->pc[t], slots[t].B.cell_off);
   }
 }
 
@@ -1239,7 +1224,7 @@ void mf_b_launch_cell_edges(const MfSlot *slots, MfBatchPlan *P, int n, bool fil
     // enumeration (cells_enum_edge), so no counting pass is needed
     k_b_plan_edges<<<1, MF_MAX_SLOTS, 0, s>>>(slots, P, n, 1, only, 0);
   } else {
-    k_b_cell_edges<true><<<sms * 8, 256, 0, s>>>(slots, P, n);
+    k_b_cells_fill<<<sms * 8, 256, 0, s>>>(slots, P, n);
   }
 }
 
@@ -1514,7 +1499,14 @@ int mf_build_domain_table(mf_ctx *ctx, MfFrame *F, cudaStream_t st);
 int mf_read_counters(mf_ctx *ctx, const MfTraceBufs &B, cudaStream_t st);
 void mf_launch_cells_fill(const MfFrame &F, const MfTraceBufs &B, uint64_t n_cells, cudaStream_t st) {
   if (n_cells == 0) return;
-  k_cells_edges<true><<<(unsigned)((n_cells + 255) / 256), 256, 0, st>>>(F, B, n_cells, B.cell_off);
+  const unsigned g = (unsigned)((n_cells + 255) / 256);
+  switch (F.d) {
+#define MF_CASE(DD) \
+  case DD: k_cells_fill<DD><<<g, 256, 0, st>>>(F, B, n_cells, B.cell_off); break;
+    MF_CASE(2) MF_CASE(3) MF_CASE(4) MF_CASE(5) MF_CASE(6) MF_CASE(7) MF_CASE(8)
+#undef MF_CASE
+    default: break;
+  }
 }
 void mf_launch_cells_enum(const MfFrame &F, const MfTraceBufs &B, uint64_t n_edges, cudaStream_t st) {
   if (n_edges == 0) return;
@@ -1882,7 +1874,6 @@ extern "C" int mf_trace(mf_ctx *ctx, const mf_rbf *rbf, const mf_domain *dom,
     rc = read_counters(ctx, B, st);
     if (rc) return rc;
     n_cells = (int64_t)ctx->h_counters->n_cells;
-    const unsigned g = (unsigned)((n_cells + 255) / 256);
     int64_t *scratch = (int64_t *)mf_ctx_buffer(ctx, MF_SLOT_SCAN,
                                                 ((size_t)n_cells / SCAN_TILE + 2) * 8);
     if (!scratch) return MF_ERR_OOM;
@@ -1901,7 +1892,7 @@ extern "C" int mf_trace(mf_ctx *ctx, const mf_rbf *rbf, const mf_domain *dom,
     if (!B.cell_idx) return MF_ERR_OOM;
     {
       MfProfScope ps(ctx, MF_PH_CSR, st, 1);
-      k_cells_edges<true><<<g, 256, 0, st>>>(F, B, (uint64_t)n_cells, B.cell_off);
+      mf_launch_cells_fill(F, B, (uint64_t)n_cells, st);
     }
   }
   rc = mf_cuda_check(ctx, cudaGetLastError(), "CSR kernels");
