@@ -33,15 +33,9 @@
 
 #include "mf_internal.cuh"
 #include "mf_ctx.h"
+#include "mf_root.cuh"
 
-#define FULL 0xffffffffu
 #define STRONG_TAU 3e-10  // terms above this magnitude use the FP64 exp
-
-__device__ __forceinline__ float ex2_approx(float x) {
-  float y;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
 
 // ---------------------------------------------------------------------------
 // RBF preparation
@@ -416,13 +410,6 @@ struct Split32 {
   float hi[D], lo[D], dir[D];
 };
 
-// Dimension of the work: a compile-time D below MF_MAXD is exact; D ==
-// MF_MAXD serves every d <= MF_MAXD at run time.
-template <int D>
-__device__ __forceinline__ int dim_of(int rt) {
-  return D < MF_MAXD ? D : rt;
-}
-
 // (All lanes, converged.)  Lane k < d converts axis k and shuffles
 // broadcast the parts: each FP64 instruction holds the FP64 pipe for the
 // whole warp, so one conversion per lane serves every axis at once.
@@ -521,33 +508,6 @@ __device__ __forceinline__ void f64_term(const MfRbfDev &R, const double *x, con
   const double e = R.alpha[j] * mf_exp_neg(-R.gamma * r2, R.exp_tab);
   acc.f += e;
   if (GRAD) acc.g = fma(e, proj, acc.g);
-}
-
-// Support vector j's row for the root path, in one gather: the hi/lo
-// coordinate pairs c[2k], c[2k + 1] (k < D) and, below 8 coordinates, alpha
-// and the strong threshold from the row's padding (else from their arrays).
-template <int D>
-__device__ __forceinline__ void sv_row(const MfRbfDev &R, int j, float *c, float &al, float &s32) {
-  constexpr int Q = D < 8 ? (2 * D + 2 + 3) / 4 : 4;
-  const float4 *row = reinterpret_cast<const float4 *>(R.svhl + (int64_t)j * 16);
-  float v[4 * Q];
-#pragma unroll
-  for (int q = 0; q < Q; q++) {
-    const float4 t = __ldg(row + q);
-    v[4 * q] = t.x;
-    v[4 * q + 1] = t.y;
-    v[4 * q + 2] = t.z;
-    v[4 * q + 3] = t.w;
-  }
-#pragma unroll
-  for (int k = 0; k < 2 * D && k < 4 * Q; k++) c[k] = v[k];
-  if (D < 8) {
-    al = v[D < 8 ? 2 * D : 0];
-    s32 = v[D < 8 ? 2 * D + 1 : 0];
-  } else {
-    al = R.alpha32[j];
-    s32 = R.strong32[j];
-  }
 }
 
 // Weak term (|alpha| e <= tau): FP32 throughout with hi/lo-split coordinates.
@@ -1105,16 +1065,6 @@ static void launch_eval_points_f64(const MfRbfDev &R, const double *pts, int64_t
 #define ROOT_WARPS 8
 #define NEAR_CAP 1024
 #define MID_CAP 256
-// The root's FP64 step evaluates in FP64 only the terms that can exceed
-// ROOT_TAU = 1e-8 (strong32 shifted by ln(ROOT_TAU / STRONG_TAU)); the band
-// between STRONG_TAU and ROOT_TAU ("mid") joins the FP32 stage's list and is
-// summed in FP32 with the weak terms in the FP64 step.
-#define ROOT_TAU_SHIFT 3.5065579f
-// The mixed paths need |dt| <= 1e-6 only: their FP64 step takes the terms
-// that can exceed 1e-5 (shift ln(1e-5 / STRONG_TAU)); the FP32 part may then
-// move t by up to 1e-7 and the accepted Newton step leaves < 1e-7.
-#define ROOT_TAU_SHIFT_FAST 10.414313f
-
 // Warp sums of four values, every lane receiving all four: a transposed
 // butterfly (lanes split the values between halves, then quarters, before
 // the plain butterfly), 10 shuffles and 6 adds instead of 20 and 20.
@@ -1262,15 +1212,6 @@ __device__ __forceinline__ void root_fp32_part(const MfRbfDev &R, const int *nea
   }
 }
 
-// Relative error bound of a cached weak term on an edge with |dir|^2 = dd32
-// (every kept vector lies within the screen radius sqrt(rs2) of the segment;
-// 1.1 covers this bound's own FP32 rounding).
-__device__ __forceinline__ float root_rel_cached(const MfRbfDev &R, int d, float dd32, float rs2) {
-  const float q = sqrtf(rs2) + 2.f * sqrtf(dd32);
-  return 1.1f * ((float)d + 8.f) * 5.9604644775390625e-08f * (float)R.gamma * q * q +
-         9.5367431640625e-07f + 2.f * 5.9604644775390625e-08f;
-}
-
 // FP64 evaluation of g and g' at x over the near list (all lanes); xs is x
 // split into FP32 hi/lo parts for the weak terms.
 template <bool ALL_STRONG, bool GRAD, int D>
@@ -1299,37 +1240,6 @@ __device__ __forceinline__ F64Acc root_eval64(const MfRbfDev &R, const int *near
   return acc;
 }
 
-// Solves the root of edge e (all lanes of the warp); near: NEAR_CAP ints,
-// qs / qw: 64-entry queues, all in this warp's shared memory.  src (srcn
-// entries, ascending) lists the support vectors that can pass the segment
-// screen (a group screen's survivors); NULL screens all of them.  FP64 work
-// that is the same for every lane (coordinates, their splits) runs once per
-// axis: lane k < d computes axis k and shuffles broadcast it.
-// The FP32 part of a root evaluation (mid and weak terms) errs by at most
-// weak_rel * sum|terms|; with the dropped terms (drop_bound) that must stay
-// below 1e-10 |g'| (t then moves by at most 1e-10), or below the vertex
-// evaluation's own limit, whichever is larger.  Otherwise the point is
-// evaluated again with every kept term in FP64.
-// (The check runs in FP32: the 1.01 factor covers its roundings.)
-__device__ __forceinline__ bool root_fp32_part_too_coarse(const MfRbfDev &R, float weak, float gp,
-                                                          bool fast) {
-  const float lim = fmaxf(R.weak_limit32, (fast ? 0.99e-7f : 0.99e-10f) * fabsf(gp) -
-                                              (fast ? R.drop_bound32_fast : R.drop_bound32));
-  return weak * (1.01f * R.weak_rel32) > lim;
-}
-
-// A root step handed to the lane-per-edge FP64 kernels (k_roots_terms,
-// k_roots_finish): the edge (~0: none), the FP32 stage's t (where the FP64
-// evaluation happens), the reused g' there and |g''|, the FP32 part of g at
-// t (mid and weak terms, already checked against its error bound), and its
-// strong entries: ns of them, in the 8-entry chunks from chunk ch on.
-struct __align__(16) RootRec {
-  unsigned long long e;
-  float t, gp, gpp, wf;
-  uint32_t ch, ns;
-};
-#define DEFER_CHUNK 8
-
 // The FP64 end points of edge e on axis k, in mf_vertex_x's operation order:
 // x1 = x(y), x2 = x(y + e(mask)), dir = x2 - x1.
 __device__ __forceinline__ void root_ends64(const MfFrame &F, double cs1, double cs2, int32_t yk,
@@ -1346,6 +1256,12 @@ struct RootWarpState {
   float hl[3 * MF_MAXD];  // Split32<D> image: hi[D], lo[D], dir[D]
 };
 
+// Solves the root of edge e (all lanes of the warp); near: NEAR_CAP ints,
+// qs / qw: 64-entry queues, all in this warp's shared memory.  src (srcn
+// entries, ascending) lists the support vectors that can pass the segment
+// screen (a group screen's survivors); NULL screens all of them.  FP64 work
+// that is the same for every lane (coordinates, their splits) runs once per
+// axis: lane k < d computes axis k and shuffles broadcast it.
 // ep32 / ep64: the chunk's end points from k_roots_prep (edge e at row
 // e - ep0), or NULL (every lane k < d then computes axis k here in FP64).
 template <int D>
@@ -1880,8 +1796,9 @@ __global__ void __launch_bounds__(256) k_roots_prep(MfFrame F, MfTraceBufs B, ui
 // The evaluation point x = x1 + t (x2 - x1) of each deferred step (thread
 // per record), in root_edge's operation order, split into three floats per
 // coordinate (x = x1 + x2 + x3 exactly) for the double-float terms: record
-// i at B.defer_x3[3 d i].
-template <int D>
+// i at B.defer_x3[3 d i].  GROUPED: the end points are computed here, into
+// row i of B.defer_x; else k_roots_prep left them in row e - e0.
+template <int D, bool GROUPED>
 __global__ void __launch_bounds__(256) k_roots_x(MfFrame F, MfTraceBufs B, uint64_t cap, uint64_t e0) {
   const unsigned long long nrec = B.cnt->n_defer < cap ? B.cnt->n_defer : cap;
   const uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
@@ -1889,14 +1806,36 @@ __global__ void __launch_bounds__(256) k_roots_x(MfFrame F, MfTraceBufs B, uint6
   const int d = dim_of<D>(F.d);
   const RootRec rec = reinterpret_cast<const RootRec *>(B.defer_rec)[i];
   if (rec.e == ~0ull) return;
-  // x1 and dir as k_roots_prep computed them (row rec.e - e0)
-  const double *row64 = B.defer_x + (rec.e - e0) * 2 * (uint64_t)d;
+  double *row64 = B.defer_x + (GROUPED ? i : rec.e - e0) * 2 * (uint64_t)d;
   const double t = (double)rec.t;
   float *xp = B.defer_x3 + i * 3 * (uint64_t)d;
+  int32_t y[D];
+  uint32_t mask = 0;
+  double cs1 = 0.0, cs2 = 0.0;
+  if (GROUPED) {
+    long long sy = 0;
+#pragma unroll
+    for (int k = 0; k < D; k++) {
+      y[k] = k < d ? B.edge_y[rec.e * d + k] : 0;
+      sy += y[k];
+    }
+    mask = B.edge_mask[rec.e] & ((1u << d) - 1u);
+    cs1 = __dmul_rn(F.c, (double)sy);
+    cs2 = __dmul_rn(F.c, (double)(sy + __popc(mask)));
+  }
 #pragma unroll
   for (int k = 0; k < D; k++) {
     if (k < d) {
-      const double x = __dadd_rn(row64[k], __dmul_rn(t, row64[d + k]));
+      double x1, dir;
+      if (GROUPED) {
+        root_ends64(F, cs1, cs2, y[k], (mask >> k) & 1u, k, x1, dir);
+        row64[k] = x1;
+        row64[d + k] = dir;
+      } else {
+        x1 = row64[k];
+        dir = row64[d + k];
+      }
+      const double x = __dadd_rn(x1, __dmul_rn(t, dir));
       const float h = (float)x;
       const double r = x - (double)h;
       const float m = (float)r;
@@ -2018,7 +1957,7 @@ __global__ void __launch_bounds__(256) k_roots_terms(MfRbfDev R, MfTraceBufs B, 
 // sums in order) + (FP32 part) + b at x, one Newton step with the reused g'
 // under root_edge's acceptance tests.  Accepted steps write t and the point
 // (x1 + t dir in root_edge's order); the others go to the redo queue.
-template <int D>
+template <int D, bool GROUPED>
 __global__ void __launch_bounds__(256) k_roots_finish(MfFrame F, MfRbfDev R, MfTraceBufs B,
                                                       uint64_t cap, double tol, int fast,
                                                       uint64_t e0) {
@@ -2033,12 +1972,13 @@ __global__ void __launch_bounds__(256) k_roots_finish(MfFrame F, MfRbfDev R, MfT
       const uint64_t e = rec.e;
       double fs = 0.0;
       float w = 0.f;
-      const uint32_t nc = (rec.ns + DEFER_CHUNK - 1) / DEFER_CHUNK;
+      const uint32_t ns = GROUPED ? rec.ns & 0x7fffffffu : rec.ns;
+      const uint32_t nc = (ns + DEFER_CHUNK - 1) / DEFER_CHUNK;
       for (uint32_t c = 0; c < nc; c++) {
         fs += B.defer_part[rec.ch + c];
         w += B.defer_bnd[rec.ch + c];
       }
-      terms += rec.ns;
+      terms += ns;
       evals++;
       const double t = (double)rec.t;
       const double f = fs + (double)rec.wf + R.b;
@@ -2048,21 +1988,24 @@ __global__ void __launch_bounds__(256) k_roots_finish(MfFrame F, MfRbfDev R, MfT
       bool ok = 2.f * 0x1p-43f * w <= (fast ? 0.99e-7f : 2e-10f) * fabsf(rec.gp);
       const long long fb = __double_as_longlong(f);
       if (ok && (fb << 1) != 0) {  // f = +-0 keeps t
-        const bool s1 = B.edge_f[2 * e] >= 0.0;
+        const bool s1 = GROUPED ? (rec.ns >> 31) != 0 : B.edge_f[2 * e] >= 0.0;
         double lo = 0.0, hi = 1.0;
         if ((fb >= 0) == s1) lo = t; else hi = t;
-        tn = fma(-f, (double)(1.0f / rec.gp), t);
+        const float ig = 1.0f / rec.gp;
+        // grouped records carry g'' signed: its term takes the step's error
+        // from second to third order
+        tn = fma(-f, (double)(GROUPED ? ig * fmaf(0.5f * (float)f * ig, rec.gpp * ig, 1.0f) : ig), t);
         ok = tn > lo && tn < hi;
         if (ok) {
           const float step = fabsf((float)(tn - t));
           ok = step <= tolf || step <= 1e-7f || hi - lo <= 9.094947017729282e-13 ||
                (step <= (fast ? 1e-3f : 1e-5f) &&
-                rec.gpp * step * step <= (fast ? 1e-7f : 5e-11f) * fabsf(rec.gp));
+                fabsf(rec.gpp) * step * step <= (fast ? 1e-7f : 5e-11f) * fabsf(rec.gp));
         }
       }
       if (ok) {
-        // x1 and dir as k_roots_prep computed them (row e - e0)
-        const double *row64 = B.defer_x + (e - e0) * 2 * (uint64_t)d;
+        // x1 and dir as k_roots_x or k_roots_prep left them
+        const double *row64 = B.defer_x + (GROUPED ? i : e - e0) * 2 * (uint64_t)d;
         B.edge_t[e] = tn;
 #pragma unroll
         for (int k = 0; k < D; k++)
@@ -2324,8 +2267,9 @@ void mf_launch_eval_vertices_mixed(const MfFrame &F, const MfRbfDev &R, const Mf
 
 template <int DD, int MINB>
 static void launch_roots_d(const MfFrame &F, const MfRbfDev &R, const MfTraceBufs &B,
-                           uint64_t n_edges, double tol, int grid, int group, int fast, int sms,
-                           cudaStream_t st) {
+                           uint64_t n_edges, double tol, int grid, int group, MfRootMode mode,
+                           int sms, cudaStream_t st) {
+  const int fast = mode.fast ? 1 : 0;
   const int dyn = group > 1 ? ROOT_WARPS * GROUP_CAP * (int)sizeof(int) : 0;
   if (dyn) cudaFuncSetAttribute(k_roots_f64<DD, MINB>, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn);
   if (!B.defer_rec || B.defer_cap == 0) {
@@ -2333,20 +2277,29 @@ static void launch_roots_d(const MfFrame &F, const MfRbfDev &R, const MfTraceBuf
                                                              0, nullptr, nullptr);
     return;
   }
-  // chunks of defer_cap edges: the warp kernel (deferring the common
+  // chunks of defer_cap edges: the FP32 stage (per base vertex where the
+  // vertices have lists; else the warp kernel, deferring the common
   // single-step case), the lane-per-edge FP64 steps, then the redo queue
+  const bool grouped = mode.grouped && B.vlist && B.vert_edges;
   const size_t off_defer = offsetof(MfCounters, n_defer);
   const size_t span = offsetof(MfCounters, n_redo) + sizeof(unsigned long long) - off_defer;
   for (uint64_t e0 = 0; e0 < n_edges; e0 += B.defer_cap) {
     const uint64_t n = n_edges - e0 < B.defer_cap ? n_edges - e0 : B.defer_cap;
     const unsigned nb = (unsigned)((n + 255) / 256);
     cudaMemsetAsync((char *)B.cnt + off_defer, 0, span, st);
-    k_roots_prep<DD><<<nb, 256, 0, st>>>(F, B, e0, n);
-    k_roots_f64<DD, MINB><<<grid, ROOT_WARPS * 32, dyn, st>>>(F, R, B, e0, n, tol, group, fast, 1,
-                                                             nullptr, nullptr);
-    k_roots_x<DD><<<nb, 256, 0, st>>>(F, B, B.defer_cap, e0);
-    k_roots_terms<DD><<<sms * 16, 256, 0, st>>>(R, B, B.defer_cap);
-    k_roots_finish<DD><<<nb, 256, 0, st>>>(F, R, B, B.defer_cap, tol, fast, e0);
+    if (grouped) {
+      mf_launch_roots_grouped(F, R, B, e0, n, fast != 0, sms, st);
+      k_roots_x<DD, true><<<nb, 256, 0, st>>>(F, B, B.defer_cap, e0);
+      k_roots_terms<DD><<<sms * 16, 256, 0, st>>>(R, B, B.defer_cap);
+      k_roots_finish<DD, true><<<nb, 256, 0, st>>>(F, R, B, B.defer_cap, tol, fast, e0);
+    } else {
+      k_roots_prep<DD><<<nb, 256, 0, st>>>(F, B, e0, n);
+      k_roots_f64<DD, MINB><<<grid, ROOT_WARPS * 32, dyn, st>>>(F, R, B, e0, n, tol, group, fast, 1,
+                                                               nullptr, nullptr);
+      k_roots_x<DD, false><<<nb, 256, 0, st>>>(F, B, B.defer_cap, e0);
+      k_roots_terms<DD><<<sms * 16, 256, 0, st>>>(R, B, B.defer_cap);
+      k_roots_finish<DD, false><<<nb, 256, 0, st>>>(F, R, B, B.defer_cap, tol, fast, e0);
+    }
     k_roots_f64<DD, MINB><<<sms * 4, ROOT_WARPS * 32, 0, st>>>(F, R, B, 0, B.defer_cap, tol, 1,
                                                               fast, 0, B.redo, &B.cnt->n_redo);
   }
@@ -2354,22 +2307,22 @@ static void launch_roots_d(const MfFrame &F, const MfRbfDev &R, const MfTraceBuf
 
 template <int MINB>
 static void launch_roots(const MfFrame &F, const MfRbfDev &R, const MfTraceBufs &B, uint64_t n_edges,
-                         double tol, int grid, int group, int fast, int sms, cudaStream_t st) {
+                         double tol, int grid, int group, MfRootMode mode, int sms, cudaStream_t st) {
   switch (F.d) {
 #define MF_CASE(DD) \
-  case DD: launch_roots_d<DD, MINB>(F, R, B, n_edges, tol, grid, group, fast, sms, st); break;
+  case DD: launch_roots_d<DD, MINB>(F, R, B, n_edges, tol, grid, group, mode, sms, st); break;
     MF_CASE(2) MF_CASE(3) MF_CASE(4) MF_CASE(5) MF_CASE(6) MF_CASE(7)
 #undef MF_CASE
-    default: launch_roots_d<MF_MAXD, MINB>(F, R, B, n_edges, tol, grid, group, fast, sms, st);
+    default: launch_roots_d<MF_MAXD, MINB>(F, R, B, n_edges, tol, grid, group, mode, sms, st);
   }
 }
 
 void mf_launch_roots_f64(const MfFrame &F, const MfRbfDev &R, const MfTraceBufs &B, uint64_t n_edges,
-                         double tol, const MfTune &T, int sms, cudaStream_t st, bool fast) {
+                         double tol, const MfTune &T, int sms, cudaStream_t st, MfRootMode mode) {
   if (n_edges == 0) return;
   const int grid = sms * T.roots_bps;
-  if (T.roots_variant == 1) launch_roots<3>(F, R, B, n_edges, tol, grid, T.roots_group, fast, sms, st);
-  else launch_roots<2>(F, R, B, n_edges, tol, grid, T.roots_group, fast, sms, st);
+  if (T.roots_variant == 1) launch_roots<3>(F, R, B, n_edges, tol, grid, T.roots_group, mode, sms, st);
+  else launch_roots<2>(F, R, B, n_edges, tol, grid, T.roots_group, mode, sms, st);
 }
 
 // ---------------------------------------------------------------------------

@@ -58,6 +58,7 @@ struct MfCounters {
   unsigned long long root_overflow;  // edges whose screen lists overflowed (full re-evaluation)
   unsigned long long n_defer;      // root steps handed to the lane-per-edge FP64 kernel
   unsigned long long n_defer_list; // their strong-term list entries
+  unsigned long long n_groups[3];  // base vertices with edges in the chunk, by list length (mf_roots.cu)
   unsigned long long n_redo;       // deferred steps not accepted (solved again in full)
   unsigned long long n_items;      // expand items given a vertex slot
   // the search's current step: edges [lv_begin, lv_begin + lv_n) of the level
@@ -111,6 +112,7 @@ struct MfTraceBufs {
   int32_t *vlist;       // pool of vector indices
   uint64_t *vlist_off;  // [MV] offset of vertex i's list in the pool
   uint32_t *vlist_n;    // [MV] its length, MF_NO_LIST when it has none
+  uint32_t *vert_edges; // [MV] root solve: each vertex's edges in the chunk, then their offset
   uint64_t vlist_cap;   // pool capacity (entries)
   float list_r2;
   // Deferred FP64 root steps of one chunk of edges (NULL: none): records of
@@ -670,11 +672,23 @@ void mf_launch_eval_vertices_f64(const MfFrame &F, const MfRbfDev &R, const MfTr
 void mf_launch_eval_vertices_mixed(const MfFrame &F, const MfRbfDev &R, const MfTraceBufs &B,
                                    int precision, double band, const MfTune &T, int sms,
                                    cudaStream_t st, bool advance = true);
-// fast: the mixed paths' root accuracy (|dt| <= 1e-6 instead of 1e-9), with
-// fewer terms in the FP64 step.
+// How the roots of a trace are solved: fast, the mixed paths' accuracy (|dt| <=
+// 1e-6 instead of 1e-9), with fewer terms in the FP64 step; grouped by base
+// vertex where the vertices have lists.  MF_MIXED_FP32 at the mixed accuracy
+// stays with the per-edge kernel: both solve to 1e-6, but an edge whose last
+// FP32 step lies near the stopping rule can stop one step apart in the two
+// (5e-8 in t), and that path's results repeat from run to run, so they stay
+// what they were.
+struct MfRootMode {
+  bool fast, grouped;
+};
+static inline MfRootMode mf_root_mode(int precision, uint32_t flags) {
+  const bool fast = precision != MF_FP64 && !(flags & MF_ROOTS_FP64_EXACT);
+  return {fast, !(fast && precision == MF_MIXED_FP32)};
+}
 void mf_launch_roots_f64(const MfFrame &F, const MfRbfDev &R, const MfTraceBufs &B,
                          uint64_t n_edges, double tol, const MfTune &T, int sms, cudaStream_t st,
-                         bool fast = false);
+                         MfRootMode mode);
 void mf_launch_eval_vertices_tc(const MfFrame &F, const MfRbfDev &R, const MfTraceBufs &B,
                                 double band, int n_chunk, int sms, cudaStream_t st);
 

@@ -321,7 +321,7 @@ extern "C" int mf_trace_noalloc(const mf_rbf *rbf, const mf_domain *dom, const m
   const uint64_t E = fe;
   if (opts->flags & MF_WANT_ROOTS)
     mf_launch_roots_f64(F, R, B, E, opts->root_tol > 0 ? opts->root_tol : 1e-12, MfTune(), sms,
-                        st, mixed && !(opts->flags & MF_ROOTS_FP64_EXACT));
+                        st, mf_root_mode(opts->precision, opts->flags));
   int64_t n_cells = 0, n_cell_edges = 0;
   if ((opts->flags & MF_WANT_CELLS) && E > 0) {
     // mf_trace's cell rule: the enumeration writes each cell's sign mask and

@@ -278,8 +278,7 @@ extern "C" int mf_subdiv_next(mf_ctx *ctx, mf_trace_out *out, int64_t *cells_lef
   const uint64_t E = ctx->h_counters->n_edges;
   if (S.flags & MF_WANT_ROOTS) {
     MfProfScope ps(ctx, MF_PH_ROOTS, st, E > 0 ? 1 : 0, (int64_t)E);
-    mf_launch_roots_f64(F, S.R, B, E, S.tol, ctx->tune, sms, st,
-                        mixed && !(S.flags & MF_ROOTS_FP64_EXACT));
+    mf_launch_roots_f64(F, S.R, B, E, S.tol, ctx->tune, sms, st, mf_root_mode(S.precision, S.flags));
   }
   rc = mf_read_counters(ctx, B, st);
   if (rc) return rc;

@@ -1647,13 +1647,14 @@ static int setup_buffers(mf_ctx *ctx, int d, uint64_t ME, uint64_t MV, uint64_t 
   if (n_sv > 0) {
     const uint64_t per = (uint64_t)std::min(n_sv, 192);
     const uint64_t cap = MV * per;
-    const size_t lb = al(TV * 4) + al(MV * 8) + al(MV * 4) + al(cap * 4);
+    const size_t lb = al(TV * 4) + al(MV * 8) + 2 * al(MV * 4) + al(cap * 4);
     std::string keep = ctx->err;
     char *l = (char *)mf_ctx_buffer(ctx, MF_SLOT_VLIST, lb);
     if (l) {
       B->vtab_idx = (uint32_t *)l; l += al(TV * 4);
       B->vlist_off = (uint64_t *)l; l += al(MV * 8);
       B->vlist_n = (uint32_t *)l; l += al(MV * 4);
+      B->vert_edges = (uint32_t *)l; l += al(MV * 4);
       B->vlist = (int32_t *)l;
       B->vlist_cap = cap;
     } else {
@@ -1859,7 +1860,7 @@ extern "C" int mf_trace(mf_ctx *ctx, const mf_rbf *rbf, const mf_domain *dom,
   if (opts->flags & MF_WANT_ROOTS) {
     MfProfScope ps(ctx, MF_PH_ROOTS, st, E > 0 ? 1 : 0, (int64_t)E);
     mf_launch_roots_f64(F, R, B, E, tol, ctx->tune, sms, st,
-                        mixed && !(opts->flags & MF_ROOTS_FP64_EXACT));
+                        mf_root_mode(opts->precision, opts->flags));
   }
 
   // Cells (Sec. IV-C) and the cell -> edge CSR.

@@ -156,7 +156,7 @@ extern "C" int mf_autotune(mf_ctx *ctx, const mf_rbf *rbf, const mf_domain *dom,
           const float ms = time_ms(
               st, [&]() {
                 mf_launch_roots_f64(L.F, L.R, L.B, es, L.tol, t, sms, st,
-                                    L.precision != MF_FP64 && !(L.flags & MF_ROOTS_FP64_EXACT));
+                                    mf_root_mode(L.precision, L.flags));
               }, 3);
           n_cand++;
           if (ms < best_roots) {
