@@ -134,6 +134,14 @@ void *mf_ctx_buffer(mf_ctx *c, int slot, size_t bytes) {
   bytes = (bytes + 255) & ~(size_t)255;
   if (bytes == 0) bytes = 256;
   if (c->slot_bytes[slot] >= bytes) return c->slot_ptr[slot];
+  if (slot != MF_SLOT_BATCHROOTS && c->slot_ptr[MF_SLOT_BATCHROOTS] &&
+      c->total - c->slot_bytes[slot] + bytes > c->budget) {
+    cudaDeviceSynchronize();
+    cudaFree(c->slot_ptr[MF_SLOT_BATCHROOTS]);
+    c->slot_ptr[MF_SLOT_BATCHROOTS] = nullptr;
+    c->total -= c->slot_bytes[MF_SLOT_BATCHROOTS];
+    c->slot_bytes[MF_SLOT_BATCHROOTS] = 0;
+  }
   size_t others = c->total - c->slot_bytes[slot];
   if (others + bytes > c->budget) {
     mf_set_error(c, MF_ERR_OOM, "HBM budget: need %zu more bytes (budget %zu, held %zu)",

@@ -9,6 +9,7 @@
 // each kernel: a trace id comes from a prefix over the slots, so uneven
 // traces (different d, support vectors, lambda, precision) fill the GPU
 // together.  Roots, cells and the CSR then run batched the same way.
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <vector>
@@ -228,6 +229,68 @@ int mf_finish_trace(mf_ctx *ctx, const mf_rbf *rbf, const mf_trace_opts *o, cons
   return MF_OK;
 }
 
+// Roots of the slots in `which` (edges[t]: slot t's traced edges).  A slot of
+// ROOTS_ALONE edges or more whose roots can be grouped goes through the single
+// trace's root solve (grouped by base vertex, its strong terms in
+// double-float): 9 launches, some 25 us, against the 2 to 4 ns per edge that
+// the batched warp-per-edge kernel costs more, so the line lies near 8192.
+// Eight BF16 traces of 87,000 to 1,049,000 edges: 72.1 -> 59.6 ms; four served
+// d = 4 FP64 traces: 16.5 -> 15.7 ms.  The rest share one launch of the batched
+// kernel per dimension, as do all slots when the pools don't fit the budget.
+// d_only: device words for the mask, n of them; the mask is kept in `mask`
+// until the stream has been waited for.
+#define ROOTS_ALONE 8192
+static void launch_slot_roots(mf_ctx *ctx, const std::vector<MfSlot> &slots, const MfSlot *d_slots,
+                              MfBatchPlan *d_plan, const std::vector<int> &which,
+                              const std::vector<unsigned long long> &edges, int32_t *d_only,
+                              std::vector<int32_t> &mask, int sms, cudaStream_t st) {
+  uint64_t most = 0, verts = 0;
+  int dmax = 0;
+  auto large = [&](int t) {
+    return slots[t].B.vlist && edges[t] >= ROOTS_ALONE &&
+           mf_root_mode(slots[t].precision, slots[t].flags).grouped;
+  };
+  for (int t : which) {
+    if (!(slots[t].flags & MF_WANT_ROOTS) || !large(t)) continue;
+    most = std::max<uint64_t>(most, edges[t]);
+    verts = std::max<uint64_t>(verts, slots[t].B.max_vertices);
+    dmax = std::max(dmax, slots[t].F.d);
+  }
+  MfTraceBufs pools;
+  memset(&pools, 0, sizeof(pools));
+  const bool alone = most > 0 && mf_setup_root_pools(ctx, MF_SLOT_BATCHROOTS, dmax,
+                                                     std::min<uint64_t>(most, 1ull << 22), verts, &pools);
+  mask.assign(slots.size(), 0);
+  uint32_t dims = 0;
+  for (int t : which) {
+    const MfSlot &S = slots[t];
+    if (!(S.flags & MF_WANT_ROOTS) || edges[t] == 0) continue;
+    if (!alone || !large(t)) {
+      mask[t] = 1;
+      dims |= 1u << S.F.d;
+      continue;
+    }
+    MfTraceBufs B = S.B;
+    B.defer_rec = pools.defer_rec;
+    B.redo = pools.redo;
+    B.defer_list = pools.defer_list;
+    B.ep32 = pools.ep32;
+    B.defer_x = pools.defer_x;
+    B.defer_x3 = pools.defer_x3;
+    B.defer_part = pools.defer_part;
+    B.defer_bnd = pools.defer_bnd;
+    B.defer_chunk = pools.defer_chunk;
+    B.defer_cap = pools.defer_cap;
+    B.defer_list_cap = pools.defer_list_cap;
+    B.vert_edges = pools.vert_edges;
+    mf_launch_roots_f64(S.F, S.R, B, edges[t], S.root_tol, MfTune(), sms, st,
+                        mf_root_mode(S.precision, S.flags));
+  }
+  if (!dims) return;
+  cudaMemcpyAsync(d_only, mask.data(), sizeof(int32_t) * mask.size(), cudaMemcpyHostToDevice, st);
+  mf_b_launch_roots(d_slots, d_plan, (int)slots.size(), d_only, dims, ctx->tune.roots_group, sms, st);
+}
+
 extern "C" int mf_trace_batch(mf_ctx *ctx, int32_t n, const mf_rbf *rbfs, const mf_domain *doms,
                               const mf_trace_opts *opts, const double *const *seeds,
                               const int64_t *n_seeds, mf_trace_out *outs, void *stream) {
@@ -252,6 +315,7 @@ extern "C" int mf_trace_batch(mf_ctx *ctx, int32_t n, const mf_rbf *rbfs, const 
   const size_t off_slots = bump.take(sizeof(MfSlot) * n);
   const size_t off_state = bump.take(sizeof(MfSlotState) * n);
   const size_t off_plan = bump.take(sizeof(MfBatchPlan));
+  const size_t off_only = bump.take(sizeof(int32_t) * n);
   char *arena = (char *)mf_ctx_buffer(ctx, MF_SLOT_BATCH, bump.off);
   if (!arena) return MF_ERR_OOM;
   MfSlot *d_slots = (MfSlot *)(arena + off_slots);
@@ -327,9 +391,17 @@ extern "C" int mf_trace_batch(mf_ctx *ctx, int32_t n, const mf_rbf *rbfs, const 
   // --- roots and cells of all traces
   uint32_t dims = 0;
   for (int t = 0; t < n; t++) dims |= 1u << slots[t].F.d;
+  std::vector<unsigned long long> n_edges(n);
+  std::vector<int32_t> root_mask;
   {
     MfProfScope ps(ctx, MF_PH_ROOTS, st, 2);
-    mf_b_launch_roots(d_slots, d_plan, n, nullptr, dims, ctx->tune.roots_group, sms, st);
+    std::vector<int> all(n);
+    for (int t = 0; t < n; t++) {
+      all[t] = t;
+      n_edges[t] = hs[t].level_end;
+    }
+    launch_slot_roots(ctx, slots, d_slots, d_plan, all, n_edges, (int32_t *)(arena + off_only),
+                      root_mask, sms, st);
   }
   bool any_cells = false;
   for (int t = 0; t < n; t++) any_cells = any_cells || (opts[t].flags & MF_WANT_CELLS);
@@ -785,10 +857,16 @@ extern "C" int mf_server_step(mf_server *s, void *stream, int32_t *n_running, in
     fin.push_back(t);
   }
   if (!fin.empty()) {
-    cudaMemcpyAsync(s->d_only, only.data(), sizeof(int32_t) * n, cudaMemcpyHostToDevice, st);
     uint32_t dims = 0;
-    for (int t : fin) dims |= 1u << s->slots[t].F.d;
-    mf_b_launch_roots(s->d_slots, s->d_plan, n, s->d_only, dims, ctx->tune.roots_group, sms, st);
+    std::vector<unsigned long long> n_edges(n, 0);
+    for (int t : fin) {
+      dims |= 1u << s->slots[t].F.d;
+      n_edges[t] = s->hstate[t].level_end;
+    }
+    std::vector<int32_t> root_mask;
+    launch_slot_roots(ctx, s->slots, s->d_slots, s->d_plan, fin, n_edges, s->d_only, root_mask, sms,
+                      st);
+    cudaMemcpyAsync(s->d_only, only.data(), sizeof(int32_t) * n, cudaMemcpyHostToDevice, st);
     bool cells = false;
     for (int t : fin) cells = cells || (s->slots[t].flags & MF_WANT_CELLS);
     if (cells) {

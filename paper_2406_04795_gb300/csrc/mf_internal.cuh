@@ -689,6 +689,10 @@ static inline MfRootMode mf_root_mode(int precision, uint32_t flags) {
 void mf_launch_roots_f64(const MfFrame &F, const MfRbfDev &R, const MfTraceBufs &B,
                          uint64_t n_edges, double tol, const MfTune &T, int sms, cudaStream_t st,
                          MfRootMode mode);
+// The pools of its deferred steps in context slot `slot`; false when the budget
+// refuses.
+bool mf_setup_root_pools(mf_ctx *ctx, int slot, int d, uint64_t chunk, uint64_t n_vert,
+                         MfTraceBufs *B);
 void mf_launch_eval_vertices_tc(const MfFrame &F, const MfRbfDev &R, const MfTraceBufs &B,
                                 double band, int n_chunk, int sms, cudaStream_t st);
 
@@ -712,7 +716,10 @@ enum {
   MF_SLOT_SORT = 15,
   MF_SLOT_DEFER = 16,
   MF_SLOT_ITEMS = 17,
-  MF_NUM_SLOTS = 18
+  // the batch's and the server's root pools: no pointer into them outlives a
+  // call, so mf_ctx_buffer gives them back when another slot needs the budget
+  MF_SLOT_BATCHROOTS = 18,
+  MF_NUM_SLOTS = 19
 };
 
 // ---------------------------------------------------------------------------

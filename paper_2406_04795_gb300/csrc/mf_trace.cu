@@ -1577,6 +1577,38 @@ static int read_counters(mf_ctx *ctx, const MfTraceBufs &B, cudaStream_t st) {
   return MF_OK;
 }
 
+// Deferred FP64 root steps: chunks of up to dc edges, ~48 strong entries each
+// on average (when the budget allows; else every step runs in the
+// warp-per-edge kernel), and n_vert words for B->vert_edges where the trace
+// has none of its own.
+bool mf_setup_root_pools(mf_ctx *ctx, int slot, int d, uint64_t dc, uint64_t n_vert,
+                         MfTraceBufs *B) {
+  auto al = [](size_t x) { return (x + 255) & ~(size_t)255; };
+  const uint64_t dl = dc * 48;
+  const size_t db = al(dc * 32) + al(dc * 8) + al(dl * 4) + al(dc * MF_EP_ROW(d) * 4) +
+                    al(dc * 2 * d * 8) + al(dc * 3 * d * 4) + al(dl) + al(dl / 2) + al(dl / 2) +
+                    al(n_vert * 4);
+  const std::string keep = ctx->err;
+  char *q = (char *)mf_ctx_buffer(ctx, slot, db);
+  if (!q) {
+    ctx->err = keep;
+    return false;
+  }
+  B->defer_rec = q; q += al(dc * 32);
+  B->redo = (uint64_t *)q; q += al(dc * 8);
+  B->defer_list = (int32_t *)q; q += al(dl * 4);
+  B->ep32 = (float *)q; q += al(dc * MF_EP_ROW(d) * 4);
+  B->defer_x = (double *)q; q += al(dc * 2 * d * 8);
+  B->defer_x3 = (float *)q; q += al(dc * 3 * d * 4);
+  B->defer_part = (double *)q; q += al(dl);  // dl / 8 doubles
+  B->defer_bnd = (float *)q; q += al(dl / 2);  // dl / 8 floats
+  B->defer_chunk = (uint32_t *)q; q += al(dl / 2);  // dl / 8 uint32
+  if (n_vert) B->vert_edges = (uint32_t *)q;
+  B->defer_cap = dc;
+  B->defer_list_cap = dl;
+  return true;
+}
+
 // Carves the trace's buffers from the context slots.
 static int setup_buffers(mf_ctx *ctx, int d, uint64_t ME, uint64_t MV, uint64_t MC, bool mixed,
                          int n_sv, MfTraceBufs *B) {
@@ -1617,31 +1649,7 @@ static int setup_buffers(mf_ctx *ctx, int d, uint64_t ME, uint64_t MV, uint64_t 
   B->max_cells = MC;
   B->cnt = (MfCounters *)mf_ctx_buffer(ctx, MF_SLOT_COUNTERS, sizeof(MfCounters));
   if (!B->cnt) return MF_ERR_OOM;
-  // deferred FP64 root steps: chunks of up to 4M edges, ~48 strong entries
-  // each on average (when the budget allows; else every step runs in the
-  // warp-per-edge kernel)
-  {
-    const uint64_t dc = std::min<uint64_t>(ME, 1ull << 22), dl = dc * 48;
-    const size_t db = al(dc * 32) + al(dc * 8) + al(dl * 4) + al(dc * MF_EP_ROW(d) * 4) +
-                      al(dc * 2 * d * 8) + al(dc * 3 * d * 4) + al(dl) + al(dl / 2) + al(dl / 2);
-    std::string keep = ctx->err;
-    char *q = (char *)mf_ctx_buffer(ctx, MF_SLOT_DEFER, db);
-    if (q) {
-      B->defer_rec = q; q += al(dc * 32);
-      B->redo = (uint64_t *)q; q += al(dc * 8);
-      B->defer_list = (int32_t *)q; q += al(dl * 4);
-      B->ep32 = (float *)q; q += al(dc * MF_EP_ROW(d) * 4);
-      B->defer_x = (double *)q; q += al(dc * 2 * d * 8);
-      B->defer_x3 = (float *)q; q += al(dc * 3 * d * 4);
-      B->defer_part = (double *)q; q += al(dl);  // dl / 8 doubles
-      B->defer_bnd = (float *)q; q += al(dl / 2);  // dl / 8 floats
-      B->defer_chunk = (uint32_t *)q;              // dl / 8 uint32
-      B->defer_cap = dc;
-      B->defer_list_cap = dl;
-    } else {
-      ctx->err = keep;
-    }
-  }
+  mf_setup_root_pools(ctx, MF_SLOT_DEFER, d, std::min<uint64_t>(ME, 1ull << 22), 0, B);
   // per-vertex lists for the root screen, when they fit the budget (else
   // the root screen scans the vector blocks)
   if (n_sv > 0) {
