@@ -351,6 +351,7 @@ __device__ __forceinline__ void cert_sincos(double x, const double2 *tab, double
 // along because the cell pass is bound by its gathers: a separate byte per
 // point costs each row entry a second 32-byte sector.
 __host__ __device__ __forceinline__ int cert_rec_stride(int d) { return (d + 2 + 3) & ~3; }
+#define CERT_REC(D) (((D) + 2 + 3) & ~3)  // cert_rec_stride at compile time
 __device__ __forceinline__ float cert_rec_word(int element, bool verdict) {
   return __int_as_float((element & 0xffff) | (verdict ? 0x10000 : 0));
 }
@@ -1236,77 +1237,80 @@ static void lipschitz_table(int NL, const std::vector<double> &dh, bool caps, in
 // (certified) or every point has slack_j + eps_j < 0 (not certified);
 // otherwise it is recomputed in FP64 from the points and margins as
 // k_certify_cells_whole does.
-// Rows of up to CERT_ROW_CACHE points are read once (the records stay in
-// registers for the second pass); longer rows read the rest twice.
-#define CERT_ROW_CACHE 9
+// Bound by the gathers of the records: CERT_ROWS of them are in flight per
+// thread, each one 32-byte load; only the cells whose points are all in
+// collision read them a second time, for the test.  (Keeping a row's records in
+// registers for the test left room for few warps and fewer loads in flight.)
+// Cells of a d = 5 proof at lambda = 0.08: 5.3 -> 2.3 ms, at 0.15: 1.0 -> 0.48;
+// of a d = 6 proof: 3.0 -> 1.1 ms.
+#define CERT_ROWS 4
 
 // Range of the cell's points (lo, hi per coordinate, P = largest |p|) from
 // one FP32 record (NV4 float4 units).
-template <int NV4>
-__device__ __forceinline__ void cert_rec_extend(const float4 (&v)[NV4], int d, float (&lo)[MF_MAXD],
-                                                float (&hi)[MF_MAXD], float &P) {
+template <int D>
+__device__ __forceinline__ void cert_rec_extend(const float (&v)[CERT_REC(D)], float (&lo)[D],
+                                                float (&hi)[D], float &P) {
 #pragma unroll
-  for (int q = 0; q < NV4; q++) {
-    const float vv[4] = {v[q].x, v[q].y, v[q].z, v[q].w};
+  for (int k = 0; k < D; k++) {
+    lo[k] = fminf(lo[k], v[k]);
+    hi[k] = fmaxf(hi[k], v[k]);
+    P = fmaxf(P, fabsf(v[k]));
+  }
+}
+
+// Record i where `in` (else zeros), in one 32-byte load where it has that size
+// (d = 3 .. 6; the records are then 32-byte aligned), else in 16-byte ones.  No
+// branch, so that the loads of several rows are in flight together.
+template <int D>
+__device__ __forceinline__ void cert_rec_load(const float *rec32, int64_t i, bool in,
+                                              float (&v)[CERT_REC(D)]) {
+  const float *p = rec32 + i * CERT_REC(D);
 #pragma unroll
-    for (int h = 0; h < 4; h++) {
-      const int k = 4 * q + h;
-      if (k < MF_MAXD && k < d) {
-        lo[k] = fminf(lo[k], vv[h]);
-        hi[k] = fmaxf(hi[k], vv[h]);
-        P = fmaxf(P, fabsf(vv[h]));
-      }
+  for (int k = 0; k < CERT_REC(D); k++) v[k] = 0.f;
+  if (CERT_REC(D) == 8) {
+    constexpr int H = CERT_REC(D) > 4 ? 4 : 0;
+    asm("{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %9, 0;\n\t"
+        "@p ld.global.nc.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];\n\t}"
+        : "+f"(v[0]), "+f"(v[1]), "+f"(v[2]), "+f"(v[3]), "+f"(v[H]), "+f"(v[H + 1]), "+f"(v[H + 2]),
+          "+f"(v[H + 3])
+        : "l"(p), "r"((int)in));
+  } else {
+#pragma unroll
+    for (int q = 0; q < CERT_REC(D) / 4; q++) {
+      const float4 t =
+          in ? __ldg(reinterpret_cast<const float4 *>(p) + q) : make_float4(0.f, 0.f, 0.f, 0.f);
+      v[4 * q] = t.x;
+      v[4 * q + 1] = t.y;
+      v[4 * q + 2] = t.z;
+      v[4 * q + 3] = t.w;
     }
   }
 }
 
 // The verdict of a point's record.
-template <int NV4>
-__device__ __forceinline__ uint32_t cert_rec_verdict(const float4 (&v)[NV4], int d) {
-  uint32_t w = 0;
-#pragma unroll
-  for (int q = 0; q < NV4; q++) {
-    const float vv[4] = {v[q].x, v[q].y, v[q].z, v[q].w};
-#pragma unroll
-    for (int h = 0; h < 4; h++)
-      if (4 * q + h == d + 1) w = (uint32_t)__float_as_int(vv[h]);
-  }
-  return (w >> 16) & 1u;
+template <int D>
+__device__ __forceinline__ uint32_t cert_rec_verdict(const float (&v)[CERT_REC(D)]) {
+  return ((uint32_t)__float_as_int(v[D + 1]) >> 16) & 1u;
 }
 
 // One point's FP32 slack test (see above): sets yes when it certifies the
-// cell, undecided when its error bound straddles the decision.
-template <int NV4>
-__device__ __forceinline__ void cert_rec_test(const float4 (&v)[NV4], int d, int NE,
-                                              const float (&lo)[MF_MAXD], const float (&hi)[MF_MAXD],
-                                              float P, const float *L32, bool &yes, bool &undecided) {
-  float m = 0.f;
-  int e = -1;
-#pragma unroll
-  for (int q = 0; q < NV4; q++) {
-    const float vv[4] = {v[q].x, v[q].y, v[q].z, v[q].w};
-#pragma unroll
-    for (int h = 0; h < 4; h++) {
-      if (4 * q + h == d) m = vv[h];
-      if (4 * q + h == d + 1) e = (int16_t)(__float_as_int(vv[h]) & 0xffff);
-    }
-  }
+// cell, undecided when its error bound straddles the decision.  sL: the
+// Lipschitz table in shared memory.
+template <int D>
+__device__ __forceinline__ void cert_rec_test(const float (&v)[CERT_REC(D)], int NE,
+                                              const float (&lo)[D], const float (&hi)[D], float P,
+                                              const float *sL, bool &yes, bool &undecided) {
+  const float m = v[D];
+  const int e = (int16_t)(__float_as_int(v[D + 1]) & 0xffff);
   if (e < 0 || e >= NE) return;
   const float u = 5.9604644775390625e-08f;
   float drop = 0.f, lsum = 0.f;
 #pragma unroll
-  for (int q = 0; q < NV4; q++) {
-    const float vv[4] = {v[q].x, v[q].y, v[q].z, v[q].w};
-#pragma unroll
-    for (int h = 0; h < 4; h++) {
-      const int k = 4 * q + h;
-      if (k < MF_MAXD && k < d) {
-        const float sp = fmaxf(hi[k] - vv[h], vv[h] - lo[k]);
-        const float Lk = __ldg(L32 + e * d + k);
-        drop = fmaf(Lk, sp, drop);
-        lsum = fmaf(Lk, fmaf((float)(d + 4), sp, 2.f * P), lsum);
-      }
-    }
+  for (int k = 0; k < D; k++) {
+    const float sp = fmaxf(hi[k] - v[k], v[k] - lo[k]);
+    const float Lk = sL[e * D + k];
+    drop = fmaf(Lk, sp, drop);
+    lsum = fmaf(Lk, fmaf((float)(D + 4), sp, 2.f * P), lsum);
   }
   const float sl = m - drop;
   const float eps = 2.f * u * (2.f * fabsf(m) + lsum) + 1e-30f;
@@ -1315,75 +1319,70 @@ __device__ __forceinline__ void cert_rec_test(const float4 (&v)[NV4], int d, int
   else if (sl + eps >= (float)CERT_ELEM_TIE) undecided = true;
 }
 
-template <int NV4>
+template <int D>
 __global__ void __launch_bounds__(256, 3) k_certify_cells_whole32(
     const int64_t *off, const int64_t *idx, int64_t n_cells, const float *rec32, const double *pts,
-    int d, const double *margin, const int16_t *element, const float *L32, const double *L, int NE,
+    const double *margin, const int16_t *element, const float *L32, const double *L, int NE,
     int64_t n_points, uint8_t *whole, unsigned *bad, uint8_t *cell_verdict) {
+  __shared__ float sL[CERT_MAX_ELEM * D];
+  for (int i = threadIdx.x; i < NE * D; i += blockDim.x) sL[i] = L32[i];
+  __syncthreads();
   const int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (c >= n_cells) return;
   const int64_t j0 = off[c], j1 = off[c + 1];
-  const int64_t nr = j1 - j0;
   // with cell_verdict: also the AND of the points' verdicts (k_certify_cells)
   uint32_t all = 1;
-  const float4 *R4 = reinterpret_cast<const float4 *>(rec32);
-  float lo[MF_MAXD], hi[MF_MAXD];
+  float lo[D], hi[D];
 #pragma unroll
-  for (int k = 0; k < MF_MAXD; k++) {
+  for (int k = 0; k < D; k++) {
     lo[k] = INFINITY;
     hi[k] = -INFINITY;
   }
   float P = 0.f;
-  float4 cache[CERT_ROW_CACHE][NV4];
-  uint32_t valid = 0;
+  for (int64_t j = j0; j < j1; j += CERT_ROWS) {
+    int64_t i[CERT_ROWS];
+    float v[CERT_ROWS][CERT_REC(D)];
 #pragma unroll
-  for (int r = 0; r < CERT_ROW_CACHE; r++) {
-    const int64_t i = r < nr ? idx[j0 + r] : -1;
-    const bool in = i >= 0 && i < n_points;
-    if (r < nr && !in) {
-      atomicOr(bad, 1u);
-      all = 0;
-    }
+    for (int r = 0; r < CERT_ROWS; r++) i[r] = j + r < j1 ? idx[j + r] : -1;
 #pragma unroll
-    for (int q = 0; q < NV4; q++)
-      cache[r][q] = in ? __ldg(R4 + i * NV4 + q) : make_float4(0.f, 0.f, 0.f, 0.f);
-    if (in) {
-      all &= cert_rec_verdict<NV4>(cache[r], d);
-      cert_rec_extend<NV4>(cache[r], d, lo, hi, P);
-      valid |= 1u << r;
-    }
-  }
-  for (int64_t j = j0 + CERT_ROW_CACHE; j < j1; j++) {
-    const int64_t i = idx[j];
-    if (i < 0 || i >= n_points) {
-      atomicOr(bad, 1u);
-      all = 0;
-      continue;
-    }
-    float4 v[NV4];
+    for (int r = 0; r < CERT_ROWS; r++)
+      cert_rec_load<D>(rec32, i[r], i[r] >= 0 && i[r] < n_points, v[r]);
 #pragma unroll
-    for (int q = 0; q < NV4; q++) v[q] = __ldg(R4 + i * NV4 + q);
-    all &= cert_rec_verdict<NV4>(v, d);
-    cert_rec_extend<NV4>(v, d, lo, hi, P);
+    for (int r = 0; r < CERT_ROWS; r++) {
+      if (i[r] >= 0 && i[r] < n_points) {
+        all &= cert_rec_verdict<D>(v[r]);
+        cert_rec_extend<D>(v[r], lo, hi, P);
+      } else if (j + r < j1) {
+        atomicOr(bad, 1u);
+        all = 0;
+      }
+    }
   }
   if (cell_verdict) cell_verdict[c] = (uint8_t)all;
   bool yes = false, undecided = false;
+  // a certified piece is in collision throughout, its points included: a
+  // cell with a free point fails without the test (half to nine tenths of the
+  // cells of a traced manifold, and neighbours alike)
+  if (!all) {
+    whole[c] = 0;
+    return;
+  }
+  for (int64_t j = j0; j < j1 && !yes; j += CERT_ROWS) {
+    float v[CERT_ROWS][CERT_REC(D)];
 #pragma unroll
-  for (int r = 0; r < CERT_ROW_CACHE; r++)
-    if ((valid >> r) & 1u) cert_rec_test<NV4>(cache[r], d, NE, lo, hi, P, L32, yes, undecided);
-  for (int64_t j = j0 + CERT_ROW_CACHE; j < j1 && !yes; j++) {
-    const int64_t i = idx[j];
-    if (i < 0 || i >= n_points) continue;
-    float4 v[NV4];
+    for (int r = 0; r < CERT_ROWS; r++) {
+      const bool in = j + r < j1;  // every index of the row is valid here
+      cert_rec_load<D>(rec32, in ? idx[j + r] : 0, in, v[r]);
+    }
 #pragma unroll
-    for (int q = 0; q < NV4; q++) v[q] = __ldg(R4 + i * NV4 + q);
-    cert_rec_test<NV4>(v, d, NE, lo, hi, P, L32, yes, undecided);
+    for (int r = 0; r < CERT_ROWS; r++)
+      if (j + r < j1) cert_rec_test<D>(v[r], NE, lo, hi, P, sL, yes, undecided);
   }
   if (!yes && undecided) {
     // close to the decision: the exact FP64 certificate
-    double dlo[MF_MAXD], dhi[MF_MAXD];
+    double dlo[D], dhi[D];
 #pragma unroll
-    for (int k = 0; k < MF_MAXD; k++) {
+    for (int k = 0; k < D; k++) {
       dlo[k] = INFINITY;
       dhi[k] = -INFINITY;
     }
@@ -1391,12 +1390,10 @@ __global__ void __launch_bounds__(256, 3) k_certify_cells_whole32(
       const int64_t i = idx[j];
       if (i < 0 || i >= n_points) continue;
 #pragma unroll
-      for (int k = 0; k < MF_MAXD; k++) {
-        if (k < d) {
-          const double v = pts[i * d + k];
-          dlo[k] = fmin(dlo[k], v);
-          dhi[k] = fmax(dhi[k], v);
-        }
+      for (int k = 0; k < D; k++) {
+        const double v = pts[i * D + k];
+        dlo[k] = fmin(dlo[k], v);
+        dhi[k] = fmax(dhi[k], v);
       }
     }
     double slack = -INFINITY;
@@ -1407,11 +1404,9 @@ __global__ void __launch_bounds__(256, 3) k_certify_cells_whole32(
       if (e < 0 || e >= NE) continue;
       double drop = 0.0;
 #pragma unroll
-      for (int k = 0; k < MF_MAXD; k++) {
-        if (k < d) {
-          const double v = pts[i * d + k];
-          drop = fma(L[e * d + k], fmax(dhi[k] - v, v - dlo[k]), drop);
-        }
+      for (int k = 0; k < D; k++) {
+        const double v = pts[i * D + k];
+        drop = fma(L[e * D + k], fmax(dhi[k] - v, v - dlo[k]), drop);
       }
       slack = fmax(slack, (margin[i] - CERT_ELEM_TIE) - drop);
     }
@@ -1531,7 +1526,7 @@ extern "C" int mf_certify_ex(mf_ctx *ctx, const mf_robot *robot, const mf_scene 
   }
   // the FP32 whole-cell pass also forms the cell verdicts (one read of
   // each row)
-  const bool fused = fast && cert_rec_stride(d) / 4 <= 3;
+  const bool fused = fast;
   if (n_cells > 0 && out->cell_verdict && !fused) {
     MfProfScope ps(ctx, MF_PH_CERT_CELLS, st, 1, n_cells);
     k_certify_cells<<<(unsigned)((n_cells + 255) / 256), 256, 0, st>>>(
@@ -1540,19 +1535,19 @@ extern "C" int mf_certify_ex(mf_ctx *ctx, const mf_robot *robot, const mf_scene 
   if (whole) {
     MfProfScope ps(ctx, MF_PH_CERT_CELLS, st, 1, n_cells);
     const unsigned gc = (unsigned)((n_cells + 255) / 256);
-    const int nv4 = cert_rec_stride(d) / 4;
-    if (fast && nv4 == 1)
-      k_certify_cells_whole32<1><<<gc, 256, 0, st>>>(cell_off, cell_idx, n_cells, rec32, points, d,
-                                                      out->margin, elem, dL32, dL, NE, n_points,
-                                                      out->cell_whole, bad, out->cell_verdict);
-    else if (fast && nv4 == 2)
-      k_certify_cells_whole32<2><<<gc, 256, 0, st>>>(cell_off, cell_idx, n_cells, rec32, points, d,
-                                                      out->margin, elem, dL32, dL, NE, n_points,
-                                                      out->cell_whole, bad, out->cell_verdict);
-    else if (fast)
-      k_certify_cells_whole32<3><<<gc, 256, 0, st>>>(cell_off, cell_idx, n_cells, rec32, points, d,
-                                                      out->margin, elem, dL32, dL, NE, n_points,
-                                                      out->cell_whole, bad, out->cell_verdict);
+    if (fast) {
+      switch (d) {
+#define MF_CASE(DD)                                                                                   \
+  case DD:                                                                                            \
+    k_certify_cells_whole32<DD><<<gc, 256, 0, st>>>(cell_off, cell_idx, n_cells, rec32, points,       \
+                                                    out->margin, elem, dL32, dL, NE, n_points,        \
+                                                    out->cell_whole, bad, out->cell_verdict);         \
+    break;
+        MF_CASE(1) MF_CASE(2) MF_CASE(3) MF_CASE(4) MF_CASE(5) MF_CASE(6) MF_CASE(7) MF_CASE(8)
+#undef MF_CASE
+        default: break;
+      }
+    }
     else
       k_certify_cells_whole<<<(unsigned)((n_cells + 255) / 256), 256, 0, st>>>(
           cell_off, cell_idx, n_cells, points, d, out->margin, elem, dL, NE, n_points,
