@@ -292,15 +292,44 @@ __global__ void k_gather_cells(int d, MfTraceBufs B, const uint32_t *perm, uint6
   if (len) len[i] = B.cell_off[o + 1] - B.cell_off[o];
 }
 
-__global__ void k_gather_csr(MfTraceBufs B, const uint32_t *perm, const uint32_t *inv_e, uint64_t n,
-                             const int64_t *new_off, int64_t *idx) {
-  const uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const uint64_t o = perm[i];
-  const int64_t a = B.cell_off[o], b = B.cell_off[o + 1], at = new_off[i];
-  for (int64_t j = a; j < b; j++) {
-    const int64_t e = B.cell_idx[j];
-    idx[at + (j - a)] = e >= 0 ? (int64_t)inv_e[e] : -1;
+// The rows in the cells' new order with the edges' new indices.  A warp takes 32
+// cells, whose output is one contiguous range: lane per entry, so that the
+// stores are whole lines and the loads whole rows (a thread per cell stored
+// 8 bytes at a time, a row apart from its neighbours: 2.5 -> 2.0 ms for a d = 5
+// proof at lambda = 0.08, 1.26 -> 0.95 ms for a d = 6 proof).
+__global__ void __launch_bounds__(256) k_gather_csr(MfTraceBufs B, const uint32_t *perm,
+                                                    const uint32_t *inv_e, uint64_t n,
+                                                    const int64_t *new_off, int64_t *idx) {
+  __shared__ uint32_t s_end[8][32];
+  __shared__ int64_t s_src[8][32];  // source of the row's entries, less its start in the warp's range
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint64_t c0 = (blockIdx.x * (uint64_t)8 + w) * 32, i = c0 + lane;
+  if (c0 >= n) return;  // whole warp
+  uint32_t len = 0;
+  int64_t a = 0;
+  if (i < n) {
+    const uint64_t o = perm[i];
+    a = B.cell_off[o];
+    len = (uint32_t)(B.cell_off[o + 1] - a);
+  }
+  uint32_t inc = len;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t v = __shfl_up_sync(0xffffffffu, inc, o);
+    if (lane >= o) inc += v;
+  }
+  s_end[w][lane] = inc;
+  s_src[w][lane] = a - (int64_t)(inc - len);
+  const uint32_t total = __shfl_sync(0xffffffffu, inc, 31);
+  __syncwarp();
+  const int64_t out = new_off[c0];
+  for (uint32_t q = lane; q < total; q += 32) {
+    int o = 0;  // the first row that ends after q
+#pragma unroll
+    for (int step = 16; step; step >>= 1)
+      if (s_end[w][o + step - 1] <= q) o += step;
+    const int64_t e = B.cell_idx[s_src[w][o] + q];
+    idx[out + q] = e >= 0 ? (int64_t)inv_e[e] : -1;
   }
 }
 
