@@ -199,8 +199,6 @@ __device__ __forceinline__ void rg_solve(const RgCtx &c, uint32_t off, uint32_t 
                                          unsigned long long &nterms) {
   constexpr int NSUB = 32 / W;
   const int lane = threadIdx.x & 31, sl = lane & (W - 1), q = lane / W;
-  const unsigned wm = W == 32 ? FULL : ((1u << (W & 31)) - 1u);
-  const unsigned below = (1u << sl) - 1u;
   const RgScratch sc = rg_scratch(c.B);
   const float *lst = c.lst + sl;
   float P[K], al[K];
@@ -272,13 +270,11 @@ __device__ __forceinline__ void rg_solve(const RgCtx &c, uint32_t off, uint32_t 
     // errs by far less than 1e-9 from it
     float wf = 0.f, wa = 0.f, m1 = 0.f, m1a = 0.f;
     unsigned strong = 0;  // bit k: entry k of this lane
-    int ns = 0;
 #pragma unroll
     for (int k = 0; k < K; k++) {
       const float e = al[k] * ex2_approx(fmaf(t32, fmaf(t32, gdd, Q[k]), P[k])), ae = fabsf(e);
       const float eq = e * Q[k];
       const bool s = ae > c.thr;
-      ns += __popc((__ballot_sync(FULL, s) >> (q * W)) & wm);
       strong |= s ? 1u << k : 0u;
       wf += s ? 0.f : e;
       wa += s ? 0.f : ae;
@@ -291,6 +287,19 @@ __device__ __forceinline__ void rg_solve(const RgCtx &c, uint32_t off, uint32_t 
     const float kc =
         fmaxf(root_rel_cached(c.R, D < MF_MAXD ? D : c.R.d, dd, c.B.list_r2) / c.R.weak_rel32, 1.f);
     const bool ok = have && reuse && !root_fp32_part_too_coarse(c.R, wa * kc, gpf, c.fast);
+    // places of the lanes' strong entries in the edge's list, lane by lane (a
+    // ballot per entry took as many instructions as a Halley evaluation, in a
+    // kernel whose first stall is the instruction fetch: 18.1 -> 13.4 ms for
+    // the 7.2M edges of a d = 5 proof at lambda = 0.08)
+    int at = __popc(strong);
+    int ns = at;
+#pragma unroll
+    for (int o = 1; o < W; o <<= 1) {
+      const int v = __shfl_up_sync(FULL, ns, o, W);
+      if (sl >= o) ns += v;
+    }
+    at = ns - at;
+    ns = __shfl_sync(FULL, ns, W - 1, W);
     // chunks of the strong list: one allocation for the edges of the round
     const uint32_t nch = ok ? (uint32_t)(ns + DEFER_CHUNK - 1) / DEFER_CHUNK : 0u;
     uint32_t my = 0, all = 0;
@@ -312,17 +321,11 @@ __device__ __forceinline__ void rg_solve(const RgCtx &c, uint32_t off, uint32_t 
       for (uint32_t h = sl; h < nch && c0 + h < ncap; h += W)
         c.B.defer_chunk[c0 + h] = fits ? rec_at : ~0u;
     const bool put = ok && fits;
-    int at = 0;
-#pragma unroll
-    for (int k = 0; k < K; k++) {
-      const bool s = (strong >> k) & 1u;
-      const unsigned m = (__ballot_sync(FULL, s) >> (q * W)) & wm;
-      if (put && s) c.B.defer_list[c0 * DEFER_CHUNK + at + __popc(m & below)] = c.src[k * W + sl];
-      at += __popc(m);
+    if (put) {
+      int32_t *to = c.B.defer_list + c0 * DEFER_CHUNK;
+      for (unsigned m = strong; m; m &= m - 1) to[at++] = c.src[(__ffs(m) - 1) * W + sl];
+      for (uint32_t h = ns + sl; h < nch * DEFER_CHUNK; h += W) to[h] = -1;
     }
-    if (put)
-      for (uint32_t h = ns + sl; h < nch * DEFER_CHUNK; h += W)
-        c.B.defer_list[c0 * DEFER_CHUNK + h] = -1;
     if (have && sl == 0) {
       RootRec r;
       r.e = put ? c.e0 + it.e : ~0ull;
