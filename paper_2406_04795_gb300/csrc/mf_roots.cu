@@ -13,8 +13,8 @@
 // (A warp per edge screened the list anew for every edge, two gathered passes
 // over it with most lanes idle after the screen.)  The chunk's edges are first
 // bucketed by base vertex.  This stage and the redo on the d = 5 FP64 proof at
-// lambda = 0.15 (1.32M edges, 0.24M vertices): 5.2 -> 3.7 ms; at lambda = 0.08
-// (7.2M edges, 1.2M vertices): 28.1 -> 20.0 ms; d = 6 BF16: 2.9 -> 2.4 ms.
+// lambda = 0.15 (1.32M edges, 0.24M vertices): 5.2 -> 3.2 ms; at lambda = 0.08
+// (7.2M edges, 1.2M vertices): 28.1 -> 13.4 ms; d = 6 BF16: 2.9 -> 1.7 ms.
 //
 // What it hands over is one RootRec per edge: the converged FP32 t, g' and g''
 // there, the FP32 sum of the terms below ROOT_TAU at t (checked against its
@@ -188,6 +188,7 @@ struct RgCtx {
   const int32_t *src;
   int nl;
   uint64_t e0;
+  const float *grad;  // sum over the list of alpha e^(-gamma |u|^2) u, at x1
   float g2, gm, b32, thr;
   bool fast;
 };
@@ -226,8 +227,19 @@ __device__ __forceinline__ void rg_solve(const RgCtx &c, uint32_t off, uint32_t 
     //   sum e (u + t dir).dir = -m1 / (2 g2) + t |dir|^2 m0, and so on
     const float iq = -0.5f / c.g2;
     // FP32 Halley iteration (cubic: the evaluation yields g'' anyway),
-    // bracketed, from the linear interpolant of the end values
-    float t32 = it.f0 / (it.f0 - it.f1);
+    // bracketed, from the parabola through the end values with the slope that
+    // the vertex's gradient gives at t = 0 (one evaluation per vertex, which
+    // saves one of two per edge on a lattice fine enough: d = 5 at lambda =
+    // 0.08 13.4 -> 11.7 ms, at 0.15 as before); else the linear interpolant
+    float g0 = 0.f;
+#pragma unroll
+    for (int a = 0; a < D; a++) g0 = fmaf(dr[a], c.grad[a], g0);
+    g0 *= -2.f * c.gm;
+    const float q2 = (it.f1 - it.f0) - g0;
+    const float r2 = g0 + copysignf(sqrtf(fmaxf(fmaf(g0, g0, -4.f * q2 * it.f0), 0.f)), g0);
+    float t32 = __fdividef(-2.f * it.f0, r2);
+    if (!(t32 > 0.f && t32 < 1.f)) t32 = __fdividef(-0.5f * r2, q2);
+    if (!(t32 > 0.f && t32 < 1.f)) t32 = it.f0 / (it.f0 - it.f1);
     if (!(t32 > 0.f && t32 < 1.f)) t32 = 0.5f;
     float lo = 0.f, hi = 1.f, gpp = INFINITY;
     bool done = false;
@@ -257,9 +269,10 @@ __device__ __forceinline__ void rg_solve(const RgCtx &c, uint32_t off, uint32_t 
         if (!inside) tn = 0.5f * (lo + hi);
         const float step = fabsf(tn - t32);
         t32 = tn;
-        // a Halley step of size s leaves an error of order s^3: below 1e-3
-        // the FP32 noise floor is reached and the FP64 step finishes
-        done = step <= 2e-6f || (halley && inside && step <= 1e-3f);
+        // a Halley step of size s leaves an error of order s^3: below 4e-3
+        // the FP32 noise floor (about 1e-6) is reached, and the last step
+        // finishes
+        done = step <= 2e-6f || (halley && inside && step <= 4e-3f);
       }
       if (__all_sync(FULL, done)) break;
     }
@@ -408,21 +421,29 @@ __global__ void __launch_bounds__(RG_WARPS * 32, RgClass<CLS>::BLOCKS) k_rg_solv
     // W K of the instantiation that takes the list
     const int held = CLS == 2 ? RG_BIG : CLS == 1 ? (nl <= 256 ? 256 : RG_MID)
                                                   : (nl <= 64 ? 64 : nl <= 128 ? 128 : RG_SMALL);
+    float gs[(D + 3) & ~3];
+#pragma unroll
+    for (int k = 0; k < ((D + 3) & ~3); k++) gs[k] = 0.f;
     for (int i = lane; i < held; i += 32) {
-      float cc[2 * D], al = 0.f, s32, A = 0.f;
+      float cc[2 * D], u[D], al = 0.f, s32, A = 0.f;
       const bool in = i < nl;
       if (in) sv_row<D>(R, src[i], cc, al, s32);
 #pragma unroll
       for (int k = 0; k < D; k++) {
-        const float u = in && k < d ? (xh[k] - cc[2 * k]) + (xl[k] - cc[2 * k + 1]) : 0.f;
-        lst[k * CAP + i] = u;
-        A = fmaf(u, u, A);
+        u[k] = in && k < d ? (xh[k] - cc[2 * k]) + (xl[k] - cc[2 * k + 1]) : 0.f;
+        lst[k * CAP + i] = u[k];
+        A = fmaf(u[k], u[k], A);
       }
       lst[D * CAP + i] = -g2 * A;
       lst[(D + 1) * CAP + i] = al;
+      const float e = al * ex2_approx(-g2 * A);
+#pragma unroll
+      for (int k = 0; k < D; k++) gs[k] = fmaf(e, u[k], gs[k]);
     }
+#pragma unroll
+    for (int k = 0; k < D; k += 4) sub_sum4<32>(gs[k], gs[k + 1], gs[k + 2], gs[k + 3]);
     __syncwarp();
-    const RgCtx c = {R,  B,  lst, dirt, src, nl, e0, g2, (float)R.gamma, (float)R.b,
+    const RgCtx c = {R,  B,  lst, dirt, src, nl, e0, gs, g2, (float)R.gamma, (float)R.b,
                      (fast ? ROOT_TAU_FAST : ROOT_TAU) * 0.60653066f, fast != 0};
     if (CLS == 2) {
       rg_solve<D, 32, RG_BIG / 32, CAP>(c, gr.off, gr.n, nterms);
