@@ -47,20 +47,26 @@ def df_term_ops(d):
     return 47 * d + 68
 
 
-# FP32-pipe operations of one FP32 term (Halley step or weak term): per
-# coordinate a hi and a lo difference, their sum, r2 and the projection
-# FMAs (5); then the exponent, ex2, alpha e and the accumulations (8)
+# FP32-pipe operations of one FP32 term of the root solve (k_rg_solve: a listed
+# vector in one evaluation at t): the exponent P + t (Q + t c) (2), ex2, alpha e,
+# e Q and the three moments (6); the coordinates enter once per vertex and edge,
+# so none of them is counted
 def f32_term_ops(d):
+    return 8
+
+
+# The same of one FP32 term of the vertex evaluation: per coordinate a hi and a
+# lo difference, their sum, r2 and the projection FMAs (5); then the exponent,
+# ex2, alpha e and the accumulations (8)
+def eval_f32_term_ops(d):
     return 5 * d + 8
 
 
-# DRAM bytes per traced edge of the root phase's kernels from their ncu
-# capture (dram__bytes_read.sum + dram__bytes_write.sum of k_roots_prep,
-# k_roots_f64 (warp and redo launches), k_roots_x, k_roots_terms and
-# k_roots_finish on the lambda = 0.15 case of the d=5 workload, divided by
-# its 880,448 edges: 1229.8 MB); None once a kernel has changed since the
-# capture
-ROOTS_DRAM_BYTES_PER_EDGE = 1396.8
+# DRAM bytes per traced edge of the root phase's kernels from an ncu capture
+# (dram__bytes_read.sum + dram__bytes_write.sum over the phase's launches,
+# divided by the traced edges); None once a kernel has changed since the
+# capture, as here: the one under profiles/ shows the per-edge kernels
+ROOTS_DRAM_BYTES_PER_EDGE = None
 
 
 def make_workload(cfg: str, rank: int, lam=None):
@@ -158,7 +164,8 @@ def roofline(stats, w, rates, E, ms_proof, n_proofs, root_traffic=True):
     # ex2 of all FP32 terms, and the algorithmic bytes of the table phases
     f64 = stats["eval"]["terms"] * per_eval
     f32 = (stats["roots"]["terms"] * df_term_ops(d) +
-           (stats["roots"]["terms_weak"] + stats["eval"]["terms_weak"]) * f32_term_ops(d))
+           stats["roots"]["terms_weak"] * f32_term_ops(d) +
+           stats["eval"]["terms_weak"] * eval_f32_term_ops(d))
     ex2 = stats["roots"]["terms_weak"] + stats["eval"]["terms_weak"]
     k = d // 2
     by = (stats["expand_vertices"]["units"] * ((4 * d + 4) + 32 * 2 ** d) +
@@ -190,8 +197,8 @@ def roofline(stats, w, rates, E, ms_proof, n_proofs, root_traffic=True):
                     work="%d RBF terms (vertex x support vector), one ex2 each" % s["terms_weak"])
     if dom == "roots":
         # the root phase's arithmetic runs on the FP32 pipe: double-float
-        # strong terms (k_roots_terms) and FP32 Halley / weak terms (the warp
-        # kernel); the few full FP64 re-evaluations are counted as strong terms
+        # strong terms (k_roots_terms) and FP32 Halley / weak terms
+        # (k_rg_solve); the few full FP64 re-evaluations are counted as strong terms
         ops = (s["terms"] * df_term_ops(d) + s["terms_weak"] * f32_term_ops(d)) / max(s["launches"], 1)
         ach = ops / (ms_per_launch * 1e-3) / 1e12
         # DRAM bytes per edge from the ncu capture of the root kernels
@@ -199,8 +206,9 @@ def roofline(stats, w, rates, E, ms_proof, n_proofs, root_traffic=True):
         # (taken on the FP64 path: none for the other precision)
         traffic = ROOTS_DRAM_BYTES_PER_EDGE * s["units"] / max(s["launches"], 1) \
             if ROOTS_DRAM_BYTES_PER_EDGE and root_traffic else None
-        return dict(base, kernel="roots phase: k_roots_prep, k_roots_f64 (warp screen and FP32 "
-                    "Halley steps), k_roots_x, k_roots_terms (double-float sums), k_roots_finish",
+        return dict(base, kernel="roots phase: k_rg_count / groups / scatter (edges by base vertex), "
+                    "k_rg_solve (FP32 Halley steps), k_roots_x, k_roots_terms (double-float "
+                    "sums), k_roots_finish, k_roots_f64 (redo)",
                     bound="alu", achieved=ach, peak=f32_peak, unit="T FP32 ops/s",
                     frac=ach / f32_peak, traffic=traffic,
                     peak_source="measured: mf_probe_rates FP32 FMA probe (one operation per "
