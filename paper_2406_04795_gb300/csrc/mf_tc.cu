@@ -50,7 +50,7 @@ struct TcShared {
   uint64_t bar[2];
   uint32_t tmem;
   int timeout;
-  int32_t y0[MF_MAXD];
+  int32_t y0[MF_MAXD], ysum[TC_M / 32][MF_MAXD];
   float q0hi[MF_MAXD], q0lo[MF_MAXD];
 };
 
@@ -114,17 +114,35 @@ __device__ __forceinline__ bool tc_tile(const MfFrame &F, const MfRbfDev &R, con
   int32_t y[D];
 #pragma unroll
   for (int k = 0; k < D; k++) y[k] = valid ? B.vert_y[v * D + k] : 0;
-  if (t == 0) {
-    int32_t ym[MF_MAXD];
-    double q0[MF_MAXD];
-#pragma unroll
-    for (int k = 0; k < MF_MAXD; k++) ym[k] = k < D ? y[k] : 0;
-    mf_vertex_x(F, ym, q0);
+  // the tile base: the mean of the tile's vertices, rounded.  The rounding of
+  // D grows with the square of a vertex's distance from the base, which the
+  // mean halves against the tile's first vertex.
+  {
+    const int64_t n = (int64_t)min((uint64_t)TC_M, v_end - v_first);
 #pragma unroll
     for (int k = 0; k < D; k++) {
-      sh.y0[k] = y[k];
-      sh.q0hi[k] = (float)q0[k];
-      sh.q0lo[k] = (float)(q0[k] - (double)sh.q0hi[k]);
+      const int s = __reduce_add_sync(0xffffffffu, valid ? y[k] : 0);
+      if ((t & 31) == 0) sh.ysum[w][k] = s;
+    }
+    __syncthreads();
+    if (t == 0) {
+      int32_t ym[MF_MAXD];
+      double q0[MF_MAXD];
+#pragma unroll
+      for (int k = 0; k < MF_MAXD; k++) ym[k] = 0;
+#pragma unroll
+      for (int k = 0; k < D; k++) {
+        int64_t s = 0;
+        for (int q = 0; q < TC_M / 32; q++) s += sh.ysum[q][k];
+        ym[k] = (int32_t)(s >= 0 ? (2 * s + n) / (2 * n) : -((n - 2 * s) / (2 * n)));
+      }
+      mf_vertex_x(F, ym, q0);
+#pragma unroll
+      for (int k = 0; k < D; k++) {
+        sh.y0[k] = ym[k];
+        sh.q0hi[k] = (float)q0[k];
+        sh.q0lo[k] = (float)(q0[k] - (double)sh.q0hi[k]);
+      }
     }
   }
   __syncthreads();
