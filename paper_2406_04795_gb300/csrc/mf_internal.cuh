@@ -38,6 +38,12 @@ struct MfFrame {
 };
 
 // Device counters of one trace; read back by the host once per BFS level.
+// A step of the search: edges [begin, begin + n) of the level that ends at end
+// (n = 0: the search has ended).
+struct MfStep {
+  unsigned long long begin, n, end;
+};
+
 struct MfCounters {
   unsigned long long n_edges;      // edges appended to the edge list
   unsigned long long n_vertices;   // vertices appended to the vertex list
@@ -61,10 +67,11 @@ struct MfCounters {
   unsigned long long n_groups[3];  // base vertices with edges in the chunk, by list length (mf_roots.cu)
   unsigned long long n_redo;       // deferred steps not accepted (solved again in full)
   unsigned long long n_items;      // expand items given a vertex slot
-  // the search's current step: edges [lv_begin, lv_begin + lv_n) of the level
-  // that ends at lv_end (lv_n = 0: the search has ended), steps of at most
+  // the search's steps: the s-th one's kernels read step[s & 1], and its edges
+  // pass writes step[(s + 1) & 1] (see mf_search_next); steps of at most
   // lv_cap edges, and the levels opened so far
-  unsigned long long lv_begin, lv_end, lv_n, lv_cap, levels;
+  MfStep step[2];
+  unsigned long long lv_cap, levels;
   unsigned int lv_ticket;          // blocks of the edges pass that have finished
   unsigned int err_table_full;     // a hash probe ran past the table
   unsigned int err_overflow;       // a list ran past its capacity
@@ -642,8 +649,8 @@ void mf_launch_seeds(const MfFrame &F, const MfTraceBufs &B, const double *seeds
                      bool vertices, cudaStream_t s);
 // One pass of the search over edges [e0, e0 + n): the new vertices of their
 // 2-simplex cofaces, or (after those are evaluated) the new crossing edges.
-// n = MF_STEP: the counters' current step, which the edges pass then advances
-// (v_evaluated and n_recheck_done included).
+// n = MF_STEP: the counters' step e0 (its record is e0 & 1), after which the
+// edges pass opens the next one (v_evaluated and n_recheck_done included).
 #define MF_STEP (~0ull)
 void mf_launch_expand(const MfFrame &F, const MfTraceBufs &B, uint64_t e0, uint64_t n, bool edges,
                       int sms, cudaStream_t st);
@@ -652,6 +659,77 @@ void mf_launch_expand(const MfFrame &F, const MfTraceBufs &B, uint64_t e0, uint6
 // fill of B.cell_idx (a missing edge sets err_missing).
 void mf_launch_cells_enum(const MfFrame &F, const MfTraceBufs &B, uint64_t n_edges, cudaStream_t st);
 void mf_launch_cells_fill(const MfFrame &F, const MfTraceBufs &B, uint64_t n_cells, cudaStream_t st);
+// ------------------------------------------------------------------------
+// The search's steps, kept in the counters, so that the host can enqueue several
+// without reading any of them back (see mf_trace).  Every block of a step's
+// edges pass reads the step's record, whenever it starts; only the blocks that
+// have work (the first mf_step_blocks of the grid) take a ticket, and the last
+// of those opens the next step while blocks without work may not have started
+// yet.  So the next step goes into the other record: no launch reads a record
+// that its own grid writes.  Shared by the kernels and the host simulation of
+// them (mf_diag_search).
+// ------------------------------------------------------------------------
+// Edges per warp of a pass over n edges by nwarps warps: 32 when the level
+// fills the chip, fewer when it does not, down to the number whose items fit
+// one round of the warp's lanes (an edge has at most 2^d - 2).  The passes
+// are chains of dependent accesses (slot, f, probe, append), so a level that
+// leaves SMs empty takes as long as its longest warp: with 32 edges per warp a
+// d = 3 level of 500 edges ran 6 rounds on 2 blocks (36 us), with 4 edges 1
+// round on 16 blocks (9 us; the vertex pass 15 -> 6).
+__host__ __device__ __forceinline__ int mf_step_group(int d, unsigned long long n,
+                                                      unsigned long long nwarps) {
+  int g = d <= 2 ? 16 : d == 3 ? 4 : d == 4 ? 2 : 1;
+  while (g < 32 && n > (unsigned long long)g * nwarps) g <<= 1;
+  return g;
+}
+
+// Blocks of the grid that have work, the first ones.
+__host__ __device__ __forceinline__ unsigned mf_step_blocks(unsigned long long n, int group,
+                                                            int warps, unsigned grid) {
+  const unsigned long long per = (unsigned long long)group * warps;
+  const unsigned long long used = (n + per - 1) / per;
+  return (unsigned)(used < grid ? used : grid);
+}
+
+// First step: the seed edges.
+__host__ __device__ __forceinline__ void mf_search_first(MfCounters &c, unsigned long long max_edges,
+                                                         unsigned long long cap) {
+  const bool err = c.err_table_full || c.err_missing || c.err_overflow || c.err_timeout;
+  const unsigned long long ne = err || c.n_edges > max_edges ? 0ull : c.n_edges;
+  c.step[0].begin = 0;
+  c.step[0].end = ne;
+  c.step[0].n = ne < cap ? ne : cap;
+  c.step[1] = c.step[0];
+  c.lv_cap = cap;
+  c.levels = ne > 0 ? 1 : 0;
+  c.lv_ticket = 0;
+}
+
+// End of step s (one thread, after every block of its edges pass that has
+// work; or of a step without edges, which passes that on): opens step s + 1,
+// the rest of the level, or the next one, or no further step when the level
+// appended no edge or an error was set.
+__host__ __device__ __forceinline__ void mf_search_next(volatile MfCounters &c, unsigned s,
+                                                        unsigned long long max_edges) {
+  const volatile MfStep &cur = c.step[s & 1];
+  volatile MfStep &next = c.step[(s + 1) & 1];
+  const bool err = c.err_table_full || c.err_missing || c.err_overflow || c.err_timeout;
+  const unsigned long long ne = c.n_edges, at = cur.begin + cur.n;
+  unsigned long long end = cur.end;
+  if (cur.n) {
+    c.v_evaluated = c.n_vertices;
+    c.n_recheck_done = c.n_recheck;
+    if (at >= end && ne > end && ne <= max_edges && !err) {
+      end = ne;
+      c.levels = c.levels + 1;
+    }
+  }
+  const unsigned long long left = err || !cur.n ? 0ull : end - at;
+  next.begin = at;
+  next.end = end;
+  next.n = left < c.lv_cap ? left : c.lv_cap;
+}
+
 // Launch choices picked by the autotuner (mf_autotune); the defaults serve
 // untuned contexts and the allocation-free entry point.
 struct MfTune {

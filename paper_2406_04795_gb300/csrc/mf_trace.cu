@@ -20,6 +20,7 @@
 //                      the edge table; first inserters append it to the edge list.
 #include <algorithm>
 #include <cmath>
+#include <random>
 #include <vector>
 #include <cstdio>
 #include <cstring>
@@ -325,19 +326,6 @@ __device__ __forceinline__ int expand_owner(const uint32_t *s_end, uint32_t j, u
 
 #define EXPAND_WARPS 8
 
-// Edges per warp of a pass over n edges by nwarps warps: 32 when the level
-// fills the chip, fewer when it does not, down to the number whose items fit
-// one round of the warp's lanes (an edge has at most 2^d - 2).  The passes
-// are chains of dependent accesses (slot, f, probe, append), so a level that
-// leaves SMs empty takes as long as its longest warp: with 32 edges per warp a
-// d = 3 level of 500 edges ran 6 rounds on 2 blocks (36 us), with 4 edges 1
-// round on 16 blocks (9 us; the vertex pass 15 -> 6).
-__device__ __forceinline__ int expand_group(int d, unsigned long long n, unsigned long long nwarps) {
-  int g = d <= 2 ? 16 : d == 3 ? 4 : d == 4 ? 2 : 1;
-  while (g < 32 && n > (unsigned long long)g * nwarps) g <<= 1;
-  return g;
-}
-
 struct ExpandShared {
   uint32_t end[EXPAND_WARPS][32], S[EXPAND_WARPS][32];
   unsigned long long off[EXPAND_WARPS][32];  // each edge's first item in the slot record
@@ -345,7 +333,7 @@ struct ExpandShared {
   double f[EXPAND_WARPS][32][2];  // edges pass: the end values
 };
 
-// Edges [e0, e0 + n): a warp takes expand_group edges, lane per coface item,
+// Edges [e0, e0 + n): a warp takes mf_step_group edges, lane per coface item,
 // so that no lane idles on masks that select no coface.  Returns the number of
 // blocks of the grid that have work (the first ones).
 template <bool EDGES>
@@ -355,7 +343,7 @@ __device__ __forceinline__ unsigned expand_range(const MfFrame &F, const MfTrace
   const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5;
   const int d = F.d;
   const uint64_t nwarps = (uint64_t)gridDim.x * EXPAND_WARPS;
-  const uint64_t G = (uint64_t)expand_group(d, n, nwarps);
+  const uint64_t G = (uint64_t)mf_step_group(d, n, nwarps);
   unsigned nb = 0;
   for (uint64_t first = (blockIdx.x * (uint64_t)EXPAND_WARPS + wi) * G; first < n;
        first += nwarps * G) {
@@ -421,42 +409,12 @@ __device__ __forceinline__ unsigned expand_range(const MfFrame &F, const MfTrace
     nb = __reduce_add_sync(0xffffffffu, nb);
     if (lane == 0 && nb) atomicAdd(&B.cnt->n_boundary, (unsigned long long)nb);
   }
-  const uint64_t used = (n + G * EXPAND_WARPS - 1) / (G * EXPAND_WARPS);
-  return (unsigned)(used < gridDim.x ? used : gridDim.x);
+  return mf_step_blocks(n, (int)G, EXPAND_WARPS, gridDim.x);
 }
 
-// The search's steps live in the counters, so that the host can enqueue several
-// without reading any of them back (see mf_trace).  First step: the seed edges.
+// First step of the search (see mf_search_first).
 __global__ void k_search_start(MfTraceBufs B, unsigned long long cap) {
-  MfCounters &c = *B.cnt;
-  const bool err = c.err_table_full || c.err_missing || c.err_overflow || c.err_timeout;
-  const unsigned long long ne = err || c.n_edges > B.max_edges ? 0ull : c.n_edges;
-  c.lv_begin = 0;
-  c.lv_end = ne;
-  c.lv_cap = cap;
-  c.lv_n = ne < cap ? ne : cap;
-  c.levels = ne > 0 ? 1 : 0;
-  c.lv_ticket = 0;
-}
-
-// End of a step (one thread, after every block of the edges pass): the rest of
-// the level, or the next one, or no further step when the level appended no
-// edge or an error was set.
-__device__ __forceinline__ void search_next(const MfTraceBufs &B) {
-  volatile MfCounters &c = *B.cnt;
-  const bool err = c.err_table_full || c.err_missing || c.err_overflow || c.err_timeout;
-  const unsigned long long ne = c.n_edges, at = c.lv_begin + c.lv_n;
-  unsigned long long end = c.lv_end;
-  c.v_evaluated = c.n_vertices;
-  c.n_recheck_done = c.n_recheck;
-  if (at >= end && ne > end && ne <= B.max_edges && !err) {
-    end = ne;
-    c.levels = c.levels + 1;
-  }
-  const unsigned long long left = err ? 0ull : end - at;
-  c.lv_begin = at;
-  c.lv_end = end;
-  c.lv_n = left < c.lv_cap ? left : c.lv_cap;
+  mf_search_first(*B.cnt, B.max_edges, cap);
 }
 
 // D < MF_MAXD: the exact dimension, so that the coordinate loops and the key
@@ -467,8 +425,9 @@ __global__ void __launch_bounds__(EXPAND_WARPS * 32) k_expand_vertices(MfFrame F
   if (D < MF_MAXD) F.d = D;  // the coordinate loops then unroll to exactly D
   mf_dep_wait();
   if (n == MF_STEP) {
-    e0 = B.cnt->lv_begin;
-    n = B.cnt->lv_n;
+    const MfStep s = B.cnt->step[e0 & 1];
+    e0 = s.begin;
+    n = s.n;
   }
   expand_range<false>(F, B, e0, n);
 }
@@ -479,10 +438,17 @@ __global__ void __launch_bounds__(EXPAND_WARPS * 32) k_expand_edges(MfFrame F, M
   if (D < MF_MAXD) F.d = D;  // the coordinate loops then unroll to exactly D
   mf_dep_wait();
   const bool step = n == MF_STEP;
+  const unsigned no = (unsigned)e0;
   if (step) {
-    e0 = B.cnt->lv_begin;
-    n = B.cnt->lv_n;
-    if (n == 0) return;  // every block of the launch sees the same step
+    // the same step for every block, however late it starts: this launch
+    // writes the other record only
+    const MfStep s = B.cnt->step[no & 1];
+    e0 = s.begin;
+    n = s.n;
+    if (n == 0) {
+      if (blockIdx.x == 0 && threadIdx.x == 0) mf_search_next(*B.cnt, no, B.max_edges);
+      return;
+    }
   }
   const unsigned used = expand_range<true>(F, B, e0, n);
   if (step && blockIdx.x < used) {  // the last of those blocks to finish opens the next step
@@ -492,7 +458,7 @@ __global__ void __launch_bounds__(EXPAND_WARPS * 32) k_expand_edges(MfFrame F, M
       if (atomicAdd(&B.cnt->lv_ticket, 1u) == used - 1) {
         __threadfence();
         B.cnt->lv_ticket = 0;
-        search_next(B);
+        mf_search_next(*B.cnt, no, B.max_edges);
       }
     }
   }
@@ -959,7 +925,7 @@ __global__ void __launch_bounds__(EXPAND_WARPS * 32) k_b_expand(const MfSlot *sl
   const int lane = threadIdx.x & 31, wi = threadIdx.x >> 5;
   const unsigned long long nwarps = (unsigned long long)gridDim.x * EXPAND_WARPS;
   // edges per warp as for one trace (the slots' dimensions differ: d = 4)
-  const unsigned long long G = (unsigned long long)expand_group(4, total, nwarps);
+  const unsigned long long G = (unsigned long long)mf_step_group(4, total, nwarps);
   for (unsigned long long first = (blockIdx.x * (unsigned long long)EXPAND_WARPS + wi) * G;
        first < total; first += nwarps * G) {
     const unsigned long long item = first + lane;
@@ -1832,11 +1798,12 @@ extern "C" int mf_trace(mf_ctx *ctx, const mf_rbf *rbf, const mf_domain *dom,
   // reads the counters of the older one while the newer one runs; steps after
   // the last find no edges and return at once (about 6 us each).
   MfCounters *const hc = ctx->h_counters;  // [2], pinned
+  uint64_t step = 0;                       // steps enqueued
   for (int it = 0;; it++) {
-    for (int k = 0; k < SEARCH_AHEAD; k++) {
+    for (int k = 0; k < SEARCH_AHEAD; k++, step++) {
       {
         MfProfScope ps(ctx, MF_PH_EXPAND_V, st, 1);
-        mf_launch_expand(F, B, 0, MF_STEP, false, sms, st);
+        mf_launch_expand(F, B, step, MF_STEP, false, sms, st);
       }
       {
         MfProfScope ps(ctx, MF_PH_EVAL, st, mixed ? (B.vlist ? 3 : 2) : 1);
@@ -1844,7 +1811,7 @@ extern "C" int mf_trace(mf_ctx *ctx, const mf_rbf *rbf, const mf_domain *dom,
       }
       {
         MfProfScope ps(ctx, MF_PH_EXPAND_E, st, 1);
-        mf_launch_expand(F, B, 0, MF_STEP, true, sms, st);
+        mf_launch_expand(F, B, step, MF_STEP, true, sms, st);
       }
     }
     cudaMemcpyAsync(&hc[it & 1], B.cnt, sizeof(MfCounters), cudaMemcpyDeviceToHost, st);
@@ -1853,7 +1820,8 @@ extern "C" int mf_trace(mf_ctx *ctx, const mf_rbf *rbf, const mf_domain *dom,
     if (it == 0) continue;
     rc = mf_cuda_check(ctx, cudaEventSynchronize(ctx->step_event[(it - 1) & 1]), "trace kernels");
     if (rc) return rc;
-    if (hc[(it - 1) & 1].lv_n == 0) break;
+    // the step after the older group's last one
+    if (hc[(it - 1) & 1].step[(step - SEARCH_AHEAD) & 1].n == 0) break;
   }
   rc = read_counters(ctx, B, st);
   if (rc) return rc;
@@ -1958,6 +1926,67 @@ extern "C" int mf_trace_fetch(mf_ctx *ctx, mf_trace_out *out, void *stream) {
   if (!ctx->last.valid) return mf_set_error(ctx, MF_ERR_INVALID, "no trace result to fetch");
   cudaSetDevice(ctx->device);
   return copy_out(ctx, ctx->last, out, (cudaStream_t)stream);
+}
+
+extern "C" int mf_diag_search(int32_t d, int32_t grid, int64_t cap, const int32_t *appends,
+                              int64_t n_edges, int64_t n_seed, uint64_t order_seed,
+                              int32_t *expanded, int64_t *levels, int64_t *steps) {
+  if (d < 2 || d > MF_MAXD || grid < 1 || cap < 1 || !appends || !expanded || !levels || !steps ||
+      n_seed < 0 || n_seed > n_edges)
+    return MF_ERR_INVALID;
+  MfCounters c;
+  memset(&c, 0, sizeof(c));
+  memset(expanded, 0, (size_t)n_edges * sizeof(*expanded));
+  c.n_edges = (unsigned long long)n_seed;
+  mf_search_first(c, (unsigned long long)n_edges, (unsigned long long)cap);
+  std::mt19937_64 rng(order_seed);
+  struct Block {
+    bool started;
+    unsigned index;
+    MfStep s;
+  };
+  std::vector<Block> live;
+  uint64_t no = 0;
+  int idle = 0;  // steps enqueued past the end, which must stay without edges
+  for (; idle < 2 * SEARCH_AHEAD; no++) {
+    if (no > (uint64_t)n_edges + 2 * SEARCH_AHEAD) return MF_ERR_TIMEOUT;
+    if (c.step[no & 1].n == 0) idle++;
+    live.clear();
+    for (int b = 0; b < grid; b++) live.push_back({false, (unsigned)b, MfStep()});
+    while (!live.empty()) {
+      const size_t at = (size_t)(rng() % live.size());
+      Block &b = live[at];
+      if (!b.started) {
+        b.started = true;
+        b.s = c.step[no & 1];
+        if (b.s.n) continue;
+        if (b.index == 0) mf_search_next(c, (unsigned)no, (unsigned long long)n_edges);
+      } else {
+        // k_expand_edges: expand_range, then the ticket
+        const uint64_t nwarps = (uint64_t)grid * EXPAND_WARPS, n = b.s.n;
+        const uint64_t G = (uint64_t)mf_step_group(d, n, nwarps);
+        for (int wi = 0; wi < EXPAND_WARPS; wi++)
+          for (uint64_t first = (b.index * (uint64_t)EXPAND_WARPS + wi) * G; first < n;
+               first += nwarps * G)
+            for (uint64_t i = first; i < n && i < first + G; i++) {
+              const uint64_t e = b.s.begin + i;
+              if (e >= c.n_edges) return MF_ERR_INVALID;
+              expanded[e]++;
+              c.n_edges = std::min<uint64_t>(c.n_edges + (uint64_t)appends[e], (uint64_t)n_edges);
+            }
+        const unsigned used = mf_step_blocks(n, (int)G, EXPAND_WARPS, (unsigned)grid);
+        if (b.index < used && c.lv_ticket++ == used - 1) {
+          c.lv_ticket = 0;
+          mf_search_next(c, (unsigned)no, (unsigned long long)n_edges);
+        }
+      }
+      live[at] = live.back();
+      live.pop_back();
+    }
+  }
+  *levels = (int64_t)c.levels;
+  *steps = (int64_t)no - idle;
+  return MF_OK;
 }
 
 extern "C" int mf_vertex_keys(int32_t d, double lambda, const mf_domain *dom, const int32_t *y,

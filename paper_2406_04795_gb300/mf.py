@@ -42,7 +42,7 @@ EXPORTS = ("mf_ctx_create", "mf_ctx_destroy", "mf_last_error", "mf_ctx_bytes", "
            "mf_server_status", "mf_server_fetch", "mf_server_done", "mf_autotune", "mf_ctx_set_tune",
            "mf_ctx_get_tune", "mf_vertex_keys", "mf_probe_rates", "mf_diag_exp",
            "mf_certify_ex", "mf_subdiv_begin", "mf_subdiv_next",
-           "mf_server_wait")
+           "mf_server_wait", "mf_diag_search")
 
 MF_PHASES = 12
 PHASE_NAMES = ("prepare", "seeds", "expand_vertices", "eval", "expand_edges", "roots", "cells",
@@ -212,6 +212,9 @@ def load(build_if_missing: bool = True):
     L.mf_probe_rates.argtypes = [V, P(mf_rates), V]
     L.mf_diag_exp.restype = C.c_int
     L.mf_diag_exp.argtypes = [V, V, C.c_int64, V, V, V]
+    L.mf_diag_search.restype = C.c_int
+    L.mf_diag_search.argtypes = [C.c_int32, C.c_int32, C.c_int64, V, C.c_int64, C.c_int64,
+                                 C.c_uint64, V, P(C.c_int64), P(C.c_int64)]
     _lib = L
     return L
 
@@ -416,6 +419,21 @@ def mf_probe_rates(ctx, stream=0) -> mf_rates:
 
 def mf_diag_exp(ctx, x_ptr, n, y_table_ptr, y_lib_ptr, stream=0):
     return _check(ctx, load().mf_diag_exp(ctx, x_ptr, n, y_table_ptr, y_lib_ptr, stream))
+
+
+def mf_diag_search(d, grid, cap, appends, n_seed, order_seed):
+    """(times each edge was expanded, levels, steps) of the search's step
+    protocol on a simulated grid (host only)."""
+    import numpy as np
+    appends = np.ascontiguousarray(appends, dtype=np.int32)
+    expanded = np.zeros(appends.size, dtype=np.int32)
+    levels, steps = C.c_int64(), C.c_int64()
+    rc = load().mf_diag_search(d, grid, cap, appends.ctypes.data_as(C.c_void_p), appends.size,
+                               n_seed, order_seed, expanded.ctypes.data_as(C.c_void_p),
+                               C.byref(levels), C.byref(steps))
+    if rc != MF_OK:
+        raise MfError(rc, "mf_diag_search")
+    return expanded, levels.value, steps.value
 
 
 def mf_ctx_set_tune(ctx, t):
