@@ -471,19 +471,21 @@ int mf_probe_rates(mf_ctx *ctx, mf_rates *out, void *stream);
 int mf_diag_exp(mf_ctx *ctx, const double *x, int64_t n, double *y_table, double *y_lib,
                 void *stream);
 
-/* The search's step protocol on a simulated grid (host only, no GPU needed):
- * edges 0 .. n_seed - 1 form the first level, expanding edge e appends
+/* The search's loop and step protocol on a simulated grid (host only, no GPU
+ * needed): edges 0 .. n_seed - 1 form the first level, expanding edge e appends
  * appends[e] further ones (up to n_edges in all), and each step's edges pass
  * runs as `grid` blocks that start and finish in a random order, the ones
  * without work as late as the last, through the functions that the kernels
  * use.  expanded[e] (host [n_edges]) counts how often edge e was expanded, once
  * each if every block saw its own step; *levels and *steps receive what the
- * search counted.  cap: most edges per step.  MF_ERR_INVALID when a block
- * reads an edge that does not exist, MF_ERR_TIMEOUT when the search does not
- * end. */
+ * search counted.  cap: most edges per step.  refused >= 0: the passes of that
+ * step and of all later ones do not run, and their launch reports `status`
+ * (MF_OK: the refusal goes unnoticed).  MF_ERR_INVALID when a block reads an
+ * edge that does not exist, MF_ERR_CUDA when the search makes no progress,
+ * MF_ERR_TIMEOUT when it does not end. */
 int mf_diag_search(int32_t d, int32_t grid, int64_t cap, const int32_t *appends, int64_t n_edges,
-                   int64_t n_seed, uint64_t order_seed, int32_t *expanded, int64_t *levels,
-                   int64_t *steps);
+                   int64_t n_seed, uint64_t order_seed, int64_t refused, int32_t status,
+                   int32_t *expanded, int64_t *levels, int64_t *steps);
 
 #ifdef __cplusplus
 }

@@ -592,7 +592,7 @@ static inline void mf_launch_dep(void (*k)(P...), unsigned grid, unsigned block,
   at[0].val.programmaticStreamSerializationAllowed = 1;
   c.attrs = at;
   c.numAttrs = 1;
-  cudaLaunchKernelEx(&c, k, P(a)...);
+  cudaLaunchKernelEx(&c, k, P(a)...);  // a refusal is the last error, as for <<<>>>
 }
 
 // ------------------------------------------------------------------------

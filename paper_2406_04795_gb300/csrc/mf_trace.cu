@@ -20,6 +20,7 @@
 //                      the edge table; first inserters append it to the edge list.
 #include <algorithm>
 #include <cmath>
+#include <functional>
 #include <random>
 #include <vector>
 #include <cstdio>
@@ -1514,7 +1515,38 @@ void mf_launch_seeds(const MfFrame &F, const MfTraceBufs &B, const double *seeds
   else k_seed_edges<<<g, 128, 0, s>>>(F, B, seeds, n);
 }
 
-#define SEARCH_AHEAD 2  // steps enqueued between two reads of the counters (see mf_trace)
+#define SEARCH_AHEAD 2  // steps enqueued between two reads of the counters
+
+// The search's loop.  The kernels of a step take its edges from the counters,
+// and its edges pass opens the next step, so nothing is read back in between:
+// the host keeps two groups of SEARCH_AHEAD steps enqueued and reads the
+// counters of the older one while the newer one runs; steps after the last
+// find no edges and return at once (about 6 us each).  G enqueues step s
+// (step), enqueues a read of the counters into q (post), waits for it (wait),
+// and waits for all of it after an error (drain).  Every step of a search that
+// has not ended moves on by an edge at least, so two reads with the same
+// beginning end it (stalled): the edges pass, the only writer of the steps,
+// did not run.
+template <class G>
+static int search_run(G &g) {
+  uint64_t step = 0;  // steps enqueued
+  unsigned long long last = ~0ull;
+  int rc = MF_OK;
+  for (int it = 0; !rc; it++) {
+    for (int k = 0; k < SEARCH_AHEAD && !rc; k++, step++) rc = g.step(step);
+    if (!rc) rc = g.post(it & 1);
+    if (rc || it == 0) continue;
+    const MfCounters *c;
+    rc = g.wait((it - 1) & 1, &c);
+    if (rc) break;
+    const MfStep &s = c->step[(step - SEARCH_AHEAD) & 1];  // after the older group's last one
+    if (s.n == 0) return MF_OK;
+    if (s.begin == last) rc = g.stalled();
+    last = s.begin;
+  }
+  g.drain();
+  return rc;
+}
 
 static int read_counters(mf_ctx *ctx, const MfTraceBufs &B, cudaStream_t st) {
   int rc = mf_cuda_check(ctx, cudaMemcpyAsync(ctx->h_counters, B.cnt, sizeof(MfCounters),
@@ -1791,38 +1823,48 @@ extern "C" int mf_trace(mf_ctx *ctx, const mf_rbf *rbf, const mf_domain *dom,
   k_search_start<<<1, 1, 0, st>>>(B, (unsigned long long)cap);
   rc = mf_cuda_check(ctx, cudaGetLastError(), "seed kernels");
   if (rc) return rc;
-
-  // Search edges (Fig. 4): the kernels of a step take its edges from the
-  // counters, and its edges pass opens the next step, so nothing is read back
-  // in between.  The host keeps two groups of SEARCH_AHEAD steps enqueued and
-  // reads the counters of the older one while the newer one runs; steps after
-  // the last find no edges and return at once (about 6 us each).
-  MfCounters *const hc = ctx->h_counters;  // [2], pinned
-  uint64_t step = 0;                       // steps enqueued
-  for (int it = 0;; it++) {
-    for (int k = 0; k < SEARCH_AHEAD; k++, step++) {
-      {
-        MfProfScope ps(ctx, MF_PH_EXPAND_V, st, 1);
-        mf_launch_expand(F, B, step, MF_STEP, false, sms, st);
-      }
-      {
-        MfProfScope ps(ctx, MF_PH_EVAL, st, mixed ? (B.vlist ? 3 : 2) : 1);
-        eval(false);
-      }
-      {
-        MfProfScope ps(ctx, MF_PH_EXPAND_E, st, 1);
-        mf_launch_expand(F, B, step, MF_STEP, true, sms, st);
-      }
+  // One step.  Its edges pass reads what the two passes before it wrote, so it
+  // is not launched when one of them was refused.
+  const std::function<int(uint64_t)> launch_step = [&](uint64_t s) {
+    {
+      MfProfScope ps(ctx, MF_PH_EXPAND_V, st, 1);
+      mf_launch_expand(F, B, s, MF_STEP, false, sms, st);
     }
-    cudaMemcpyAsync(&hc[it & 1], B.cnt, sizeof(MfCounters), cudaMemcpyDeviceToHost, st);
-    rc = mf_cuda_check(ctx, cudaEventRecord(ctx->step_event[it & 1], st), "BFS kernels");
-    if (rc) return rc;
-    if (it == 0) continue;
-    rc = mf_cuda_check(ctx, cudaEventSynchronize(ctx->step_event[(it - 1) & 1]), "trace kernels");
-    if (rc) return rc;
-    // the step after the older group's last one
-    if (hc[(it - 1) & 1].step[(step - SEARCH_AHEAD) & 1].n == 0) break;
-  }
+    {
+      MfProfScope ps(ctx, MF_PH_EVAL, st, mixed ? (B.vlist ? 3 : 2) : 1);
+      eval(false);
+    }
+    const int r = mf_cuda_check(ctx, cudaGetLastError(), "BFS kernels");
+    if (r) return r;
+    MfProfScope ps(ctx, MF_PH_EXPAND_E, st, 1);
+    mf_launch_expand(F, B, s, MF_STEP, true, sms, st);
+    return (int)MF_OK;
+  };
+
+  // Search edges (Fig. 4)
+  MfCounters *const hc = ctx->h_counters;  // [2], pinned
+  struct {
+    mf_ctx *ctx;
+    const std::function<int(uint64_t)> &launch;
+    const MfTraceBufs &B;
+    cudaStream_t st;
+    int step(uint64_t s) { return launch(s); }
+    int post(int q) {
+      cudaMemcpyAsync(&ctx->h_counters[q], B.cnt, sizeof(MfCounters), cudaMemcpyDeviceToHost, st);
+      const int r = mf_cuda_check(ctx, cudaGetLastError(), "BFS kernels");
+      return r ? r : mf_cuda_check(ctx, cudaEventRecord(ctx->step_event[q], st), "BFS kernels");
+    }
+    int wait(int q, const MfCounters **c) {
+      *c = &ctx->h_counters[q];
+      return mf_cuda_check(ctx, cudaEventSynchronize(ctx->step_event[q]), "trace kernels");
+    }
+    int stalled() {
+      return mf_set_error(ctx, MF_ERR_CUDA, "trace kernels: the search made no progress");
+    }
+    void drain() { cudaStreamSynchronize(st); }
+  } run = {ctx, launch_step, B, st};
+  rc = search_run(run);
+  if (rc) return rc;
   rc = read_counters(ctx, B, st);
   if (rc) return rc;
   const uint64_t E = hc->n_edges;
@@ -1930,7 +1972,8 @@ extern "C" int mf_trace_fetch(mf_ctx *ctx, mf_trace_out *out, void *stream) {
 
 extern "C" int mf_diag_search(int32_t d, int32_t grid, int64_t cap, const int32_t *appends,
                               int64_t n_edges, int64_t n_seed, uint64_t order_seed,
-                              int32_t *expanded, int64_t *levels, int64_t *steps) {
+                              int64_t refused, int32_t status, int32_t *expanded, int64_t *levels,
+                              int64_t *steps) {
   if (d < 2 || d > MF_MAXD || grid < 1 || cap < 1 || !appends || !expanded || !levels || !steps ||
       n_seed < 0 || n_seed > n_edges)
     return MF_ERR_INVALID;
@@ -1939,54 +1982,77 @@ extern "C" int mf_diag_search(int32_t d, int32_t grid, int64_t cap, const int32_
   memset(expanded, 0, (size_t)n_edges * sizeof(*expanded));
   c.n_edges = (unsigned long long)n_seed;
   mf_search_first(c, (unsigned long long)n_edges, (unsigned long long)cap);
-  std::mt19937_64 rng(order_seed);
   struct Block {
     bool started;
     unsigned index;
     MfStep s;
   };
-  std::vector<Block> live;
-  uint64_t no = 0;
-  int idle = 0;  // steps enqueued past the end, which must stay without edges
-  for (; idle < 2 * SEARCH_AHEAD; no++) {
-    if (no > (uint64_t)n_edges + 2 * SEARCH_AHEAD) return MF_ERR_TIMEOUT;
-    if (c.step[no & 1].n == 0) idle++;
-    live.clear();
-    for (int b = 0; b < grid; b++) live.push_back({false, (unsigned)b, MfStep()});
-    while (!live.empty()) {
-      const size_t at = (size_t)(rng() % live.size());
-      Block &b = live[at];
-      if (!b.started) {
-        b.started = true;
-        b.s = c.step[no & 1];
-        if (b.s.n) continue;
-        if (b.index == 0) mf_search_next(c, (unsigned)no, (unsigned long long)n_edges);
-      } else {
-        // k_expand_edges: expand_range, then the ticket
-        const uint64_t nwarps = (uint64_t)grid * EXPAND_WARPS, n = b.s.n;
-        const uint64_t G = (uint64_t)mf_step_group(d, n, nwarps);
-        for (int wi = 0; wi < EXPAND_WARPS; wi++)
-          for (uint64_t first = (b.index * (uint64_t)EXPAND_WARPS + wi) * G; first < n;
-               first += nwarps * G)
-            for (uint64_t i = first; i < n && i < first + G; i++) {
-              const uint64_t e = b.s.begin + i;
-              if (e >= c.n_edges) return MF_ERR_INVALID;
-              expanded[e]++;
-              c.n_edges = std::min<uint64_t>(c.n_edges + (uint64_t)appends[e], (uint64_t)n_edges);
-            }
-        const unsigned used = mf_step_blocks(n, (int)G, EXPAND_WARPS, (unsigned)grid);
-        if (b.index < used && c.lv_ticket++ == used - 1) {
-          c.lv_ticket = 0;
-          mf_search_next(c, (unsigned)no, (unsigned long long)n_edges);
+  struct Sim {
+    int32_t d, grid;
+    const int32_t *appends;
+    uint64_t n_edges;
+    int64_t refused;
+    int32_t status;
+    int32_t *expanded;
+    MfCounters &c, read[2];
+    std::mt19937_64 rng;
+    std::vector<Block> live;
+    int64_t with_edges;
+    bool drained;
+    int step(uint64_t no) {
+      if (no > n_edges + 4 * SEARCH_AHEAD) return MF_ERR_TIMEOUT;
+      if (refused >= 0 && no >= (uint64_t)refused) return status;
+      if (c.step[no & 1].n) with_edges++;
+      live.clear();
+      for (int b = 0; b < grid; b++) live.push_back({false, (unsigned)b, MfStep()});
+      while (!live.empty()) {
+        const size_t at = (size_t)(rng() % live.size());
+        Block &b = live[at];
+        if (!b.started) {
+          b.started = true;
+          b.s = c.step[no & 1];
+          if (b.s.n) continue;
+          if (b.index == 0) mf_search_next(c, (unsigned)no, n_edges);
+        } else {
+          // k_expand_edges: expand_range, then the ticket
+          const uint64_t nwarps = (uint64_t)grid * EXPAND_WARPS, n = b.s.n;
+          const uint64_t G = (uint64_t)mf_step_group(d, n, nwarps);
+          for (int wi = 0; wi < EXPAND_WARPS; wi++)
+            for (uint64_t first = (b.index * (uint64_t)EXPAND_WARPS + wi) * G; first < n;
+                 first += nwarps * G)
+              for (uint64_t i = first; i < n && i < first + G; i++) {
+                const uint64_t e = b.s.begin + i;
+                if (e >= c.n_edges) return MF_ERR_INVALID;
+                expanded[e]++;
+                c.n_edges = std::min<uint64_t>(c.n_edges + (uint64_t)appends[e], n_edges);
+              }
+          const unsigned used = mf_step_blocks(n, (int)G, EXPAND_WARPS, (unsigned)grid);
+          if (b.index < used && c.lv_ticket++ == used - 1) {
+            c.lv_ticket = 0;
+            mf_search_next(c, (unsigned)no, n_edges);
+          }
         }
+        live[at] = live.back();
+        live.pop_back();
       }
-      live[at] = live.back();
-      live.pop_back();
+      return MF_OK;
     }
-  }
+    int post(int q) {
+      read[q] = c;
+      return MF_OK;
+    }
+    int wait(int q, const MfCounters **r) {
+      *r = &read[q];
+      return MF_OK;
+    }
+    int stalled() { return MF_ERR_CUDA; }
+    void drain() { drained = true; }
+  } sim = {d, grid, appends, (uint64_t)n_edges, refused, status, expanded, c, {},
+           std::mt19937_64(order_seed), {}, 0, false};
+  const int rc = search_run(sim);
   *levels = (int64_t)c.levels;
-  *steps = (int64_t)no - idle;
-  return MF_OK;
+  *steps = sim.with_edges;
+  return rc && !sim.drained ? MF_ERR_INVALID : rc;
 }
 
 extern "C" int mf_vertex_keys(int32_t d, double lambda, const mf_domain *dom, const int32_t *y,

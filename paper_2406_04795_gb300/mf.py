@@ -214,7 +214,7 @@ def load(build_if_missing: bool = True):
     L.mf_diag_exp.argtypes = [V, V, C.c_int64, V, V, V]
     L.mf_diag_search.restype = C.c_int
     L.mf_diag_search.argtypes = [C.c_int32, C.c_int32, C.c_int64, V, C.c_int64, C.c_int64,
-                                 C.c_uint64, V, P(C.c_int64), P(C.c_int64)]
+                                 C.c_uint64, C.c_int64, C.c_int32, V, P(C.c_int64), P(C.c_int64)]
     _lib = L
     return L
 
@@ -421,15 +421,15 @@ def mf_diag_exp(ctx, x_ptr, n, y_table_ptr, y_lib_ptr, stream=0):
     return _check(ctx, load().mf_diag_exp(ctx, x_ptr, n, y_table_ptr, y_lib_ptr, stream))
 
 
-def mf_diag_search(d, grid, cap, appends, n_seed, order_seed):
-    """(times each edge was expanded, levels, steps) of the search's step
-    protocol on a simulated grid (host only)."""
+def mf_diag_search(d, grid, cap, appends, n_seed, order_seed, refused=-1, status=MF_OK):
+    """(times each edge was expanded, levels, steps) of the search's loop and
+    step protocol on a simulated grid (host only)."""
     import numpy as np
     appends = np.ascontiguousarray(appends, dtype=np.int32)
     expanded = np.zeros(appends.size, dtype=np.int32)
     levels, steps = C.c_int64(), C.c_int64()
     rc = load().mf_diag_search(d, grid, cap, appends.ctypes.data_as(C.c_void_p), appends.size,
-                               n_seed, order_seed, expanded.ctypes.data_as(C.c_void_p),
+                               n_seed, order_seed, refused, status, expanded.ctypes.data_as(C.c_void_p),
                                C.byref(levels), C.byref(steps))
     if rc != MF_OK:
         raise MfError(rc, "mf_diag_search")

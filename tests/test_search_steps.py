@@ -1,7 +1,8 @@
 """The search's step protocol (host simulation over the kernels' own functions):
 whatever the order in which the blocks of an edges pass start and finish, those
 without work last among them, every edge is expanded exactly once, in the levels
-of the breadth-first search and in steps of at most the cap."""
+of the breadth-first search and in steps of at most the cap; and a search whose
+kernels the device refuses ends with an error, noticed or not."""
 import numpy as np
 import pytest
 
@@ -35,3 +36,12 @@ def test_every_edge_is_expanded_once_in_any_block_order(d, grid, cap):
 def test_no_seed_edges():
     got, levels, steps = mf.mf_diag_search(3, 8, 100, np.ones(10, np.int32), 0, 1)
     assert not got.any() and (levels, steps) == (0, 0)
+
+
+@pytest.mark.parametrize("refused", [0, 1, 2, 5, 10])
+@pytest.mark.parametrize("status", [mf.MF_OK, mf.MF_ERR_CUDA])
+def test_refused_launches_end_the_search(refused, status):
+    appends = _appends(np.random.default_rng(3), np.array([5, 40, 300, 700, 200, 90, 30, 7, 5, 3, 2, 1, 1]))
+    with pytest.raises(mf.MfError) as e:
+        mf.mf_diag_search(3, 8, 1 << 24, appends, 5, 1, refused=refused, status=status)
+    assert e.value.code == mf.MF_ERR_CUDA
