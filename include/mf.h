@@ -423,10 +423,10 @@ int mf_ctx_get_stats(mf_ctx *ctx, mf_stats *out);
 /* Autotuning (batched multi-trace and single traces; no counterpart in the
  * paper, which runs fixed launch shapes).  mf_autotune traces the request
  * once per BFS-chunk candidate (roots and cells off), then times on that
- * trace the launch variants of the root solve (register cap x grid x group
- * screen size), of the
- * FP64 vertex evaluation (grid) and, for MF_MIXED_BF16, of the tensor-core
- * chunk width (64 or 128 support vectors per MMA).  The fastest of each is
+ * trace the launch variants of the edge-by-edge root solve (register cap x
+ * grid x group screen size; the solve grouped by base vertex takes none of
+ * them), of the FP64 vertex evaluation (grid) and, for MF_MIXED_BF16, of the
+ * tensor-core chunk width (64 or 128 support vectors per MMA).  The fastest of each is
  * kept in the context and used by every later mf_trace on it; *out (host)
  * receives the choices and their times.  Results of earlier traces are
  * invalidated (mf_trace_fetch fails until the next mf_trace). */
@@ -439,7 +439,7 @@ typedef struct {
   double ms_bfs;               /* measured: breadth-first search with the chosen chunk */
   double ms_roots;             /* measured: root solve of the sampled edges */
   double ms_eval;              /* measured: evaluation of every traced vertex */
-  int32_t n_candidates;        /* launch variants timed */
+  int32_t n_candidates;        /* launch variants timed (each of them reaches a launch) */
   int32_t roots_group;         /* consecutive edges sharing one group screen (1: none) */
 } mf_tune;
 int mf_autotune(mf_ctx *ctx, const mf_rbf *rbf, const mf_domain *dom, const mf_trace_opts *opts,

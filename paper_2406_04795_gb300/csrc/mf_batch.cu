@@ -283,7 +283,7 @@ static void launch_slot_roots(mf_ctx *ctx, const std::vector<MfSlot> &slots, con
     B.defer_cap = pools.defer_cap;
     B.defer_list_cap = pools.defer_list_cap;
     B.vert_edges = pools.vert_edges;
-    mf_launch_roots_f64(S.F, S.R, B, edges[t], S.root_tol, MfTune(), sms, st,
+    mf_launch_roots_f64(S.F, S.R, B, edges[t], S.root_tol, ctx->tune, sms, st,
                         mf_root_mode(S.precision, S.flags));
   }
   if (!dims) return;

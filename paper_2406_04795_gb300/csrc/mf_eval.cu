@@ -2300,7 +2300,7 @@ void mf_launch_eval_vertices_mixed(const MfFrame &F, const MfRbfDev &R, const Mf
 }
 
 template <int DD, int MINB>
-static void launch_roots_d(const MfFrame &F, const MfRbfDev &R, const MfTraceBufs &B,
+static bool launch_roots_d(const MfFrame &F, const MfRbfDev &R, const MfTraceBufs &B,
                            uint64_t n_edges, double tol, int grid, int group, MfRootMode mode,
                            int sms, cudaStream_t st) {
   const int fast = mode.fast ? 1 : 0;
@@ -2309,7 +2309,7 @@ static void launch_roots_d(const MfFrame &F, const MfRbfDev &R, const MfTraceBuf
   if (!B.defer_rec || B.defer_cap == 0) {
     k_roots_f64<DD, MINB><<<grid, ROOT_WARPS * 32, dyn, st>>>(F, R, B, 0, n_edges, tol, group, fast,
                                                              0, nullptr, nullptr);
-    return;
+    return true;
   }
   // chunks of defer_cap edges: the FP32 stage (per base vertex where the
   // vertices have lists; else the warp kernel, deferring the common
@@ -2337,26 +2337,28 @@ static void launch_roots_d(const MfFrame &F, const MfRbfDev &R, const MfTraceBuf
     k_roots_f64<DD, MINB><<<sms * 4, ROOT_WARPS * 32, 0, st>>>(F, R, B, 0, B.defer_cap, tol, 1,
                                                               fast, 0, B.redo, &B.cnt->n_redo);
   }
+  return !grouped;
 }
 
 template <int MINB>
-static void launch_roots(const MfFrame &F, const MfRbfDev &R, const MfTraceBufs &B, uint64_t n_edges,
+static bool launch_roots(const MfFrame &F, const MfRbfDev &R, const MfTraceBufs &B, uint64_t n_edges,
                          double tol, int grid, int group, MfRootMode mode, int sms, cudaStream_t st) {
   switch (F.d) {
 #define MF_CASE(DD) \
-  case DD: launch_roots_d<DD, MINB>(F, R, B, n_edges, tol, grid, group, mode, sms, st); break;
+  case DD: return launch_roots_d<DD, MINB>(F, R, B, n_edges, tol, grid, group, mode, sms, st);
     MF_CASE(2) MF_CASE(3) MF_CASE(4) MF_CASE(5) MF_CASE(6) MF_CASE(7)
 #undef MF_CASE
-    default: launch_roots_d<MF_MAXD, MINB>(F, R, B, n_edges, tol, grid, group, mode, sms, st);
+    default: return launch_roots_d<MF_MAXD, MINB>(F, R, B, n_edges, tol, grid, group, mode, sms, st);
   }
 }
 
-void mf_launch_roots_f64(const MfFrame &F, const MfRbfDev &R, const MfTraceBufs &B, uint64_t n_edges,
+bool mf_launch_roots_f64(const MfFrame &F, const MfRbfDev &R, const MfTraceBufs &B, uint64_t n_edges,
                          double tol, const MfTune &T, int sms, cudaStream_t st, MfRootMode mode) {
-  if (n_edges == 0) return;
+  if (n_edges == 0) return false;
   const int grid = sms * T.roots_bps;
-  if (T.roots_variant == 1) launch_roots<3>(F, R, B, n_edges, tol, grid, T.roots_group, mode, sms, st);
-  else launch_roots<2>(F, R, B, n_edges, tol, grid, T.roots_group, mode, sms, st);
+  return T.roots_variant == 1
+             ? launch_roots<3>(F, R, B, n_edges, tol, grid, T.roots_group, mode, sms, st)
+             : launch_roots<2>(F, R, B, n_edges, tol, grid, T.roots_group, mode, sms, st);
 }
 
 // ---------------------------------------------------------------------------

@@ -764,7 +764,9 @@ static inline MfRootMode mf_root_mode(int precision, uint32_t flags) {
   const bool fast = precision != MF_FP64 && !(flags & MF_ROOTS_FP64_EXACT);
   return {fast, !(fast && precision == MF_MIXED_FP32)};
 }
-void mf_launch_roots_f64(const MfFrame &F, const MfRbfDev &R, const MfTraceBufs &B,
+// Returns whether the choices of T reached the solve (they shape the per-edge
+// kernel; the grouped one takes none of them).
+bool mf_launch_roots_f64(const MfFrame &F, const MfRbfDev &R, const MfTraceBufs &B,
                          uint64_t n_edges, double tol, const MfTune &T, int sms, cudaStream_t st,
                          MfRootMode mode);
 // The pools of its deferred steps in context slot `slot`; false when the budget

@@ -3,8 +3,9 @@
 //
 // Candidates:
 //   BFS chunk (edges per expansion step): the batch cap, 2^20, 2^18;
-//   root solve: register cap (2 or 3 blocks per SM) x grid (2, 4, 8 blocks
-//     per SM) x group screen (1, 8, 16 edges), on the first 2^20 traced edges;
+//   root solve edge by edge: register cap (2 or 3 blocks per SM) x grid (2, 4,
+//     8 blocks per SM) x group screen (1, 8, 16 edges), on the first 2^20 traced
+//     edges;
 //   FP64 vertex evaluation: grid (4, 8, 16 blocks per SM), all vertices;
 //   tensor-core evaluation (MF_MIXED_BF16): chunk width 64 or 128.
 // Each kernel candidate is timed three times with CUDA events on the
@@ -140,11 +141,14 @@ extern "C" int mf_autotune(mf_ctx *ctx, const mf_rbf *rbf, const mf_domain *dom,
   if (!L.valid) return mf_set_error(ctx, MF_ERR_INVALID, "mf_autotune: the trace left no state");
   const int sms = ctx->sms;
 
-  // 2. root solve on the first 2^20 edges
+  // 2. root solve on the first 2^20 edges, edge by edge: the grouped solve takes
+  // none of these choices, but slots and precisions that are not grouped, and
+  // edges without lists, do
   const uint64_t es = L.n_edges < (int64_t)(1 << 20) ? (uint64_t)L.n_edges : (1ull << 20);
   float best_roots = 1e30f;
   if (es > 0) {
     MfTune best = ctx->tune;
+    const MfRootMode mode = mf_root_mode(L.precision, L.flags), per_edge = {mode.fast, false};
     const int bps[3] = {2, 4, 8}, groups[3] = {1, 8, 16};
     for (int v = 0; v < 2; v++)
       for (int g = 0; g < 3; g++)
@@ -153,11 +157,12 @@ extern "C" int mf_autotune(mf_ctx *ctx, const mf_rbf *rbf, const mf_domain *dom,
           t.roots_variant = v;
           t.roots_bps = bps[g];
           t.roots_group = groups[q];
+          bool tuned = false;
           const float ms = time_ms(
               st, [&]() {
-                mf_launch_roots_f64(L.F, L.R, L.B, es, L.tol, t, sms, st,
-                                    mf_root_mode(L.precision, L.flags));
+                tuned = mf_launch_roots_f64(L.F, L.R, L.B, es, L.tol, t, sms, st, per_edge);
               }, 3);
+          if (!tuned) continue;
           n_cand++;
           if (ms < best_roots) {
             best_roots = ms;
@@ -167,6 +172,9 @@ extern "C" int mf_autotune(mf_ctx *ctx, const mf_rbf *rbf, const mf_domain *dom,
     ctx->tune.roots_variant = best.roots_variant;
     ctx->tune.roots_bps = best.roots_bps;
     ctx->tune.roots_group = best.roots_group;
+    // what a trace's own solve takes with them
+    best_roots = time_ms(
+        st, [&]() { mf_launch_roots_f64(L.F, L.R, L.B, es, L.tol, ctx->tune, sms, st, mode); }, 3);
   }
 
   // 3. vertex evaluation of every traced vertex, through scratch counters
