@@ -239,15 +239,22 @@ int mf_finish_trace(mf_ctx *ctx, const mf_rbf *rbf, const mf_trace_opts *o, cons
 // kernel per dimension, as do all slots when the pools don't fit the budget.
 // d_only: device words for the mask, n of them; the mask is kept in `mask`
 // until the stream has been waited for.
+// fixed: pools of that size whatever the slots (a slot with more vertices takes
+// the batched kernel), else as the largest slot needs them.
 #define ROOTS_ALONE 8192
+struct RootPools {
+  uint64_t chunk, verts;
+};
 static void launch_slot_roots(mf_ctx *ctx, const std::vector<MfSlot> &slots, const MfSlot *d_slots,
                               MfBatchPlan *d_plan, const std::vector<int> &which,
                               const std::vector<unsigned long long> &edges, int32_t *d_only,
-                              std::vector<int32_t> &mask, int sms, cudaStream_t st) {
+                              std::vector<int32_t> &mask, const RootPools *fixed, int sms,
+                              cudaStream_t st) {
   uint64_t most = 0, verts = 0;
   int dmax = 0;
   auto large = [&](int t) {
     return slots[t].B.vlist && edges[t] >= ROOTS_ALONE &&
+           (!fixed || slots[t].B.max_vertices <= fixed->verts) &&
            mf_root_mode(slots[t].precision, slots[t].flags).grouped;
   };
   for (int t : which) {
@@ -258,8 +265,11 @@ static void launch_slot_roots(mf_ctx *ctx, const std::vector<MfSlot> &slots, con
   }
   MfTraceBufs pools;
   memset(&pools, 0, sizeof(pools));
-  const bool alone = most > 0 && mf_setup_root_pools(ctx, MF_SLOT_BATCHROOTS, dmax,
-                                                     std::min<uint64_t>(most, 1ull << 22), verts, &pools);
+  const bool alone =
+      most > 0 && (fixed ? mf_setup_root_pools(ctx, MF_SLOT_BATCHROOTS, MF_MAXD, fixed->chunk,
+                                               fixed->verts, &pools)
+                         : mf_setup_root_pools(ctx, MF_SLOT_BATCHROOTS, dmax,
+                                               std::min<uint64_t>(most, 1ull << 22), verts, &pools));
   mask.assign(slots.size(), 0);
   uint32_t dims = 0;
   for (int t : which) {
@@ -401,7 +411,7 @@ extern "C" int mf_trace_batch(mf_ctx *ctx, int32_t n, const mf_rbf *rbfs, const 
       n_edges[t] = hs[t].level_end;
     }
     launch_slot_roots(ctx, slots, d_slots, d_plan, all, n_edges, (int32_t *)(arena + off_only),
-                      root_mask, sms, st);
+                      root_mask, nullptr, sms, st);
   }
   bool any_cells = false;
   for (int t = 0; t < n; t++) any_cells = any_cells || (opts[t].flags & MF_WANT_CELLS);
@@ -593,6 +603,7 @@ struct mf_server {
   char *arena = nullptr;
   size_t arena_bytes = 0, data_off = 0;
   RangeAlloc alloc;
+  RootPools roots = {};  // of the finished traces' root solve, taken at creation
   MfSlot *d_slots = nullptr;
   MfSlotState *d_state = nullptr;
   MfBatchPlan *d_plan = nullptr;
@@ -637,6 +648,17 @@ extern "C" int mf_server_create(mf_ctx *ctx, int32_t max_slots, size_t hbm_bytes
   s->d_plan = (MfBatchPlan *)(s->arena + o_plan);
   s->d_only = (int32_t *)(s->arena + o_only);
   s->alloc.init(hbm_bytes - s->data_off);
+  // The root pools, once and beside the arena: about 4 % of it, chunks of 2^16
+  // to 2^22 edges, and at least the vertices of a request's default capacity
+  // four times over.  Growing them as larger traces finished stopped every
+  // running request for a cudaFree and a cudaMalloc of up to some GB each time.
+  // A budget that refuses them leaves the roots to the batched kernel.
+  s->roots.chunk = std::min<uint64_t>(std::max<uint64_t>(hbm_bytes >> 14, 1ull << 16), 1ull << 22);
+  s->roots.verts = std::max<uint64_t>(4 * s->roots.chunk, 1ull << 22);
+  {
+    MfTraceBufs pools;
+    mf_setup_root_pools(ctx, MF_SLOT_BATCHROOTS, MF_MAXD, s->roots.chunk, s->roots.verts, &pools);
+  }
   s->slots.assign(max_slots, MfSlot());
   memset(s->slots.data(), 0, sizeof(MfSlot) * max_slots);
   s->slot_req.assign(max_slots, -1);
@@ -864,8 +886,8 @@ extern "C" int mf_server_step(mf_server *s, void *stream, int32_t *n_running, in
       n_edges[t] = s->hstate[t].level_end;
     }
     std::vector<int32_t> root_mask;
-    launch_slot_roots(ctx, s->slots, s->d_slots, s->d_plan, fin, n_edges, s->d_only, root_mask, sms,
-                      st);
+    launch_slot_roots(ctx, s->slots, s->d_slots, s->d_plan, fin, n_edges, s->d_only, root_mask,
+                      &s->roots, sms, st);
     cudaMemcpyAsync(s->d_only, only.data(), sizeof(int32_t) * n, cudaMemcpyHostToDevice, st);
     bool cells = false;
     for (int t : fin) cells = cells || (s->slots[t].flags & MF_WANT_CELLS);

@@ -773,6 +773,7 @@ bool mf_launch_roots_f64(const MfFrame &F, const MfRbfDev &R, const MfTraceBufs 
 // refuses.
 bool mf_setup_root_pools(mf_ctx *ctx, int slot, int d, uint64_t chunk, uint64_t n_vert,
                          MfTraceBufs *B);
+size_t mf_root_pool_bytes(int d, uint64_t chunk, uint64_t n_vert);
 void mf_launch_eval_vertices_tc(const MfFrame &F, const MfRbfDev &R, const MfTraceBufs &B,
                                 double band, int n_chunk, int sms, cudaStream_t st);
 

@@ -1579,15 +1579,19 @@ static int read_counters(mf_ctx *ctx, const MfTraceBufs &B, cudaStream_t st) {
 // on average (when the budget allows; else every step runs in the
 // warp-per-edge kernel), and n_vert words for B->vert_edges where the trace
 // has none of its own.
+size_t mf_root_pool_bytes(int d, uint64_t dc, uint64_t n_vert) {
+  auto al = [](size_t x) { return (x + 255) & ~(size_t)255; };
+  const uint64_t dl = dc * 48;
+  return al(dc * 32) + al(dc * 8) + al(dl * 4) + al(dc * MF_EP_ROW(d) * 4) + al(dc * 2 * d * 8) +
+         al(dc * 3 * d * 4) + al(dl) + al(dl / 2) + al(dl / 2) + al(n_vert * 4);
+}
+
 bool mf_setup_root_pools(mf_ctx *ctx, int slot, int d, uint64_t dc, uint64_t n_vert,
                          MfTraceBufs *B) {
   auto al = [](size_t x) { return (x + 255) & ~(size_t)255; };
   const uint64_t dl = dc * 48;
-  const size_t db = al(dc * 32) + al(dc * 8) + al(dl * 4) + al(dc * MF_EP_ROW(d) * 4) +
-                    al(dc * 2 * d * 8) + al(dc * 3 * d * 4) + al(dl) + al(dl / 2) + al(dl / 2) +
-                    al(n_vert * 4);
   const std::string keep = ctx->err;
-  char *q = (char *)mf_ctx_buffer(ctx, slot, db);
+  char *q = (char *)mf_ctx_buffer(ctx, slot, mf_root_pool_bytes(d, dc, n_vert));
   if (!q) {
     ctx->err = keep;
     return false;
