@@ -2,7 +2,7 @@
 // (precision MF_MIXED_BF16): the RBF decision function of Sec. IV-A with its
 // distance term computed as a GEMM.
 //
-// A CTA evaluates tiles of 128 vertices.  With y0 the tile's first vertex,
+// A CTA evaluates tiles of 128 vertices.  With y0 the mean of the tile's vertices,
 // q0 = x(y0), dy = y - y0 (small integers) and u_j = q0 - s_j,
 //   |q - s_j|^2 = |u_j|^2 + dy . w_j + |lam L dy|^2,     w_j = 2 lam L u_j
 // (L = I - c 11^T is symmetric).  Per chunk of 64 support vectors one
@@ -50,7 +50,8 @@ struct TcShared {
   uint64_t bar[2];
   uint32_t tmem;
   int timeout;
-  int32_t y0[MF_MAXD], ysum[TC_M / 32][MF_MAXD];
+  int32_t y0[MF_MAXD];
+  int64_t ysum[TC_M / 32][MF_MAXD];
   float q0hi[MF_MAXD], q0lo[MF_MAXD];
 };
 
@@ -116,13 +117,16 @@ __device__ __forceinline__ bool tc_tile(const MfFrame &F, const MfRbfDev &R, con
   for (int k = 0; k < D; k++) y[k] = valid ? B.vert_y[v * D + k] : 0;
   // the tile base: the mean of the tile's vertices, rounded.  The rounding of
   // D grows with the square of a vertex's distance from the base, which the
-  // mean halves against the tile's first vertex.
+  // mean halves against the tile's first vertex.  Summed as two halves of 16
+  // bits: coordinates reach 2^30, and a base off by a wrapped sum sends the
+  // whole tile to the FP64 recheck.
   {
     const int64_t n = (int64_t)min((uint64_t)TC_M, v_end - v_first);
 #pragma unroll
     for (int k = 0; k < D; k++) {
-      const int s = __reduce_add_sync(0xffffffffu, valid ? y[k] : 0);
-      if ((t & 31) == 0) sh.ysum[w][k] = s;
+      const int hi = __reduce_add_sync(0xffffffffu, valid ? y[k] >> 16 : 0);
+      const int lo = __reduce_add_sync(0xffffffffu, valid ? y[k] & 0xffff : 0);
+      if ((t & 31) == 0) sh.ysum[w][k] = (int64_t)hi * 65536 + lo;
     }
     __syncthreads();
     if (t == 0) {
