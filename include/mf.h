@@ -473,6 +473,13 @@ int mf_probe_rates(mf_ctx *ctx, mf_rates *out, void *stream);
 int mf_diag_exp(mf_ctx *ctx, const double *x, int64_t n, double *y_table, double *y_lib,
                 void *stream);
 
+/* The context's device arena on a fake device (host only, no GPU needed): asks
+ * a context of that budget, on a device with device_bytes left, for n buffers
+ * in turn, bytes[i] in slot slots[i].  held[2 i] receives the slot's bytes (0:
+ * refused), held[2 i + 1] all bytes that the context then holds. */
+int mf_diag_arena(uint64_t budget, uint64_t device_bytes, int32_t n, const int32_t *slots,
+                  const uint64_t *bytes, uint64_t *held);
+
 /* The search's loop and step protocol on a simulated grid (host only, no GPU
  * needed): edges 0 .. n_seed - 1 form the first level, expanding edge e appends
  * appends[e] further ones (up to n_edges in all), and each step's edges pass

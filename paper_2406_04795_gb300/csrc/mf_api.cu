@@ -4,6 +4,7 @@
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
+#include <map>
 #include <string>
 
 #include "mf_internal.cuh"
@@ -130,33 +131,37 @@ int mf_cuda_check(mf_ctx *c, cudaError_t e, const char *what) {
 
 int mf_ctx_sm_count(mf_ctx *c) { return c->sms; }
 
+static void drop_slot(mf_ctx *c, int slot) {
+  if (!c->slot_ptr[slot]) return;
+  c->mem->release(c->slot_ptr[slot]);
+  c->slot_ptr[slot] = nullptr;
+  c->total -= c->slot_bytes[slot];
+  c->slot_bytes[slot] = 0;
+}
+
+// A slot that finds no room takes it from MF_SLOT_BATCHROOTS, whether it is the
+// budget that refuses or the device (whose other users can leave less than the
+// budget).
 void *mf_ctx_buffer(mf_ctx *c, int slot, size_t bytes) {
   bytes = (bytes + 255) & ~(size_t)255;
   if (bytes == 0) bytes = 256;
   if (c->slot_bytes[slot] >= bytes) return c->slot_ptr[slot];
-  if (slot != MF_SLOT_BATCHROOTS && c->slot_ptr[MF_SLOT_BATCHROOTS] &&
-      c->total - c->slot_bytes[slot] + bytes > c->budget) {
-    cudaDeviceSynchronize();
-    cudaFree(c->slot_ptr[MF_SLOT_BATCHROOTS]);
-    c->slot_ptr[MF_SLOT_BATCHROOTS] = nullptr;
-    c->total -= c->slot_bytes[MF_SLOT_BATCHROOTS];
-    c->slot_bytes[MF_SLOT_BATCHROOTS] = 0;
-  }
+  if (slot != MF_SLOT_BATCHROOTS && c->total - c->slot_bytes[slot] + bytes > c->budget)
+    drop_slot(c, MF_SLOT_BATCHROOTS);
   size_t others = c->total - c->slot_bytes[slot];
   if (others + bytes > c->budget) {
     mf_set_error(c, MF_ERR_OOM, "HBM budget: need %zu more bytes (budget %zu, held %zu)",
                  bytes - c->slot_bytes[slot], c->budget, c->total);
     return nullptr;
   }
-  if (c->slot_ptr[slot]) {
-    cudaDeviceSynchronize();
-    cudaFree(c->slot_ptr[slot]);
-    c->slot_ptr[slot] = nullptr;
-    c->total -= c->slot_bytes[slot];
-    c->slot_bytes[slot] = 0;
-  }
+  drop_slot(c, slot);
   void *p = nullptr;
-  cudaError_t e = cudaMalloc(&p, bytes);
+  cudaError_t e = c->mem->alloc(&p, bytes);
+  if (e != cudaSuccess && slot != MF_SLOT_BATCHROOTS && c->slot_ptr[MF_SLOT_BATCHROOTS]) {
+    cudaGetLastError();
+    drop_slot(c, MF_SLOT_BATCHROOTS);
+    e = c->mem->alloc(&p, bytes);
+  }
   if (e != cudaSuccess) {
     cudaGetLastError();
     mf_set_error(c, MF_ERR_OOM, "cudaMalloc(%zu) failed: %s", bytes, cudaGetErrorString(e));
@@ -166,6 +171,40 @@ void *mf_ctx_buffer(mf_ctx *c, int slot, size_t bytes) {
   c->slot_bytes[slot] = bytes;
   c->total += bytes;
   return p;
+}
+
+extern "C" int mf_diag_arena(uint64_t budget, uint64_t device_bytes, int32_t n,
+                             const int32_t *slots, const uint64_t *bytes, uint64_t *held) {
+  if (n < 0 || !slots || !bytes || !held) return MF_ERR_INVALID;
+  for (int i = 0; i < n; i++)
+    if (slots[i] < 0 || slots[i] >= MF_NUM_SLOTS) return MF_ERR_INVALID;
+  struct Fake : MfDevMem {
+    uint64_t left;
+    std::map<void *, size_t> taken;
+    uintptr_t next = 4096;
+    cudaError_t alloc(void **p, size_t b) override {
+      if (b > left) return cudaErrorMemoryAllocation;
+      left -= b;
+      *p = (void *)next;
+      next += 4096;
+      taken[*p] = b;
+      return cudaSuccess;
+    }
+    void release(void *p) override {
+      left += taken[p];
+      taken.erase(p);
+    }
+  } fake;
+  fake.left = device_bytes;
+  mf_ctx c;
+  c.mem = &fake;
+  c.budget = (size_t)budget;
+  for (int i = 0; i < n; i++) {
+    const bool got = mf_ctx_buffer(&c, slots[i], (size_t)bytes[i]) != nullptr;
+    held[2 * i] = got ? (uint64_t)c.slot_bytes[slots[i]] : 0;
+    held[2 * i + 1] = (uint64_t)c.total;
+  }
+  return MF_OK;
 }
 
 // ---------------------------------------------------------------------------

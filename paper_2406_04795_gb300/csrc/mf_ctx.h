@@ -55,7 +55,18 @@ struct MfProfiler {
   size_t used = 0;
 };
 
+// Where the context's slots come from (a host fake in mf_diag_arena).
+struct MfDevMem {
+  virtual ~MfDevMem() {}
+  virtual cudaError_t alloc(void **p, size_t bytes) { return cudaMalloc(p, bytes); }
+  virtual void release(void *p) {  // waits for what may still use it
+    cudaDeviceSynchronize();
+    cudaFree(p);
+  }
+};
+
 struct mf_ctx {
+  MfDevMem cuda_mem, *mem = &cuda_mem;
   int device = 0;
   int sms = 0;
   size_t budget = 0;

@@ -42,7 +42,7 @@ EXPORTS = ("mf_ctx_create", "mf_ctx_destroy", "mf_last_error", "mf_ctx_bytes", "
            "mf_server_status", "mf_server_fetch", "mf_server_done", "mf_autotune", "mf_ctx_set_tune",
            "mf_ctx_get_tune", "mf_vertex_keys", "mf_probe_rates", "mf_diag_exp",
            "mf_certify_ex", "mf_subdiv_begin", "mf_subdiv_next",
-           "mf_server_wait", "mf_diag_search")
+           "mf_server_wait", "mf_diag_search", "mf_diag_arena")
 
 MF_PHASES = 12
 PHASE_NAMES = ("prepare", "seeds", "expand_vertices", "eval", "expand_edges", "roots", "cells",
@@ -212,6 +212,8 @@ def load(build_if_missing: bool = True):
     L.mf_probe_rates.argtypes = [V, P(mf_rates), V]
     L.mf_diag_exp.restype = C.c_int
     L.mf_diag_exp.argtypes = [V, V, C.c_int64, V, V, V]
+    L.mf_diag_arena.restype = C.c_int
+    L.mf_diag_arena.argtypes = [C.c_uint64, C.c_uint64, C.c_int32, V, V, V]
     L.mf_diag_search.restype = C.c_int
     L.mf_diag_search.argtypes = [C.c_int32, C.c_int32, C.c_int64, V, C.c_int64, C.c_int64,
                                  C.c_uint64, C.c_int64, C.c_int32, V, P(C.c_int64), P(C.c_int64)]
@@ -419,6 +421,20 @@ def mf_probe_rates(ctx, stream=0) -> mf_rates:
 
 def mf_diag_exp(ctx, x_ptr, n, y_table_ptr, y_lib_ptr, stream=0):
     return _check(ctx, load().mf_diag_exp(ctx, x_ptr, n, y_table_ptr, y_lib_ptr, stream))
+
+
+def mf_diag_arena(budget, device_bytes, requests):
+    """[(slot's bytes, 0 when refused; bytes held by the context)] of buffer
+    requests [(slot, bytes)] on a fake device (host only)."""
+    import numpy as np
+    slots = np.array([r[0] for r in requests], np.int32)
+    size = np.array([r[1] for r in requests], np.uint64)
+    held = np.zeros((len(requests), 2), np.uint64)
+    rc = load().mf_diag_arena(budget, device_bytes, len(requests), slots.ctypes.data_as(C.c_void_p),
+                              size.ctypes.data_as(C.c_void_p), held.ctypes.data_as(C.c_void_p))
+    if rc != MF_OK:
+        raise MfError(rc, "mf_diag_arena")
+    return [tuple(int(v) for v in r) for r in held]
 
 
 def mf_diag_search(d, grid, cap, appends, n_seed, order_seed, refused=-1, status=MF_OK):
