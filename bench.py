@@ -47,12 +47,14 @@ def df_term_ops(d):
     return 47 * d + 68
 
 
-# FP32-pipe operations of one FP32 term of the root solve (k_rg_solve: a listed
-# vector in one evaluation at t): the exponent P + t (Q + t c) (2), ex2, alpha e,
-# e Q and the three moments (6); the coordinates enter once per vertex and edge,
-# so none of them is counted
-def f32_term_ops(d):
-    return 8
+# FP32-pipe operations of one FP32 term of the root solve.  Grouped by base vertex
+# (k_rg_solve: a listed vector in one evaluation at t): the exponent
+# P + t (Q + t c) (2), ex2, alpha e, e Q and the three moments (6); the
+# coordinates enter once per vertex and edge (Q: d + 1 more per listed vector,
+# whatever the evaluations) and are not counted.  Edge by edge (k_roots_f64, which
+# MF_MIXED_FP32 traces take): as a term of the vertex evaluation below.
+def f32_term_ops(d, grouped=True):
+    return 8 if grouped else 5 * d + 8
 
 
 # The same of one FP32 term of the vertex evaluation: per coordinate a hi and a
@@ -163,8 +165,9 @@ def roofline(stats, w, rates, E, ms_proof, n_proofs, root_traffic=True):
     # terms; FP32 Halley and weak terms) and of the evaluation's weak terms,
     # ex2 of all FP32 terms, and the algorithmic bytes of the table phases
     f64 = stats["eval"]["terms"] * per_eval
+    f32_ops = f32_term_ops(d, grouped=w.precision != "mixed_fp32")
     f32 = (stats["roots"]["terms"] * df_term_ops(d) +
-           stats["roots"]["terms_weak"] * f32_term_ops(d) +
+           stats["roots"]["terms_weak"] * f32_ops +
            stats["eval"]["terms_weak"] * eval_f32_term_ops(d))
     ex2 = stats["roots"]["terms_weak"] + stats["eval"]["terms_weak"]
     k = d // 2
@@ -199,7 +202,7 @@ def roofline(stats, w, rates, E, ms_proof, n_proofs, root_traffic=True):
         # the root phase's arithmetic runs on the FP32 pipe: double-float
         # strong terms (k_roots_terms) and FP32 Halley / weak terms
         # (k_rg_solve); the few full FP64 re-evaluations are counted as strong terms
-        ops = (s["terms"] * df_term_ops(d) + s["terms_weak"] * f32_term_ops(d)) / max(s["launches"], 1)
+        ops = (s["terms"] * df_term_ops(d) + s["terms_weak"] * f32_ops) / max(s["launches"], 1)
         ach = ops / (ms_per_launch * 1e-3) / 1e12
         # DRAM bytes per edge from the ncu capture of the root kernels
         # (profiles/), scaled by the edges one launch processes
@@ -214,7 +217,7 @@ def roofline(stats, w, rates, E, ms_proof, n_proofs, root_traffic=True):
                     peak_source="measured: mf_probe_rates FP32 FMA probe (one operation per "
                     "instruction)",
                     work="%d strong terms x %d FP32 ops (double-float) + %d FP32 terms x %d ops" % (
-                        s["terms"], df_term_ops(d), s["terms_weak"], f32_term_ops(d)))
+                        s["terms"], df_term_ops(d), s["terms_weak"], f32_ops))
     if dom == "eval":
         flops = s["terms"] * per_eval / max(s["launches"], 1)
         ach = flops / (ms_per_launch * 1e-3) / 1e12

@@ -197,7 +197,7 @@ struct RgCtx {
 // each holding K entries of the list, zeros past its end.
 template <int D, int W, int K, int CAP>
 __device__ __forceinline__ void rg_solve(const RgCtx &c, uint32_t off, uint32_t n,
-                                         unsigned long long &nterms) {
+                                         uint32_t &nterms) {
   constexpr int NSUB = 32 / W;
   const int lane = threadIdx.x & 31, sl = lane & (W - 1), q = lane / W;
   const RgScratch sc = rg_scratch(c.B);
@@ -243,6 +243,7 @@ __device__ __forceinline__ void rg_solve(const RgCtx &c, uint32_t off, uint32_t 
     if (!(t32 > 0.f && t32 < 1.f)) t32 = 0.5f;
     float lo = 0.f, hi = 1.f, gpp = INFINITY;
     bool done = false;
+    if (have && sl == 0) nterms += c.nl;  // the last evaluation
     for (int step_no = 0; step_no < 12; step_no++) {
       float m0 = 0.f, m1 = 0.f, m2 = 0.f, none = 0.f;
 #pragma unroll
@@ -253,7 +254,7 @@ __device__ __forceinline__ void rg_solve(const RgCtx &c, uint32_t off, uint32_t 
         m1 += eq;
         m2 = fmaf(eq, Q[k], m2);
       }
-      nterms += c.nl * min((uint32_t)NSUB, n - i0);
+      if (have && sl == 0 && !done) nterms += c.nl;
       sub_sum4<W>(m0, m1, m2, none);
       if (!done) {
         const float td = t32 * dd;
@@ -386,7 +387,9 @@ __global__ void __launch_bounds__(RG_WARPS * 32, RgClass<CLS>::BLOCKS) k_rg_solv
   const RgScratch sc = rg_scratch(B);
   const uint64_t ng = B.cnt->n_groups[CLS];
   const uint64_t nwarps = (uint64_t)gridDim.x * RG_WARPS;
-  unsigned long long nterms = 0;
+  // the lane's FP32 terms: at most 13 evaluations of 512 for each edge of the
+  // warp's share of a chunk, far below 2^32
+  uint32_t nterms = 0;
   for (uint64_t g = blockIdx.x * (uint64_t)RG_WARPS + w; g < ng; g += nwarps) {
     const RgGroup gr = CLS == 0 ? sc.group[g] : CLS == 1 ? sc.mid[g] : sc.group[B.defer_cap - 1 - g];
     const int nl = (int)B.vlist_n[gr.vi];
@@ -456,7 +459,8 @@ __global__ void __launch_bounds__(RG_WARPS * 32, RgClass<CLS>::BLOCKS) k_rg_solv
       else rg_solve<D, 16, RG_SMALL / 16, CAP>(c, gr.off, gr.n, nterms);
     }
   }
-  if (lane == 0 && nterms) atomicAdd(&B.cnt->root_terms_weak, nterms);
+  const unsigned long long all = mf_warp_sum_ull(nterms);
+  if (lane == 0 && all) atomicAdd(&B.cnt->root_terms_weak, all);
 }
 
 template <int D, int CLS>
