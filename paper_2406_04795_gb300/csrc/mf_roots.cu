@@ -171,13 +171,6 @@ __device__ __forceinline__ void sub_sum4(float &a, float &b, float &c, float &e)
   e = __shfl_sync(FULL, z, 3 * W / 4, W);
 }
 
-template <int W>
-__device__ __forceinline__ float sub_sum(float v) {
-#pragma unroll
-  for (int o = W / 2; o; o >>= 1) v += __shfl_xor_sync(FULL, v, o);
-  return v;
-}
-
 // Per warp: u, P and alpha of the list (CAP entries each, D + 2 arrays), padded
 // with zeros to the W K entries that the lanes hold.
 struct RgCtx {
