@@ -833,14 +833,15 @@ __global__ void k_advance_eval(MfCounters *c) {
 #define MIX_WARPS 8
 #define MIX_TILE 256
 
+// Followed in shared memory by each warp's tile, [axis, then alpha][MIX_TILE]
+// (the launch reserves one for each of its warps).
 template <int D>
-struct MixShared {
+struct __align__(16) MixShared {
   double x[D][32];
   float part[MIX_WARPS][32], A[MIX_WARPS][32], Q[MIX_WARPS][32];
-  // [warp][axis, then alpha][MIX_TILE], 16-byte rows; the launch reserves it
-  // for its own number of warps
-  __align__(16) float sv[1][D + 1][MIX_TILE];
 };
+template <int D>
+using MixTile = float[D + 1][MIX_TILE];
 
 // Source of points: vertex list (lattice) or a plain [n][d] array.
 template <bool VERTS, int D>
@@ -851,6 +852,7 @@ __global__ void __launch_bounds__(MIX_WARPS * 32) k_eval_mixed_f32(MfFrame F, Mf
   extern __shared__ __align__(16) unsigned char mix_raw[];
   MixShared<D> &sh = *reinterpret_cast<MixShared<D> *>(mix_raw);
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, W = blockDim.x >> 5;
+  MixTile<D> &sv = reinterpret_cast<MixTile<D> *>(mix_raw + sizeof(MixShared<D>))[w];
   mf_dep_wait();
   uint64_t begin = 0, end = (uint64_t)npts;
   if (VERTS) {
@@ -898,8 +900,8 @@ __global__ void __launch_bounds__(MIX_WARPS * 32) k_eval_mixed_f32(MfFrame F, Mf
         for (int i = lane; i < cnt4; i += 32) {
           const bool in = i < cnt;  // the padding adds zeros
 #pragma unroll
-          for (int k = 0; k < D; k++) sh.sv[w][k][i] = in ? R.sv32[(int64_t)k * R.n + j0 + i] : 0.f;
-          sh.sv[w][D][i] = in ? R.alpha32[j0 + i] : 0.f;
+          for (int k = 0; k < D; k++) sv[k][i] = in ? R.sv32[(int64_t)k * R.n + j0 + i] : 0.f;
+          sv[D][i] = in ? R.alpha32[j0 + i] : 0.f;
         }
         __syncwarp();
 #pragma unroll 2
@@ -907,12 +909,12 @@ __global__ void __launch_bounds__(MIX_WARPS * 32) k_eval_mixed_f32(MfFrame F, Mf
           float r2[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
           for (int k = 0; k < D; k++) {
-            const float4 s = *reinterpret_cast<const float4 *>(&sh.sv[w][k][j]);
+            const float4 s = *reinterpret_cast<const float4 *>(&sv[k][j]);
             const float t[4] = {xs[k] - s.x, xs[k] - s.y, xs[k] - s.z, xs[k] - s.w};
 #pragma unroll
             for (int i = 0; i < 4; i++) r2[i] = fmaf(t[i], t[i], r2[i]);
           }
-          const float4 a4 = *reinterpret_cast<const float4 *>(&sh.sv[w][D][j]);
+          const float4 a4 = *reinterpret_cast<const float4 *>(&sv[D][j]);
           const float al[4] = {a4.x, a4.y, a4.z, a4.w};
 #pragma unroll
           for (int i = 0; i < 4; i++) {
@@ -983,7 +985,7 @@ static void launch_mixed_f32_d(const MfFrame &F, const MfRbfDev &R, const MfTrac
                                const double *pts, int64_t npts, double *fout, uint8_t *flag,
                                double band, int sms, cudaStream_t st) {
   const int W = std::min(MIX_WARPS, (R.n + MIX_TILE - 1) / MIX_TILE);
-  const int bytes = (int)(sizeof(MixShared<D>) + (W - 1) * sizeof(MixShared<D>::sv));
+  const int bytes = (int)(sizeof(MixShared<D>) + W * sizeof(MixTile<D>));
   cudaFuncSetAttribute(k_eval_mixed_f32<VERTS, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
   const int64_t full = (int64_t)sms * 8;
   const int64_t g = VERTS ? full : std::min(full, (npts + 31) / 32);
