@@ -67,7 +67,8 @@ def eval_f32_term_ops(d):
 # DRAM bytes per traced edge of the root phase's kernels from an ncu capture
 # (dram__bytes_read.sum + dram__bytes_write.sum over the phase's launches,
 # divided by the traced edges); None once a kernel has changed since the
-# capture, as here: the one under profiles/ shows the per-edge kernels
+# capture, as here: the one under profiles/ shows k_rg_solve and k_roots_terms,
+# not the whole phase
 ROOTS_DRAM_BYTES_PER_EDGE = None
 
 

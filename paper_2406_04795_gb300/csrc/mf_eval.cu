@@ -22,9 +22,10 @@
 // support vectors within the root screen's reach (the per-vertex lists the
 // root solve screens instead of all vectors).
 //
-// Mixed FP32 SIMT path: one thread per two points, support vectors broadcast
-// from shared memory, FP32 differences and ex2, and a per-point rigorous bound
-// B on |f~ - f|; points with |f~| <= max(B, band) are re-evaluated in FP64.
+// Mixed FP32 SIMT path: a block per 32 points, lane per point, its warps over
+// tiles of 256 support vectors in shared memory, FP32 differences and ex2, and a
+// per-point rigorous bound B on |f~ - f|; points with |f~| <= max(B, band) are
+// re-evaluated in FP64.
 #include <cmath>
 #include <algorithm>
 #include <cstdio>

@@ -14,7 +14,7 @@
 // over it with most lanes idle after the screen.)  The chunk's edges are first
 // bucketed by base vertex.  This stage and the redo on the d = 5 FP64 proof at
 // lambda = 0.15 (1.32M edges, 0.24M vertices): 5.2 -> 3.2 ms; at lambda = 0.08
-// (7.2M edges, 1.2M vertices): 28.1 -> 13.4 ms; d = 6 BF16: 2.9 -> 1.7 ms.
+// (7.2M edges, 1.2M vertices): 28.1 -> 11.7 ms; d = 6 BF16: 2.9 -> 1.7 ms.
 //
 // What it hands over is one RootRec per edge: the converged FP32 t, g' and g''
 // there, the FP32 sum of the terms below ROOT_TAU at t (checked against its
