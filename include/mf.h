@@ -273,8 +273,9 @@ int mf_subdiv_next(mf_ctx *ctx, mf_trace_out *out, int64_t *cells_left, void *st
  * planner-side loop is out of scope, this is the serving runtime around the
  * traced path).  The server holds up to max_slots concurrent traces in an HBM
  * arena of hbm_bytes (one server per context), beside which its creation takes
- * about 4 % more for the root solve where the context's budget has room for it
- * (serving allocates nothing).  Requests queue FIFO; each
+ * about 4 % more for the root solve where the context's budget has room for it.
+ * Serving allocates nothing, unless another call on the context has taken that
+ * room meanwhile.  Requests queue FIFO; each
  * mf_server_step admits queued requests while a slot is free and the
  * request's buffers (sized from its opts capacities, defaults 2^20 edges) fit
  * the arena, runs up to MF_SERVER_STEPS breadth-first steps of every running

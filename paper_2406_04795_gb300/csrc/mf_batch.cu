@@ -240,7 +240,8 @@ int mf_finish_trace(mf_ctx *ctx, const mf_rbf *rbf, const mf_trace_opts *o, cons
 // d_only: device words for the mask, n of them; the mask is kept in `mask`
 // until the stream has been waited for.
 // fixed: pools of that size whatever the slots (a slot with more vertices takes
-// the batched kernel), else as the largest slot needs them.
+// the batched kernel; all of them do when it is zero), else as the largest slot
+// needs them.
 #define ROOTS_ALONE 8192
 struct RootPools {
   uint64_t chunk, verts;
@@ -657,7 +658,8 @@ extern "C" int mf_server_create(mf_ctx *ctx, int32_t max_slots, size_t hbm_bytes
   s->roots.verts = std::max<uint64_t>(4 * s->roots.chunk, 1ull << 22);
   {
     MfTraceBufs pools;
-    mf_setup_root_pools(ctx, MF_SLOT_BATCHROOTS, MF_MAXD, s->roots.chunk, s->roots.verts, &pools);
+    if (!mf_setup_root_pools(ctx, MF_SLOT_BATCHROOTS, MF_MAXD, s->roots.chunk, s->roots.verts, &pools))
+      s->roots = {0, 0};  // not asked for again while serving
   }
   s->slots.assign(max_slots, MfSlot());
   memset(s->slots.data(), 0, sizeof(MfSlot) * max_slots);
